@@ -588,6 +588,139 @@ __global__ void __launch_bounds__(GW_T) k_gains_warp(GainArgs G, const int32_t *
     }
 }
 
+// ---------------------------------------------------------------- gains from part bits
+// Levels whose cut hyperedges span many parts (random nets: lambda(e) near
+// |e|).  k_part_bits writes, for every cut hyperedge, one row of 4 * WQ words
+// with bit p set when e touches part p; k_gains_bits then reads a node's rows
+// instead of its pins lists.  A lane owns the parts p = 32 k + lane: the row's
+// words arrive by a warp-uniform 16-byte load and every lane adds w(e) to the
+// counters of its set bits, so a row costs two instructions per 32 parts and
+// neither a hash probe nor an atomic.  The list form needs a match, a warp
+// reduction and a shared-memory update per list entry.  Bound by the L1 return
+// of the uniform loads (a row's bytes to 32 lanes).  Measured per repetition,
+// summed over the node lists: 16,384-node random net, 413 parts, lambda about
+// 100: 7.4 ms of list kernels, 0.33 ms of bit kernels, 30 us for the rows;
+// 20,011-node irregular net, 206 parts, lambda about 26: 1.93 and 0.13 ms.
+constexpr int PB_T = 256, PB_MAXQ = 8;
+constexpr int32_t PB_PARTS = PB_MAXQ * 128;   // largest number of parts with a row
+constexpr int64_t PB_BYTES = int64_t(1) << 30;
+__global__ void __launch_bounds__(PB_T) k_part_bits(const int32_t *off, Plist PL, int32_t e, int wq, uint4 *bits) {
+    HP_KERNEL_ENTER();
+    __shared__ __align__(16) uint32_t s_row[PB_T / 32][PB_MAXQ * 4];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    uint32_t *row = s_row[wid];
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = w0; i < e; i += nw) {
+        const int32_t a = off[i];
+        if (off[i + 1] - a < 2) continue;   // single-pin hyperedges have no pins list
+        const int32_t lam = PL.lam[i];
+        if (lam < 2) continue;              // not cut: no node lists it
+        if (lane < 4 * wq) row[lane] = 0;
+        __syncwarp();
+        for (int32_t k = lane; k < lam; k += 32) {
+            const int32_t p = PL.p[a + k];
+            atomicOr(&row[p >> 5], 1u << (p & 31));
+        }
+        __syncwarp();
+        if (lane < wq) bits[i * wq + lane] = reinterpret_cast<const uint4 *>(row)[lane];
+        __syncwarp();
+    }
+}
+
+// One node per CTA of NW warps, the warps taking its cut hyperedges in chunks
+// of 32.  The counters are 32 bits wide: the host takes this path only when
+// the sum of all weights is below 2^32.
+template <int WQ, int NW>
+__global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 *bits, int32_t nparts,
+                                                        const int32_t *list, const int32_t *count_p) {
+    HP_KERNEL_ENTER();
+    __shared__ uint32_t s_conn[WQ * 128];
+    __shared__ long long s_rg[NW];
+    __shared__ int32_t s_rp[NW];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t my = 1u << lane;
+    const int32_t count = *count_p;
+    for (int i = threadIdx.x; i < WQ * 128; i += NW * 32) s_conn[i] = 0;
+    __syncthreads();
+    for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
+        const int32_t v = list[k], s = G.rho[v];
+        const int32_t c0 = G.ioff[v], c1 = G.ioff[v + 1];
+        uint32_t acc[WQ * 4];
+#pragma unroll
+        for (int q = 0; q < WQ * 4; q++) acc[q] = 0;
+        for (int32_t base = c0 + wid * 32; base < c1; base += NW * 32) {
+            const int32_t t = base + lane;
+            int32_t e = 0;
+            uint32_t we = 0;
+            if (t < c1) {
+                e = G.inc[t];
+                we = (uint32_t)G.w[e];
+            }
+            const int cnt = min(32, c1 - base);
+#pragma unroll 4
+            for (int u = 0; u < cnt; u++) {
+                const uint4 *r = bits + (int64_t)__shfl_sync(FULL, e, u) * WQ;
+                const uint32_t wu = __shfl_sync(FULL, we, u);
+#pragma unroll
+                for (int q = 0; q < WQ; q++) {
+                    const uint4 x = __ldg(r + q);
+                    if (x.x & my) acc[4 * q] += wu;
+                    if (x.y & my) acc[4 * q + 1] += wu;
+                    if (x.z & my) acc[4 * q + 2] += wu;
+                    if (x.w & my) acc[4 * q + 3] += wu;
+                }
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < WQ * 4; q++)
+            if (acc[q]) atomicAdd(&s_conn[32 * q + lane], acc[q]);
+        __syncthreads();
+        // the best part (gain, then the larger id) of the ones v touches
+        long long bg = 0;
+        int32_t bp = -1;
+        const long long basev = G.saving[v] - G.wns[v];
+        const long long room = (long long)G.omega - G.size[v];
+        for (int32_t p = threadIdx.x; p < nparts; p += NW * 32) {
+            const uint32_t c = s_conn[p];
+            s_conn[p] = 0;
+            if (c == 0 || p == s || (G.second_half && G.psize[p] > room)) continue;
+            const long long g = basev + (long long)c;
+            if (bp < 0 || g >= bg) {   // p ascends
+                bg = g;
+                bp = p;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long og = __shfl_down_sync(FULL, bg, o);
+            const int32_t op = __shfl_down_sync(FULL, bp, o);
+            if (op >= 0 && (bp < 0 || og > bg || (og == bg && op > bp))) {
+                bg = og;
+                bp = op;
+            }
+        }
+        if (lane == 0) {
+            s_rg[wid] = bg;
+            s_rp[wid] = bp;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int x = 1; x < NW; x++)
+                if (s_rp[x] >= 0 && (bp < 0 || s_rg[x] > bg || (s_rg[x] == bg && s_rp[x] > bp))) {
+                    bg = s_rg[x];
+                    bp = s_rp[x];
+                }
+            if (bp >= 0 && bg > 0) {
+                const int32_t i = atomicAdd(G.M.count, 1);
+                G.M.node[i] = v;
+                G.M.src[i] = s;
+                G.M.dst[i] = bp;
+                G.M.gain[i] = bg;
+            }
+        }
+    }
+}
+
 // ---------------------------------------------------------------- per level constants
 // Per node: Wns(v) = sum of w(e) over incident hyperedges with |e| >= 2, and
 // the number of singleton hyperedges {v} that hold v as a destination.
@@ -2051,6 +2184,9 @@ struct LevelWs {
     // algorithmic bytes of the repetitions (host): running total, and the cut
     // entries and their list entries of the last rebuilt repetition
     int64_t alg_bytes = 0, cuts = 0, cut_lam = 0;
+    bool bits_valid = false;
+    uint4 *bits = nullptr;   // [ce][wq] parts of every cut hyperedge (k_part_bits), or none
+    int wq = 0;
     int32_t *touched, *ttouched;             // hyperedges with a moved pin (more than / at most 8 pins)
     Moves M, S;
     uint64_t *keys;
@@ -2190,6 +2326,13 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->gc = A.get<long long>((int64_t)W->gnb * W->gcap);
     fill_i32(W->gk, (int64_t)W->gnb * 2 * W->gcap, -1, s);
     HPC(cudaMemsetAsync(W->gc, 0, sizeof(long long) * W->gnb * W->gcap, s));
+    // rows of part bits (16 * wq bytes per hyperedge) where every sum of
+    // weights fits their 32-bit counters and they take at most PB_BYTES
+    W->wq = (int)cdiv(nparts, 128);
+    if (nparts <= PB_PARTS && P.wsum < (1ll << 32) && P.o.debug_table_cap == 0) {
+        W->wq = (int)pow2_at_least(std::max(W->wq, 1));
+        if ((int64_t)e * W->wq * 16 <= PB_BYTES) W->bits = A.get<uint4>((int64_t)e * W->wq);
+    }
     // hyperedges above 512 pins: tables and buffers in global memory
     W->ptab = W->ibuf = nullptr;
     W->pnb = 0;
@@ -2218,7 +2361,7 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
              W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cflag, W->cpos, W->cut, W->cut_off, W->tiny, W->mid, W->touched, W->ttouched, W->M.node, W->M.src, W->M.dst, W->M.gain,
              W->S.node, W->S.src, W->S.dst, W->S.gain, W->keys, W->idx, W->msz, W->mni, W->first, W->choice, W->accnode, W->pen,
              W->minpen, W->acc1, W->acc2, W->pos, W->clen, W->lens, W->starts, W->cstart, W->seqmove, W->heads, W->hkeys,
-             W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->ovf, W->gk, W->gc, W->ptab, W->ibuf})
+             W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
         A.release(p);
     delete W;
 }
@@ -2289,6 +2432,39 @@ static void level_prepare(const Level &L, const int32_t *w, const int32_t *rho, 
     if (W.n_big > 0 && !W.ptab) throw Error(HP_ERR_INTERNAL, "large hyperedge buffers missing");
 }
 
+// Whether the gains of the next repetition are computed from part bits: the
+// average number of list entries behind a cut incidence entry, as counted by
+// the last repetition that rebuilt the lists (of this level, or of the coarser
+// one, whose lambda(e) the projection keeps), against the row's words.  At
+// one entry per word the bits win (262k-node Gaussian net with the learned
+// first level, lambda about 3 and 8 to 16 words: 462.8 ms by this rule, 483.1
+// with bits from a quarter of an entry per word on; 4,096-node random net,
+// 25 entries to 4 words: 27.0 ms against 46.1 without bits).
+static bool bits_pay(const Level &L, const LevelWs &W) {
+    if (!W.bits) return false;
+    if (W.cuts == 0) return L.np >= 16 * (int64_t)L.e;
+    return W.cut_lam >= W.cuts * 4 * W.wq;
+}
+
+template <int WQ>
+static void gains_bits(const GainArgs &G, const LevelWs &W, const int32_t *cnt, int32_t n, cudaStream_t s) {
+    // hub nodes on the side stream, beside the two lists of smaller ones
+    HPC(cudaEventRecord(W.ev[0], s));
+    HPC(cudaStreamWaitEvent(W.side, W.ev[0], 0));
+    const int occ_h = prepare_kernel((const void *)k_gains_bits<WQ, 16>, 512, 0);
+    launch_k(k_gains_bits<WQ, 16>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 512, 0, W.side, G, W.bits, W.nparts,
+             W.hubs, cnt + C_HUB);
+    HP_LAUNCH_CHECK();
+    HPC(cudaEventRecord(W.ev[1], W.side));
+    const int occ = prepare_kernel((const void *)k_gains_bits<WQ, 4>, 128, 0);
+    const int grid = std::max(1, std::min<int>(n, num_sms() * occ));
+    launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cw, cnt + C_CW);
+    HP_LAUNCH_CHECK();
+    launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cl, cnt + C_CAND);
+    HP_LAUNCH_CHECK();
+    HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
+}
+
 // One repetition; returns the number of moves applied.
 // reuse: rho is unchanged since the previous repetition of this level (which
 // applied nothing), so its pins lists, D(p), |p|, saving(v) and cut lists,
@@ -2304,6 +2480,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
     launch_k(k_rep_zero, grid_of(zspan, 256), 256, 0, s, R, reuse ? 1 : 0);
     HP_LAUNCH_CHECK();
     if (!reuse) {
+        W.bits_valid = false;
         launch_k(k_rep_nodes, grid_of(n, 256), 256, 0, s, rho, L.size, W.singin, n, R.psize, R.D0);
         HP_LAUNCH_CHECK();
         // pins(p,e), pins_in(p,e), D(p), saving(v)
@@ -2351,36 +2528,48 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
              W.cw, cnt + C_CW);
     HP_LAUNCH_CHECK();
     GainArgs G{L.off, W.cut_off, W.cut, w, rho, L.size, R.psize, R.saving, W.wns, W.PL, P.omega, second_half, W.M};
-    uint32_t gcap_smem = 2048;
-    if (P.o.debug_table_cap > 0) gcap_smem = (uint32_t)P.o.debug_table_cap;
-    const size_t gsm = (size_t)gcap_smem * 12 + (size_t)(gcap_smem * 3 / 4) * 4;
-    {
-        // hub nodes on the side stream, beside the warp and CTA tiers (disjoint
-        // node lists; all append to the same move and overflow lists by atomics)
-        HPC(cudaEventRecord(W.ev[0], s));
-        HPC(cudaStreamWaitEvent(W.side, W.ev[0], 0));
-        const int occ_h = prepare_kernel((const void *)k_gains_smem<1024>, 1024, gsm);
-        launch_k(k_gains_smem<1024>, num_sms() * std::max(occ_h, 1), 1024, gsm, W.side, G, W.hubs, cnt + C_HUB, gcap_smem,
-                 W.ovf, cnt + C_OVF);
-        HP_LAUNCH_CHECK();
-        HPC(cudaEventRecord(W.ev[1], W.side));
-    }
-    {
-        const uint32_t wlimit = P.o.debug_table_cap > 0 ? std::min<uint32_t>(GW_SLOTS * 3 / 4, P.o.debug_table_cap / 2)
-                                                        : GW_SLOTS * 3 / 4;
-        int occ = prepare_kernel((const void *)k_gains_warp, GW_T, 0);
-        int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(n, GW_T / 32), (int64_t)num_sms() * occ));
-        launch_k(k_gains_warp, grid, GW_T, 0, s, G, W.cw, cnt + C_CW, wlimit, W.cl, cnt + C_CAND);
-        HP_LAUNCH_CHECK();
-    }
-    {
-        int occ = prepare_kernel((const void *)k_gains_smem<GN_T>, GN_T, gsm);
-        int grid = std::max(1, std::min<int>(n, num_sms() * occ));
-        launch_k(k_gains_smem<GN_T>, grid, GN_T, gsm, s, G, W.cl, cnt + C_CAND, gcap_smem, W.ovf, cnt + C_OVF);
-        HP_LAUNCH_CHECK();
-        HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
-        launch_k(k_gains_global, W.gnb, GN_T, 0, s, G, W.ovf, cnt + C_OVF, W.gcap, W.gk, W.gc, W.cl, cnt + C_BAD);
-        HP_LAUNCH_CHECK();
+    if (bits_pay(L, W)) {
+        if (!reuse || !W.bits_valid) {
+            launch_k(k_part_bits, grid_of((int64_t)L.e * 32, PB_T), PB_T, 0, s, L.off, W.PL, L.e, W.wq, W.bits);
+            HP_LAUNCH_CHECK();
+            W.bits_valid = true;
+        }
+        if (W.wq == 1) gains_bits<1>(G, W, cnt, n, s);
+        else if (W.wq == 2) gains_bits<2>(G, W, cnt, n, s);
+        else if (W.wq == 4) gains_bits<4>(G, W, cnt, n, s);
+        else gains_bits<8>(G, W, cnt, n, s);
+    } else {
+        uint32_t gcap_smem = 2048;
+        if (P.o.debug_table_cap > 0) gcap_smem = (uint32_t)P.o.debug_table_cap;
+        const size_t gsm = (size_t)gcap_smem * 12 + (size_t)(gcap_smem * 3 / 4) * 4;
+        {
+            // hub nodes on the side stream, beside the warp and CTA tiers (disjoint
+            // node lists; all append to the same move and overflow lists by atomics)
+            HPC(cudaEventRecord(W.ev[0], s));
+            HPC(cudaStreamWaitEvent(W.side, W.ev[0], 0));
+            const int occ_h = prepare_kernel((const void *)k_gains_smem<1024>, 1024, gsm);
+            launch_k(k_gains_smem<1024>, num_sms() * std::max(occ_h, 1), 1024, gsm, W.side, G, W.hubs, cnt + C_HUB, gcap_smem,
+                     W.ovf, cnt + C_OVF);
+            HP_LAUNCH_CHECK();
+            HPC(cudaEventRecord(W.ev[1], W.side));
+        }
+        {
+            const uint32_t wlimit = P.o.debug_table_cap > 0 ? std::min<uint32_t>(GW_SLOTS * 3 / 4, P.o.debug_table_cap / 2)
+                                                            : GW_SLOTS * 3 / 4;
+            int occ = prepare_kernel((const void *)k_gains_warp, GW_T, 0);
+            int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(n, GW_T / 32), (int64_t)num_sms() * occ));
+            launch_k(k_gains_warp, grid, GW_T, 0, s, G, W.cw, cnt + C_CW, wlimit, W.cl, cnt + C_CAND);
+            HP_LAUNCH_CHECK();
+        }
+        {
+            int occ = prepare_kernel((const void *)k_gains_smem<GN_T>, GN_T, gsm);
+            int grid = std::max(1, std::min<int>(n, num_sms() * occ));
+            launch_k(k_gains_smem<GN_T>, grid, GN_T, gsm, s, G, W.cl, cnt + C_CAND, gcap_smem, W.ovf, cnt + C_OVF);
+            HP_LAUNCH_CHECK();
+            HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
+            launch_k(k_gains_global, W.gnb, GN_T, 0, s, G, W.ovf, cnt + C_OVF, W.gcap, W.gk, W.gc, W.cl, cnt + C_BAD);
+            HP_LAUNCH_CHECK();
+        }
     }
     // The rest of the repetition; `end` reads its counters back (the one
     // host read of a repetition on a small level) and returns the moves applied.
