@@ -1045,26 +1045,77 @@ struct ChainCtx {
     int32_t *linked;                      // linked[r]: round r linked something
 };
 
+// The pick of one free chain end i by its warp (packed acceptance, 64-bit
+// grades: |G| < 2^62 when the weights sum to at most 2^38): among the first
+// `window` moves of [j0, jend) not taken and not i, the one of maximum grade
+// G = gain * 10^7 - penalty, earliest on ties; lanes over moves.  The moves
+// leaving a part are sorted by gain, and no penalty is negative, so the scan
+// ends at the first move whose gain * 10^7 does not exceed the best grade
+// found: usually after the moves that tie with the best gain.  Bound by the
+// latency of the scan's steps.  A thread per free end, four moves at a time
+// from L2 and to the window's end, took 372 us a call of k_seq_cluster on the
+// 262k layered net (1,831 moves, 13 rounds on average), 556 us on the 20k
+// irregular net (1,543 moves, 6.5 rounds) and 45 us a round of the device-wide
+// form on the 1M Gaussian net; a warp per free end, from shared memory in the
+// cluster kernel: 116, 119 and 12.6 us.
+template <class Taken, class Gain, class Sn>
+__device__ __forceinline__ int32_t warp_pick(int32_t i, int32_t jbeg, int32_t jend, int32_t window, int32_t szi,
+                                             int32_t nii, Taken taken, Gain gain, Sn sn, uint32_t &pen_out) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    long long bG = LLONG_MIN;
+    int32_t best = -1, seen = 0;
+    uint32_t bpen = 0;
+    for (int32_t j0 = jbeg; j0 < jend && seen < window; j0 += 32) {
+        const int32_t j = j0 + lane;
+        const bool in = j < jend;
+        const long long top = in ? gain(j) * 10000000ll : 0;
+        if (__any_sync(FULL, bG >= __shfl_sync(FULL, top, 0))) break;
+        bool ok = in && j != i && !taken(j);
+        const unsigned bal = __ballot_sync(FULL, ok);
+        ok = ok && seen + __popc(bal & lt) < window;
+        if (ok) {
+            const int2 x = sn(j);
+            const long long ds = (long long)szi - x.x, di = (long long)nii - x.y;
+            const long long pen = 10 * (ds < 0 ? -ds : ds) + (di < 0 ? -di : di);
+            if (top - pen > bG) {
+                bG = top - pen;
+                best = j;
+                bpen = (uint32_t)pen;
+            }
+        }
+        seen += __popc(bal);
+    }
+    // maximum grade over the lanes (high word, then low word), then the earliest move
+    const int32_t hi = (int32_t)(bG >> 32);
+    const int32_t mhi = __reduce_max_sync(FULL, hi);
+    const uint32_t mlo = __reduce_max_sync(FULL, hi == mhi ? (uint32_t)bG : 0u);
+    const bool top_lane = best >= 0 && hi == mhi && (uint32_t)bG == mlo;
+    const uint32_t bj = __reduce_min_sync(FULL, top_lane ? (uint32_t)best : 0xffffffffu);
+    if (bj == 0xffffffffu) return -1;
+    pen_out = __shfl_sync(FULL, bpen, (int)(bj - (uint32_t)jbeg) & 31);
+    return (int32_t)bj;
+}
+
 // Sec. VI-C: every free chain end picks, among the first `window` moves
 // leaving its destination that have no predecessor, the one of maximum
 // grade G = gain(m)*10^7 - 10|size(n)-size(m)| - |nin(n)-nin(m)|, earliest on
 // ties.  For a chosen move all choosers share gain(m), so the acceptor of
 // maximum (G, node id) is the chooser of minimum penalty, then maximum id.
-__device__ void ph_choose(const ChainCtx &C, int r, int packed, int32_t m, int64_t t0, int64_t nt) {
+__device__ void ph_choose(const ChainCtx &C, int32_t m, int64_t t0, int64_t nt) {
     constexpr int B = 4;   // candidates loaded together, ahead of their evaluation
     STRIDE(i0, m, t0, nt) {
         int32_t i = (int32_t)i0;
         C.choice[i] = -1;
-        if (!packed) {
-            C.minpen[i] = ~0ull;
-            C.accnode[i] = -1;
-        }
+        C.minpen[i] = ~0ull;
+        C.accnode[i] = -1;
         if (C.succ[i] >= 0) continue;
         const int32_t d = C.dst[i];
         int32_t seen = 0, best = -1;
         __int128 bG = 0;
         unsigned long long bpen = 0;
-        const int32_t vi = C.node[i], szi = C.msz[i], nii = C.mni[i];
+        const int32_t szi = C.msz[i], nii = C.mni[i];
         const int32_t jend = C.first[d + 1];
         for (int32_t j0 = C.first[d]; j0 < jend && seen < C.window; j0 += B) {
             int32_t pr[B], sz[B], ni[B];
@@ -1082,6 +1133,10 @@ __device__ void ph_choose(const ChainCtx &C, int r, int packed, int32_t m, int64
             for (int u = 0; u < B; u++) {
                 const int32_t j = j0 + u;
                 if (j >= jend || seen >= C.window) break;
+                if (best >= 0 && (__int128)gn[u] * 10000000 <= bG) {   // none from here on has a higher grade
+                    seen = C.window;
+                    break;
+                }
                 if (pr[u] >= 0 || j == i) continue;
                 seen++;
                 const long long ds = (long long)szi - sz[u], di = (long long)nii - ni[u];
@@ -1097,9 +1152,6 @@ __device__ void ph_choose(const ChainCtx &C, int r, int packed, int32_t m, int64
         }
         C.choice[i] = best;
         C.pen[i] = bpen;
-        if (best >= 0 && packed)
-            atomicMax(&((r & 1) ? C.acc[1] : C.acc[0])[best],
-                      ((0xffffffffull - bpen) << 32) | (unsigned long long)(uint32_t)vi);
     }
 }
 __device__ void ph_accept_min(const ChainCtx &C, int32_t m, int64_t t0, int64_t nt) {
@@ -1147,64 +1199,59 @@ __device__ void ph_link(const ChainCtx &C, int r, int packed, int32_t m, int64_t
 __device__ __forceinline__ unsigned long long chain_key(unsigned long long pen, int32_t node) {
     return ((0xffffffffull - pen) << 32) | (unsigned long long)(uint32_t)node;
 }
-__device__ void ph_round(const ChainCtx &C, int r, int32_t m, int64_t t0, int64_t nt) {
-    constexpr int B = 4;
+// The free ends are dealt to the warps a lane at a time (a warp of few moves
+// otherwise scans for 32 of them one after another).
+template <class Taken, class Gain, class Sn>
+__device__ void ph_round(const ChainCtx &C, int r, int32_t m, int gw, int nw, Taken taken, Gain gain, Sn sn) {
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
     unsigned long long *accr = C.acc[r % 3], *accp = C.acc[(r + 2) % 3], *accn = C.acc[(r + 1) % 3];
-    STRIDE(i0, m, t0, nt) {
-        const int32_t i = (int32_t)i0;
-        bool taken_end = C.succ[i] >= 0;
-        if (r > 0) {
-            const int32_t j = C.choice[i];
-            if (j >= 0 && accp[j] == chain_key(C.pen[i], C.node[i])) {
-                C.pred[j] = i;
-                C.succ[i] = j;
-                taken_end = true;
-            }
-        }
-        accn[i] = 0;
-        C.choice[i] = -1;
-        if (taken_end) continue;
-        const int32_t d = C.dst[i];
-        int32_t seen = 0, best = -1;
-        __int128 bG = 0;
-        unsigned long long bpen = 0;
-        const int32_t szi = C.msz[i], nii = C.mni[i];
-        const int32_t jend = C.first[d + 1];
-        for (int32_t j0 = C.first[d]; j0 < jend && seen < C.window; j0 += B) {
-            bool tk[B];
-            int32_t sz[B], ni[B];
-            long long gn[B];
-#pragma unroll
-            for (int u = 0; u < B; u++) {
-                const int32_t j = j0 + u;
-                const bool ok = j < jend;
-                tk[u] = ok ? (C.pred[j] >= 0 || (r > 0 && accp[j] != 0ull)) : true;
-                sz[u] = ok ? C.msz[j] : 0;
-                ni[u] = ok ? C.mni[j] : 0;
-                gn[u] = ok ? C.gain[j] : 0;
-            }
-#pragma unroll
-            for (int u = 0; u < B; u++) {
-                const int32_t j = j0 + u;
-                if (j >= jend || seen >= C.window) break;
-                if (tk[u] || j == i) continue;
-                seen++;
-                const long long ds = (long long)szi - sz[u], di = (long long)nii - ni[u];
-                const unsigned long long pen =
-                    10ull * (unsigned long long)(ds < 0 ? -ds : ds) + (unsigned long long)(di < 0 ? -di : di);
-                const __int128 G = (__int128)gn[u] * 10000000 - (__int128)pen;
-                if (best < 0 || G > bG) {
-                    best = j;
-                    bG = G;
-                    bpen = pen;
+    for (int32_t base = 0; base < m; base += 32 * nw) {
+        const int32_t i = base + lane * nw + gw;
+        bool free_end = false;
+        int32_t j0 = 0, jend = 0, szi = 0, nii = 0, vi = 0;
+        if (i < m) {
+            free_end = C.succ[i] < 0;
+            vi = C.node[i];
+            if (r > 0) {
+                const int32_t j = C.choice[i];
+                if (j >= 0 && accp[j] == chain_key(C.pen[i], vi)) {
+                    C.pred[j] = i;
+                    C.succ[i] = j;
+                    free_end = false;
                 }
             }
+            accn[i] = 0;
+            if (free_end) {
+                const int32_t d = C.dst[i];
+                j0 = C.first[d];
+                jend = C.first[d + 1];
+                szi = C.msz[i];
+                nii = C.mni[i];
+            }
         }
-        C.choice[i] = best;
-        C.pen[i] = bpen;
-        if (best >= 0) {
-            atomicMax(&accr[best], chain_key(bpen, C.node[i]));
-            C.linked[r] = 1;
+        int32_t best = -1;
+        uint32_t pen = 0;
+        unsigned todo = __ballot_sync(FULL, free_end && j0 < jend);
+        while (todo) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1;
+            uint32_t p = 0;
+            const int32_t x = warp_pick(__shfl_sync(FULL, i, l), __shfl_sync(FULL, j0, l), __shfl_sync(FULL, jend, l),
+                                        C.window, __shfl_sync(FULL, szi, l), __shfl_sync(FULL, nii, l), taken, gain,
+                                        sn, p);
+            if (lane == l) {
+                best = x;
+                pen = p;
+            }
+        }
+        if (i < m) {
+            C.choice[i] = best;
+            C.pen[i] = pen;
+            if (best >= 0) {
+                atomicMax(&accr[best], chain_key(pen, vi));
+                C.linked[r] = 1;
+            }
         }
     }
 }
@@ -1506,10 +1553,34 @@ __global__ void k_gather_moves(const Moves M, const uint32_t *idx, const int32_t
     HP_KERNEL_ENTER();
     ph_gather(M, idx, *cntp, S, pc, size, nin, msz, mni, G_T0, G_NT);
 }
-__global__ void k_choose(ChainCtx C, const int32_t *mcount, int r, int packed) {
+__global__ void k_choose(ChainCtx C, const int32_t *mcount, int r) {
     HP_KERNEL_ENTER();
     if (r > 0 && !C.linked[r - 1]) return;
-    ph_choose(C, r, packed, *mcount, G_T0, G_NT);
+    ph_choose(C, *mcount, G_T0, G_NT);
+}
+// packed acceptance: a warp per free end
+__global__ void __launch_bounds__(128) k_choose_warp(ChainCtx C, const int32_t *mcount, int r) {
+    HP_KERNEL_ENTER();
+    if (r > 0 && !C.linked[r - 1]) return;
+    const int32_t m = *mcount;
+    const int lane = threadIdx.x & 31;
+    unsigned long long *acc = (r & 1) ? C.acc[1] : C.acc[0];
+    for (int64_t x = G_T0 >> 5; x < m; x += G_NT >> 5) {
+        const int32_t i = (int32_t)x;
+        int32_t best = -1;
+        uint32_t pen = 0;
+        if (C.succ[i] < 0) {
+            const int32_t d = C.dst[i];
+            best = warp_pick(i, C.first[d], C.first[d + 1], C.window, C.msz[i], C.mni[i],
+                             [&](int32_t j) { return C.pred[j] >= 0; }, [&](int32_t j) { return C.gain[j]; },
+                             [&](int32_t j) { return make_int2(C.msz[j], C.mni[j]); }, pen);
+        }
+        if (lane == 0) {
+            C.choice[i] = best;
+            C.pen[i] = pen;
+            if (best >= 0) atomicMax(&acc[best], chain_key(pen, C.node[i]));
+        }
+    }
 }
 __global__ void k_accept_min(ChainCtx C, const int32_t *mcount, int r) {
     HP_KERNEL_ENTER();
@@ -1588,6 +1659,9 @@ __global__ void k_apply(const int32_t *seqmove, const int32_t *node, const int32
 // each phase's global loads is spread over 8 SMs.
 static_assert(SQ_T == SEQ_T, "cluster CTA size");
 constexpr int32_t SEQ_CLUSTER_M = 4096;   // moves of a larger level sequenced by one cluster
+// moves whose gain, size and |in| (16 bytes each) fit the sort buffers of one CTA
+constexpr int32_t CHAIN_SMEM_M = (int32_t)(SQ_SMEM / 16);
+static_assert(CHAIN_SMEM_M / 32 <= 32 * 256, "their taken bits fit the digit counters");
 static_assert(SMALL_LEVEL <= sq_max<uint64_t>() && 2 * SMALL_LEVEL <= sq_max<uint32_t>(),
               "a small level's moves fit the cluster sorts");
 
@@ -1666,21 +1740,55 @@ __global__ void __cluster_dims__(SQ_CS, 1, 1) __launch_bounds__(SEQ_T) k_seq_clu
     cl.sync();
     ph_first_of(A.S.src, m, A.nparts, A.first, t0, nt);
     cl.sync();
-    // chaining rounds (Sec. VI-C)
+    // chaining rounds (Sec. VI-C).  Up to CHAIN_SMEM_M moves, every CTA keeps
+    // a copy of what the window scans read: gain, size and |in| of each move,
+    // and a bit per move with a predecessor, to which each round adds the
+    // moves chosen in the one before.
+    const bool in_smem = A.packed && m <= CHAIN_SMEM_M;
+    long long *c_gain = reinterpret_cast<long long *>(smem);
+    int2 *c_sn = reinterpret_cast<int2 *>(c_gain + CHAIN_SMEM_M);
+    uint32_t *c_taken = s_wc;
+    if (in_smem) {
+        for (int32_t j = threadIdx.x; j < m; j += blockDim.x) {
+            c_gain[j] = A.S.gain[j];
+            c_sn[j] = make_int2(A.C.msz[j], A.C.mni[j]);
+        }
+        for (int32_t x = threadIdx.x; x < (m + 31) / 32; x += blockDim.x) c_taken[x] = 0;
+        __syncthreads();
+    }
+    const int gw = (int)(t0 >> 5), nwarps = (int)(nt >> 5);
     for (int rr = 0; rr < A.rounds; rr++) {
         if (rr > 0 && !*(volatile int32_t *)&A.C.linked[rr - 1]) break;
         if (A.packed) {
-            ph_round(A.C, rr, m, t0, nt);
+            const unsigned long long *accp = A.C.acc[(rr + 2) % 3];
+            if (in_smem) {
+                if (rr > 0) {
+                    for (int32_t x = threadIdx.x >> 5; x < (m + 31) / 32; x += blockDim.x >> 5) {
+                        const int32_t j = 32 * x + (threadIdx.x & 31);
+                        const unsigned b = __ballot_sync(0xffffffffu, j < m && accp[j] != 0ull);
+                        if ((threadIdx.x & 31) == 0) c_taken[x] |= b;
+                    }
+                    __syncthreads();
+                }
+                ph_round(A.C, rr, m, gw, nwarps,
+                         [&](int32_t j) { return (c_taken[j >> 5] >> (j & 31)) & 1u; },
+                         [&](int32_t j) { return c_gain[j]; }, [&](int32_t j) { return c_sn[j]; });
+            } else {
+                ph_round(A.C, rr, m, gw, nwarps,
+                         [&](int32_t j) { return A.C.pred[j] >= 0 || (rr > 0 && accp[j] != 0ull); },
+                         [&](int32_t j) { return A.S.gain[j]; },
+                         [&](int32_t j) { return make_int2(A.C.msz[j], A.C.mni[j]); });
+            }
             cl.sync();
             continue;
         }
-        ph_choose(A.C, rr, A.packed, m, t0, nt);
+        ph_choose(A.C, m, t0, nt);
         cl.sync();
         ph_accept_min(A.C, m, t0, nt);
         cl.sync();
         ph_accept_id(A.C, m, t0, nt);
         cl.sync();
-        ph_link(A.C, rr, A.packed, m, t0, nt);
+        ph_link(A.C, rr, 0, m, t0, nt);
         cl.sync();
     }
     if (A.packed && A.rounds > 0 && *(volatile int32_t *)&A.C.linked[A.rounds - 1]) {
@@ -2612,7 +2720,8 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
               sb = bits_for((uint64_t)std::max(nparts - 1, 1));
     const long long cgbound = (long long)std::min<double>((double)gbound * (double)std::max(n, 1), 9.0e18);
     const int cgb = bits_for((uint64_t)cgbound);
-    const int packed = (10ll * P.omega + (long long)P.delta) < 0xffffffffll;
+    // packed acceptance and 64-bit grades: penalties below 2^32, gains of at most 2^38
+    const int packed = (10ll * P.omega + (long long)P.delta) < 0xffffffffll && P.wsum <= (1ll << 38);
     ChainCtx C;
     C.window = P.o.chain_window;
     C.node = W.S.node;
@@ -2678,9 +2787,12 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         // long, and the one-pass round's extra slot read per scanned move
         // costs more than the barrier it saves)
         for (int32_t r = 0; r < P.o.chain_rounds; r++) {
-            launch_k(k_choose, grid_of(m, 128), 128, 0, s, C, cnt + C_MOVES, r, packed);
-            HP_LAUNCH_CHECK();
-            if (!packed) {
+            if (packed) {
+                launch_k(k_choose_warp, grid_of((int64_t)m * 32, 128), 128, 0, s, C, cnt + C_MOVES, r);
+                HP_LAUNCH_CHECK();
+            } else {
+                launch_k(k_choose, grid_of(m, 128), 128, 0, s, C, cnt + C_MOVES, r);
+                HP_LAUNCH_CHECK();
                 launch_k(k_accept_min, grid_of(m, 256), 256, 0, s, C, cnt + C_MOVES, r);
                 HP_LAUNCH_CHECK();
                 launch_k(k_accept_id, grid_of(m, 256), 256, 0, s, C, cnt + C_MOVES, r);
