@@ -339,23 +339,26 @@ __device__ __forceinline__ void warp_chunk(const PropCtx &C, int32_t v, int32_t 
         if (m == v) m = -1;
         const unsigned g = __match_any_sync(FULL, m);
         const bool on = m >= 0;
-        const unsigned lo = __reduce_add_sync(g, on ? (unsigned)(qe & 0x1FFFFFull) : 0u);
-        const unsigned hi = __reduce_add_sync(g, on ? (unsigned)(qe >> 21) : 0u);
-        const unsigned ic = __reduce_add_sync(g, (on && vin && a + j >= dst0) ? 1u : 0u);
+        uint32_t x[3] = {(uint32_t)(qe & 0x1FFFFFull), (uint32_t)(qe >> 21), vin && a + j >= dst0 ? 1u : 0u};
+        group_sum(g, on, x);
         if (on && (g & lt) == 0u && size_ok(C, slack, m))
-            ins(m, (unsigned long long)lo + ((unsigned long long)hi << 21), ic);
+            ins(m, (unsigned long long)x[0] + ((unsigned long long)x[1] << 21), x[2]);
     }
     const unsigned bigm = __ballot_sync(FULL, large);
     if (!bigm) return;
     // groups of large hyperedges with equal destination lists
     const int32_t *canon = dst_groups_of(C);
-    const int32_t key = large ? (canon ? canon[e] : e) : -1 - lane;
-    const unsigned grp = __match_any_sync(FULL, key);
-    const unsigned qlo = __reduce_add_sync(grp, large ? (unsigned)(qe & 0x1FFFFFull) : 0u);
-    const unsigned qhi = __reduce_add_sync(grp, large ? (unsigned)(qe >> 21) : 0u);
-    const unsigned long long qsum = (unsigned long long)qlo + ((unsigned long long)qhi << 21);
-    const uint32_t icnt = vin ? (uint32_t)__popc(grp) : 0u;
-    const bool lead = large && (grp & lt) == 0u;
+    unsigned long long qsum = qe;
+    uint32_t icnt = vin ? 1u : 0u;
+    bool lead = large;
+    if (canon) {
+        const unsigned grp = __match_any_sync(FULL, large ? canon[e] : -1 - lane);
+        uint32_t x[2] = {(uint32_t)(qe & 0x1FFFFFull), (uint32_t)(qe >> 21)};
+        group_sum(grp, large, x);
+        qsum = (unsigned long long)x[0] + ((unsigned long long)x[1] << 21);
+        icnt = vin ? (uint32_t)__popc(grp) : 0u;
+        lead = large && (grp & lt) == 0u;
+    }
     if (large)
         for (int32_t j = a; j < dst0; j++) {
             const int32_t m = C.pin[j];

@@ -345,8 +345,9 @@ __device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, c
                 int32_t p = k < lam ? PL.p[a + k] : -1;
                 if (p == s) p = -1;
                 const unsigned m = __match_any_sync(0xffffffffu, p);
-                const unsigned sw = __reduce_add_sync(m, p >= 0 ? we : 0u);
-                if (p >= 0 && lane == __ffs(m) - 1) add(p, (long long)sw);
+                uint32_t sw[1] = {we};
+                group_sum(m, p >= 0, sw);
+                if (p >= 0 && lane == __ffs(m) - 1) add(p, (long long)sw[0]);
             }
         }
     }
@@ -523,7 +524,8 @@ __global__ void __launch_bounds__(GW_T) k_gains_warp(GainArgs G, const int32_t *
                 int32_t p = k2 < lam ? G.PL.p[a + k2] : -1;
                 if (p == s) p = -1;
                 const unsigned m = __match_any_sync(FULL, p);
-                const unsigned sw = __reduce_add_sync(m, p >= 0 ? we : 0u);
+                uint32_t sw[1] = {we};
+                group_sum(m, p >= 0, sw);
                 if (p >= 0 && lane == __ffs(m) - 1) {
                     uint32_t h = hslot(p, GW_SLOTS - 1);
                     for (int probe = 0; probe < GW_SLOTS; probe++) {
@@ -538,7 +540,7 @@ __global__ void __launch_bounds__(GW_T) k_gains_warp(GainArgs G, const int32_t *
                             }
                         }
                         if (kk == p) {
-                            atomicAdd((unsigned long long *)&conn[h], (unsigned long long)sw);
+                            atomicAdd((unsigned long long *)&conn[h], (unsigned long long)sw[0]);
                             break;
                         }
                         h = (h + 1) & (GW_SLOTS - 1);
@@ -861,9 +863,10 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
                     if (u < nu && up[u] == pp[j]) c = uc[u];
                 const int32_t key = (j < sz && c == 1) ? vv[j] : -1;
                 const unsigned m = __match_any_sync(FULL, key);
-                const unsigned sw = __reduce_add_sync(m, key >= 0 ? we : 0u);
+                uint32_t sw[1] = {we};
+                group_sum(m, key >= 0, sw);
                 if (key >= 0 && lane == __ffs(m) - 1)
-                    atomicAdd((unsigned long long *)&saving[key], (unsigned long long)sw);
+                    atomicAdd((unsigned long long *)&saving[key], (unsigned long long)sw[0]);
             }
         }
     }
@@ -2255,9 +2258,9 @@ __global__ void __launch_bounds__(IST_T) k_inseq_tiny(SeqSim Q, const int32_t *l
             }
             // |g| <= 65536 per lane, so the warp sums fit 32 bits
             const unsigned grp = __match_any_sync(FULL, k);
-            const int gs = (int)__reduce_add_sync(grp, (unsigned)g);
-            const int dss = (int)__reduce_add_sync(grp, (unsigned)ds);
-            const int dds = (int)__reduce_add_sync(grp, (unsigned)dd);
+            uint32_t sum[3] = {(uint32_t)g, (uint32_t)ds, (uint32_t)dd};
+            group_sum(grp, k >= 0, sum);
+            const int gs = (int)sum[0], dss = (int)sum[1], dds = (int)sum[2];
             if (k >= 0 && (grp & lt) == 0u) {
                 if (gs) atomicAdd(&Q.gseq[k], (unsigned long long)(long long)gs);
                 if (dss) atomicAdd(&Q.dDs[k], dss);
