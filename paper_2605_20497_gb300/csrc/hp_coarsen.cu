@@ -5,11 +5,17 @@
 //
 // The proposal fuses neighbour deduplication with the eta/inter histogram:
 // one CTA per node walks I(n) and the pins of every incident hyperedge and
-// accumulates into a shared-memory table (direct-indexed when the level has
-// at most 16384 nodes, open-addressing otherwise; nodes whose neighbourhood
-// outgrows the table are redone with a larger table and finally with a table
-// in global memory).  Sums and counts are integers, so the result does not
-// depend on the order of the atomic updates.
+// accumulates into a shared-memory table (direct-indexed on levels of at most
+// 4,096 nodes, and for large neighbourhoods up to 16,384; open-addressing
+// otherwise; nodes whose neighbourhood outgrows the table are redone with a
+// larger table and finally with a table in global memory).  Sums and counts
+// are integers, so the result does not depend on the order of the atomic
+// updates.  Bound by instruction issue and shared-memory updates per pin
+// visit.  Against one 16-byte entry a neighbour with a returning 64-bit add, a
+// 512-thread CTA a node and fixed shares of the hyperedges: level 0 of the 1M
+// Gaussian net 122 -> 69.6 ms, of the 16,384-node random net 9.1 -> 3.1 ms, of
+// the 262k layered net 15.7 -> 12.1 ms; whole calls 1.30 -> 1.12 s, 210 -> 159
+// ms and 249 -> 234 ms, 20k irregular net 96.8 -> 71.6 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,17 +46,23 @@ __device__ __forceinline__ uint64_t sm64_mix(uint64_t z) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
     return z ^ (z >> 31);
 }
-__device__ __forceinline__ uint64_t pair_noise(uint64_t level_key, int32_t a, int32_t b, uint64_t cap) {
+// The reduction is Barrett's, by inv = floor((2^64 - 1) / (cap + 1)): the
+// quotient estimate is low by at most two.
+__device__ __forceinline__ uint64_t pair_noise(uint64_t level_key, int32_t a, int32_t b, uint64_t cap, uint64_t inv) {
     uint32_t lo = (uint32_t)min(a, b), hi = (uint32_t)max(a, b);
     uint64_t h = sm64_mix(level_key ^ (((uint64_t)lo << 32) | (uint64_t)hi));
-    return h % (cap + 1);
+    uint64_t r = h - __umul64hi(h, inv) * (cap + 1);
+    if (r > cap) r -= cap + 1;
+    if (r > cap) r -= cap + 1;
+    return r;
 }
 
 struct PropCtx {
     int32_t n, pi;
     const int32_t *off, *pin, *nsrc, *size, *ioff, *inc, *nin;
     const uint64_t *q;
-    const uint64_t *cap;   // device scalar
+    const uint64_t *cap;   // device scalars: the noise cap and its reciprocal (pair_noise)
+    int32_t deg_narrow;    // nodes of at most this many hyperedges take two-word counters (see Tab)
     uint64_t level_key;
     int32_t omega, delta;
     int32_t *cand;         // [n*pi]
@@ -152,9 +164,11 @@ __global__ void k_node_bounds(const long long *nsum, int32_t n, int32_t *bound, 
                               int32_t permille) {
     HP_KERNEL_ENTER();
     // the noise cap of the level from the sum of q (complete: k_level_q ran before)
-    if (blockIdx.x == 0 && threadIdx.x == 0)
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
         box->cap = e > 0 ? (uint64_t)((box->qsum / (unsigned long long)e) * (unsigned long long)permille / 1000ull)
                          : 0ull;
+        box->cap_inv = ~0ull / (box->cap + 1);
+    }
     GRID_STRIDE(v, (int64_t)n) {
         long long b = bound[v];
         if (nsum[v] < b) b = nsum[v];
@@ -170,17 +184,6 @@ struct Cand {
 };
 __device__ __forceinline__ bool cand_gt(const Cand &a, const Cand &b) {
     return a.eta > b.eta || (a.eta == b.eta && a.id > b.id);
-}
-
-// x added to the 64-bit counter at p with two 32-bit atomics: the low word's
-// carry goes to the high word, so the counter ends equal to the exact sum
-// (all updates of p use this form).
-__device__ __forceinline__ void add_u64_split(unsigned long long *p, unsigned long long x) {
-    uint32_t *w = reinterpret_cast<uint32_t *>(p);
-    const uint32_t xl = (uint32_t)x, xh = (uint32_t)(x >> 32);
-    const uint32_t old = atomicAdd(&w[0], xl);
-    const uint32_t hi = xh + (uint32_t)((uint32_t)(old + xl) < old);
-    if (hi) atomicAdd(&w[1], hi);
 }
 
 template <int PIMAX> struct TopList {
@@ -211,18 +214,14 @@ template <int PIMAX> struct TopList {
 // then merges the warps' lists from s_top (32 * PIMAX entries).
 template <int PIMAX>
 __device__ __forceinline__ Cand warp_pop_best(TopList<PIMAX> &tl) {
-    Cand best = tl.c[0];
-    int owner = threadIdx.x & 31;
-    for (int o = 16; o > 0; o >>= 1) {
-        Cand ob{__shfl_xor_sync(0xffffffffu, best.eta, o), __shfl_xor_sync(0xffffffffu, best.id, o)};
-        const int oo = __shfl_xor_sync(0xffffffffu, owner, o);
-        if (cand_gt(ob, best) || (ob.id == best.id && oo < owner)) {
-            best = ob;
-            owner = oo;
-        }
-    }
-    if (best.id >= 0 && (int)(threadIdx.x & 31) == owner) tl.pop();
-    return best;
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t hi = (uint32_t)(tl.c[0].eta >> 32), lo = (uint32_t)tl.c[0].eta;
+    const uint32_t mhi = __reduce_max_sync(FULL, hi);
+    const uint32_t mlo = __reduce_max_sync(FULL, hi == mhi ? lo : 0u);
+    const bool top = hi == mhi && lo == mlo;
+    const int32_t id = __reduce_max_sync(FULL, top ? tl.c[0].id : -1);   // -1: every list is empty
+    if (id >= 0 && top && tl.c[0].id == id) tl.pop();
+    return Cand{((uint64_t)mhi << 32) | mlo, id};
 }
 template <int PIMAX>
 __device__ void block_emit_top(TopList<PIMAX> &tl, const PropCtx &C, int32_t v, Cand *s_top) {
@@ -280,9 +279,20 @@ __device__ Cand block_emit_range(TopList<EMIT_W> &tl, const PropCtx &C, int32_t 
     return *s_last;
 }
 
-__device__ __forceinline__ bool pair_valid(const PropCtx &C, int32_t v, int32_t m, int32_t inter) {
-    if ((int64_t)C.size[v] + C.size[m] > C.omega) return false;
-    return (int64_t)C.nin[v] + C.nin[m] - inter <= C.delta;
+// v's side of Eq. 5-6, read once per node
+struct Self {
+    int32_t v, size, nin;
+    uint64_t cap, inv;
+};
+__device__ __forceinline__ Self self_of(const PropCtx &C, int32_t v) {
+    return Self{v, C.size[v], C.nin[v], C.cap[0], C.cap[1]};
+}
+__device__ __forceinline__ bool pair_valid(const PropCtx &C, const Self &S, int32_t m, int32_t inter) {
+    if ((int64_t)S.size + C.size[m] > C.omega) return false;
+    return (int64_t)S.nin + C.nin[m] - inter <= C.delta;
+}
+__device__ __forceinline__ uint64_t noise_of(const PropCtx &C, const Self &S, int32_t m) {
+    return pair_noise(C.level_key, S.v, m, S.cap, S.inv);
 }
 
 __device__ __forceinline__ int32_t block_sum_i32(int32_t x, int32_t *s_tmp) {
@@ -296,166 +306,280 @@ __device__ __forceinline__ int32_t block_sum_i32(int32_t x, int32_t *s_tmp) {
     return t;
 }
 
-// One chunk of v's incidence for the calling warp: lane l takes the
-// hyperedge at incidence index t = base + l (none when t >= deg).
-// Hyperedges of 2..32 pins: the j-th pins of the warp's hyperedges are
-// combined by neighbour (match_any) and one table update per distinct
-// neighbour carries the warp's sums of q(e) and of the inbound-overlap
-// counts; q(e) <= 2^40 is summed as two 21-bit halves so that 32-bit warp
-// reductions cannot overflow.  Larger hyperedges: each lane inserts its own
-// source pins; the destination pins are walked once per group of the warp's
-// hyperedges with equal destination lists (C.canon; every hyperedge alone
-// when it is null), carrying the group's sum of q(e) and, when v is one of
-// those destinations, the group's size as the inbound overlap.  That walk is
-// handed to big(e, qsum, icnt) when it is given, else the warp takes the
-// groups one at a time, lanes over pins.
-template <class Ins, class Big>
-__device__ __forceinline__ void warp_chunk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, int32_t nin_v,
-                                           int32_t t, Ins &ins, Big *big) {
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const uint32_t lt = (1u << lane) - 1u;
-    int32_t e = -1, a = 0, sz = 0, dst0 = 0;
-    unsigned long long qe = 0;
-    bool vin = false;
-    if (t < deg) {
-        e = C.inc[i0 + t];
-        a = C.off[e];
-        sz = C.off[e + 1] - a;
-        if (sz < 2) {
-            sz = 0;
-        } else {
-            dst0 = a + C.nsrc[e];
-            qe = C.q[e];
-            vin = t < nin_v;
-        }
+// ---------------------------------------------------------------- neighbour counters
+// A neighbour's eta (a sum of q(e), below 2^60) and inbound overlap as 32-bit
+// words updated by shared-memory atomics that return nothing: a 64-bit sum
+// through a returning add and its carry costs more than the rest of an update.
+// Narrow form, for nodes of deg <= deg_narrow hyperedges: with B the bits of
+// deg and k = 32 - B, the low k bits of every q are summed in `lo` (fewer than
+// 2^B updates of less than 2^k), and `it` holds the overlap in its low B bits
+// (at most deg) and the sum of the q >> k above them.  That sum has at most
+// B + Q - k bits for q of at most Q bits, so both fit when 3 B + Q <= 64: up to
+// 8,191 hyperedges with unit weights (Q = 24), 255 with weights of 65,536.
+// Wide form, beyond that: eta in lo and hi with a carry, the overlap in `it`.
+struct Tab {
+    int32_t *keys;            // hashed tables: neighbour of every slot, -1 free
+    uint32_t *lo, *hi, *it;   // clean: 0
+};
+struct Fmt {
+    int B, k;
+};
+__device__ __forceinline__ Fmt fmt_of(int32_t deg) {
+    const int B = 32 - __clz(max(deg, 1));
+    return Fmt{B, 32 - B};
+}
+template <bool WIDE>
+__device__ __forceinline__ void tab_add(const Tab &T, Fmt f, uint32_t h, unsigned long long q, uint32_t ic) {
+    if constexpr (WIDE) {
+        const uint32_t ql = (uint32_t)q, old = atomicAdd(&T.lo[h], ql);
+        const uint32_t up = (uint32_t)(q >> 32) + (uint32_t)((uint32_t)(old + ql) < old);
+        if (up) atomicAdd(&T.hi[h], up);
+        if (ic) atomicAdd(&T.it[h], ic);
+    } else {
+        atomicAdd(&T.lo[h], (uint32_t)q & ((1u << f.k) - 1u));
+        const uint32_t up = ic + ((uint32_t)(q >> f.k) << f.B);
+        if (up) atomicAdd(&T.it[h], up);
     }
-    const bool large = sz > 32;
-    const int32_t len = large ? 0 : sz;
-    const int32_t slack = size_slack(C, v);
-    const int jmax = (int)__reduce_max_sync(FULL, (unsigned)len);
-    for (int j = 0; j < jmax; j++) {
-        int32_t m = j < len ? C.pin[a + j] : -1;
-        if (m == v) m = -1;
-        const unsigned g = __match_any_sync(FULL, m);
-        const bool on = m >= 0;
-        uint32_t x[3] = {(uint32_t)(qe & 0x1FFFFFull), (uint32_t)(qe >> 21), vin && a + j >= dst0 ? 1u : 0u};
-        group_sum(g, on, x);
-        if (on && (g & lt) == 0u && size_ok(C, slack, m))
-            ins(m, (unsigned long long)x[0] + ((unsigned long long)x[1] << 21), x[2]);
-    }
-    const unsigned bigm = __ballot_sync(FULL, large);
-    if (!bigm) return;
-    // groups of large hyperedges with equal destination lists
-    const int32_t *canon = dst_groups_of(C);
-    unsigned long long qsum = qe;
-    uint32_t icnt = vin ? 1u : 0u;
-    bool lead = large;
-    if (canon) {
-        const unsigned grp = __match_any_sync(FULL, large ? canon[e] : -1 - lane);
-        uint32_t x[2] = {(uint32_t)(qe & 0x1FFFFFull), (uint32_t)(qe >> 21)};
-        group_sum(grp, large, x);
-        qsum = (unsigned long long)x[0] + ((unsigned long long)x[1] << 21);
-        icnt = vin ? (uint32_t)__popc(grp) : 0u;
-        lead = large && (grp & lt) == 0u;
-    }
-    if (large)
-        for (int32_t j = a; j < dst0; j++) {
-            const int32_t m = C.pin[j];
-            if (m != v && size_ok(C, slack, m)) ins(m, qe, 0u);
-        }
-    if (big) {
-        if (lead) (*big)(e, qsum, icnt);
-        return;
-    }
-    unsigned lm = __ballot_sync(FULL, lead);
-    while (lm) {
-        const int l = __ffs(lm) - 1;
-        lm &= lm - 1;
-        const int32_t ld0 = __shfl_sync(FULL, dst0, l), lb = __shfl_sync(FULL, a, l) + __shfl_sync(FULL, sz, l);
-        const unsigned long long lq = __shfl_sync(FULL, qsum, l);
-        const uint32_t lc = __shfl_sync(FULL, icnt, l);
-        for (int32_t j = ld0 + lane; j < lb; j += 32) {
-            const int32_t m = C.pin[j];
-            if (m != v && size_ok(C, slack, m)) ins(m, lq, lc);
-        }
+}
+template <bool WIDE>
+__device__ __forceinline__ void tab_read(const Tab &T, Fmt f, uint32_t h, uint64_t &eta, int32_t &inter) {
+    const uint32_t lo = T.lo[h], it = T.it[h];
+    if constexpr (WIDE) {
+        eta = ((uint64_t)T.hi[h] << 32) | lo;
+        inter = (int32_t)it;
+    } else {
+        eta = ((uint64_t)(it >> f.B) << f.k) + lo;
+        inter = (int32_t)(it & ((1u << f.B) - 1u));
     }
 }
 
-struct NoBig {
-    __device__ void operator()(int32_t, unsigned long long, uint32_t) const {}
+// Updates of one warp: every lane calls, lanes with `on` add (q, ic) to
+// neighbour m.  Direct-indexed table:
+template <bool WIDE> struct DenseIns {
+    Tab T;
+    Fmt f;
+    __device__ __forceinline__ void operator()(bool on, int32_t m, unsigned long long q, uint32_t ic) const {
+        if (on) tab_add<WIDE>(T, f, (uint32_t)m, q, ic);
+    }
 };
+__device__ __forceinline__ uint32_t hslot(int32_t m, uint32_t mask) {
+    return mask ? ((uint32_t)m * 0x9E3779B1u) >> __clz(mask) : 0u;   // top bits (Fibonacci hashing)
+}
+// slot of key m, entered if absent (`fresh`); false when the table is full
+__device__ __forceinline__ bool tab_probe(int32_t *keys, uint32_t mask, int32_t m, uint32_t &h, bool &fresh) {
+    h = hslot(m, mask);
+    for (uint32_t probe = 0; probe <= mask; probe++) {
+        int32_t k = ((volatile int32_t *)keys)[h];
+        if (k == -1) {
+            k = atomicCAS(&keys[h], -1, m);
+            if (k == -1) {
+                fresh = true;
+                return true;
+            }
+        }
+        if (k == m) return true;
+        h = (h + 1) & mask;
+    }
+    return false;
+}
+// Hashed table of mask + 1 slots: all lanes find their slots first, then all
+// update; the slots entered are appended to a list, `flag` is set once the
+// list passes `limit`.
+template <bool WIDE, class Slot> struct HashIns {
+    Tab T;
+    Fmt f;
+    uint32_t mask, limit;
+    Slot *slots;
+    int32_t *n_slots;
+    int *flag;
+    __device__ __forceinline__ void operator()(bool on, int32_t m, unsigned long long q, uint32_t ic) const {
+        const unsigned FULL = 0xffffffffu;
+        uint32_t h = 0;
+        bool fresh = false;
+        if (on) on = tab_probe(T.keys, mask, m, h, fresh);
+        __syncwarp();
+        const unsigned nb = __ballot_sync(FULL, fresh);
+        if (nb) {
+            const int lane = threadIdx.x & 31, lead = __ffs(nb) - 1;
+            uint32_t at = 0;
+            if (lane == lead) at = (uint32_t)atomicAdd(n_slots, __popc(nb));
+            at = __shfl_sync(FULL, at, lead) + __popc(nb & ((1u << lane) - 1u));
+            if (fresh) {
+                if (at < limit) slots[at] = (Slot)h;
+                else *(volatile int *)flag = 1;
+            }
+        }
+        if (on) tab_add<WIDE>(T, f, h, q, ic);
+    }
+};
+// warp-private hashed table (large enough: no list, no overflow)
+struct WarpIns {
+    Tab T;
+    Fmt f;
+    uint32_t mask;
+    __device__ __forceinline__ void operator()(bool on, int32_t m, unsigned long long q, uint32_t ic) const {
+        uint32_t h = 0;
+        bool fresh = false;
+        if (on) on = tab_probe(T.keys, mask, m, h, fresh);
+        __syncwarp();
+        if (on) tab_add<false>(T, f, h, q, ic);
+    }
+};
+
+// ---------------------------------------------------------------- walk
+// one incident hyperedge as its thread reads it (sz = 0: none, or one pin)
+struct Hedge {
+    int32_t e, a, sz, d0;
+    unsigned long long q;
+    bool vin;
+};
+__device__ __forceinline__ Hedge hedge_of(const PropCtx &C, int32_t i0, int32_t t, int32_t deg, int32_t nin_v) {
+    Hedge x{-1, 0, 0, 0, 0ull, false};
+    if (t < deg) {
+        x.e = C.inc[i0 + t];
+        x.a = C.off[x.e];
+        x.sz = C.off[x.e + 1] - x.a;
+        x.d0 = x.a + C.nsrc[x.e];
+        x.q = C.q[x.e];
+        x.vin = t < nin_v;
+        if (x.sz < 2) x.sz = 0;
+    }
+    return x;
+}
+
+// Hyperedges of up to SMALL_E pins, one per lane: the j-th pins of the warp's
+// hyperedges are combined by neighbour (match_any) and one update per distinct
+// neighbour carries the warp's sums; q(e) <= 2^40 is summed as two 21-bit
+// halves so that 32-bit sums cannot overflow.  Larger ones are walked by a
+// warp each, lanes over pins, which are distinct: no combining.
+constexpr int32_t SMALL_E = 12;
+template <class Ins>
+__device__ __forceinline__ void walk_small(const PropCtx &C, int32_t v, int32_t slack, const Hedge &x, const Ins &ins) {
+    const unsigned FULL = 0xffffffffu;
+    const uint32_t lt = (1u << (threadIdx.x & 31)) - 1u;
+    const int32_t len = x.sz <= SMALL_E ? x.sz : 0;
+    const int jmax = (int)__reduce_max_sync(FULL, (unsigned)len);
+    int32_t mn = len > 0 ? C.pin[x.a] : -1;
+    for (int j = 0; j < jmax; j++) {
+        int32_t m = mn;
+        mn = j + 1 < len ? C.pin[x.a + j + 1] : -1;
+        if (m == v) m = -1;
+        const unsigned g = __match_any_sync(FULL, m);
+        const bool on = m >= 0;
+        uint32_t y[3] = {(uint32_t)(x.q & 0x1FFFFFull), (uint32_t)(x.q >> 21), x.vin && x.a + j >= x.d0 ? 1u : 0u};
+        group_sum(g, on, y);
+        const bool lead = on && (g & lt) == 0u && size_ok(C, slack, m);
+        ins(lead, m, (unsigned long long)y[0] + ((unsigned long long)y[1] << 21), y[2]);
+    }
+}
+// pins [beg, end) by one warp; the ones from d0 on carry the overlap ic
+template <class Ins>
+__device__ __forceinline__ void walk_list(const PropCtx &C, int32_t v, int32_t slack, int32_t beg, int32_t end,
+                                          int32_t d0, unsigned long long q, uint32_t ic, const Ins &ins) {
+    int32_t j = beg + (int32_t)(threadIdx.x & 31);
+    int32_t mn = j < end ? __ldg(&C.pin[j]) : -1;
+    for (int32_t j0 = beg; j0 < end; j0 += 32, j += 32) {
+        const int32_t m = mn;
+        mn = j + 32 < end ? __ldg(&C.pin[j + 32]) : -1;   // the next pin is loaded before this one is entered
+        ins(m >= 0 && m != v && size_ok(C, slack, m), m, q, j >= d0 ? ic : 0u);
+    }
+}
 
 // A warp's walk over all of v's hyperedges.
 template <class Ins>
 __device__ __forceinline__ void warp_walk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, int32_t nin_v,
-                                          Ins ins) {
-    for (int32_t base = 0; base < deg; base += 32)
-        warp_chunk(C, v, i0, deg, nin_v, base + (int32_t)(threadIdx.x & 31), ins, (NoBig *)nullptr);
+                                          const Ins &ins) {
+    const unsigned FULL = 0xffffffffu;
+    const int32_t slack = size_slack(C, v);
+    for (int32_t base = 0; base < deg; base += 32) {
+        const Hedge x = hedge_of(C, i0, base + (int32_t)(threadIdx.x & 31), deg, nin_v);
+        walk_small(C, v, slack, x, ins);
+        unsigned lm = __ballot_sync(FULL, x.sz > SMALL_E);
+        while (lm) {
+            const int l = __ffs(lm) - 1;
+            lm &= lm - 1;
+            const int32_t la = __shfl_sync(FULL, x.a, l);
+            walk_list(C, v, slack, la, la + __shfl_sync(FULL, x.sz, l), __shfl_sync(FULL, x.d0, l),
+                      __shfl_sync(FULL, x.q, l), __shfl_sync(FULL, (uint32_t)x.vin, l), ins);
+        }
+    }
 }
 
-// Shared-memory queue of destination walks of one CTA: blockDim.x entries.
-struct BigQueue {
-    int32_t *e;
-    unsigned long long *q;
-    uint32_t *c;
-    int32_t *n;   // == 0 on entry and on exit of cta_walk
+// Shared-memory queue of the lists one CTA walks: blockDim.x entries.  n and
+// next are two words each, zero on entry and on exit of cta_walk.
+template <int BT> struct ListQueue {
+    unsigned long long q[BT];
+    int32_t beg[BT], end[BT], d0[BT];
+    uint32_t ic[BT];
+    int32_t n[2], next[2];
 };
 
-// A CTA's walk over all of v's hyperedges in chunks of blockDim.x: small
-// ones and source pins as above, destination walks of large ones queued in
-// shared memory and then taken a warp each, lanes over pins, so that every
-// warp gets a share of them.  Stops early (for every thread) once *stop is
-// set.
-//
-// On levels without destination-list groups (small hyperedges, the coarse
-// levels, nets whose lists are all distinct) every warp walks its own
-// contiguous share of ceil(deg / warps) incidence entries, 32 at a time, with
-// no CTA barrier until the end, and walks its large hyperedges itself: even
-// a node of a few dozen hyperedges spreads them over all warps.
-template <class Ins>
+// A CTA's walk over all of v's hyperedges in chunks of BT: small ones as
+// above, larger ones queued and taken by the warps as they come free.  On
+// levels with destination-list groups the queue holds one entry per group of a
+// warp's hyperedges with equal lists, with the group's sum of q(e) and, when v
+// is one of those destinations, its size as the overlap; their source pins
+// are entered by the hyperedge's own lane.  The chunk after the current one
+// is loaded ahead.  Stops early (for every thread) once *stop is set.
+template <int BT, class Ins>
 __device__ void cta_walk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, int32_t nin_v, const int *stop,
-                         BigQueue Q, Ins ins) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (!dst_groups_of(C)) {
-        const int32_t share = (deg + nw - 1) / nw, lo = wid * share, hi = min(deg, lo + share);
-        for (int32_t base = lo; base < hi; base += 32) {
-            if (__any_sync(0xffffffffu, stop ? *(volatile const int *)stop : 0)) break;
-            warp_chunk(C, v, i0, deg, nin_v, base + lane < hi ? base + lane : deg, ins, (NoBig *)nullptr);
-        }
-        __syncthreads();
-        return;
-    }
+                         ListQueue<BT> &Q, const Ins &ins) {
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const uint32_t lt = (1u << lane) - 1u;
     const int32_t slack = size_slack(C, v);
-    auto push = [&](int32_t e, unsigned long long qsum, uint32_t icnt) {
-        const int32_t i = atomicAdd(Q.n, 1);
-        Q.e[i] = e;
-        Q.q[i] = qsum;
-        Q.c[i] = icnt;
-    };
-    for (int32_t base = 0; base < deg; base += blockDim.x) {
-        if (__syncthreads_or(stop ? *(volatile const int *)stop : 0)) break;
-        warp_chunk(C, v, i0, deg, nin_v, base + (int32_t)threadIdx.x, ins, &push);
-        __syncthreads();
-        const int32_t nb = *(volatile int32_t *)Q.n;
-        for (int32_t i = wid; i < nb; i += nw) {
-            const int32_t e = Q.e[i];
-            const unsigned long long qsum = Q.q[i];
-            const uint32_t icnt = Q.c[i];
-            const int32_t b = C.off[e + 1];
-            // the next pin is loaded before the current one is inserted
-            int32_t j = C.off[e] + C.nsrc[e] + lane;
-            int32_t mn = j < b ? __ldg(&C.pin[j]) : -1;
-            while (j < b) {
-                const int32_t m = mn, jn = j + 32;
-                mn = jn < b ? __ldg(&C.pin[jn]) : -1;
-                if (m != v && size_ok(C, slack, m)) ins(m, qsum, icnt);
-                j = jn;
+    const int32_t *canon = dst_groups_of(C);
+    int par = 0;
+    Hedge nx = hedge_of(C, i0, tid, deg, nin_v);
+    for (int32_t base = 0; base < deg; base += BT, par ^= 1) {
+        const Hedge x = nx;
+        if (base + BT < deg) nx = hedge_of(C, i0, base + BT + tid, deg, nin_v);
+        walk_small(C, v, slack, x, ins);
+        const bool large = x.sz > SMALL_E;
+        if (__any_sync(FULL, large)) {
+            unsigned long long q = x.q;
+            uint32_t ic = x.vin ? 1u : 0u;
+            int32_t beg = x.a;
+            bool lead = large;
+            if (canon) {
+                const unsigned grp = __match_any_sync(FULL, large ? canon[x.e] : -1 - lane);
+                uint32_t y[2] = {(uint32_t)(q & 0x1FFFFFull), (uint32_t)(q >> 21)};
+                group_sum(grp, large, y);
+                const int smax = (int)__reduce_max_sync(FULL, large ? (unsigned)(x.d0 - x.a) : 0u);
+                for (int j = 0; j < smax; j++) {
+                    const int32_t m = large && x.a + j < x.d0 ? C.pin[x.a + j] : -1;
+                    ins(m >= 0 && m != v && size_ok(C, slack, m), m, x.q, 0u);
+                }
+                q = (unsigned long long)y[0] + ((unsigned long long)y[1] << 21);
+                if (ic) ic = (uint32_t)__popc(grp);
+                lead = large && (grp & lt) == 0u;
+                beg = x.d0;
+            }
+            const unsigned bm = __ballot_sync(FULL, lead);
+            int32_t at = 0;
+            if (lane == 0) at = atomicAdd(&Q.n[par], __popc(bm));
+            at = __shfl_sync(FULL, at, 0) + __popc(bm & lt);
+            if (lead) {
+                Q.beg[at] = beg;
+                Q.end[at] = x.a + x.sz;
+                Q.d0[at] = x.d0;
+                Q.q[at] = q;
+                Q.ic[at] = ic;
             }
         }
         __syncthreads();
-        if (threadIdx.x == 0) *Q.n = 0;
+        const int32_t nb = *(volatile int32_t *)&Q.n[par];
+        if (tid == 0) Q.n[par ^ 1] = Q.next[par ^ 1] = 0;   // the next chunk's counters
+        while (nb > 0) {
+            int32_t i = 0;
+            if (lane == 0) i = atomicAdd(&Q.next[par], 1);
+            i = __shfl_sync(FULL, i, 0);
+            if (i >= nb || (stop && __any_sync(FULL, *(volatile const int *)stop))) break;
+            walk_list(C, v, slack, Q.beg[i], Q.end[i], Q.d0[i], Q.q[i], Q.ic[i], ins);
+        }
+        if (__syncthreads_or(stop ? *(volatile const int *)stop : 0)) break;
     }
+    if (tid == 0) Q.n[0] = Q.n[1] = Q.next[0] = Q.next[1] = 0;
     __syncthreads();
 }
 
@@ -517,272 +641,219 @@ __global__ void k_dst_canon(const uint32_t *val, const int32_t *newrun, const in
     GRID_STRIDE(i, (int64_t)e) canon[val[i]] = rep[runpos[i] + newrun[i] - 1];
 }
 
+// ---------------------------------------------------------------- candidate lists
+// C(v) from a table whose entries i = 0 .. n-1 (strided over `stride` threads
+// from `first`) give get(i, m, eta, inter) (false: empty), are rewritten by
+// put(i, w0, w1) / rescored by peek(i, m, w0, w1), and cleaned by clear(i).
+// Lists of up to four are kept per thread and merged; longer ones are emitted
+// in rounds of four, each below the last entry of the round before: the first
+// round stores every entry's noised score (below 2^63) and, in the top bit,
+// its validity, and the later rounds only compare.
+template <int PIMAX, class Tabl, class Emit>
+__device__ __forceinline__ int32_t list_best(const PropCtx &C, const Self &S, int32_t n, int first, int stride,
+                                             const Tabl &tab, Emit emit) {
+    int32_t cnt = 0;
+    if constexpr (PIMAX <= EMIT_W) {
+        TopList<PIMAX> tl;
+        tl.init();
+        for (int32_t i = first; i < n; i += stride) {
+            int32_t m, inter;
+            uint64_t eta;
+            if (!tab.get(i, m, eta, inter)) continue;
+            cnt++;
+            if (pair_valid(C, S, m, inter)) tl.push(Cand{eta + noise_of(C, S, m), m});
+            tab.clear(i);
+        }
+        emit(tl, 0, C.pi);
+    } else {
+        Cand thr{~0ull, INT32_MAX};
+        for (int r0 = 0; r0 < C.pi; r0 += EMIT_W) {
+            TopList<EMIT_W> tl;
+            tl.init();
+            for (int32_t i = first; i < n; i += stride) {
+                int32_t m;
+                uint64_t sc;
+                if (r0 == 0) {
+                    int32_t inter;
+                    if (!tab.get(i, m, sc, inter)) continue;
+                    cnt++;
+                    if (pair_valid(C, S, m, inter)) sc = (sc + noise_of(C, S, m)) | (1ull << 63);
+                    else sc = 1;   // neither empty nor valid
+                    tab.put(i, sc);
+                } else if (!tab.peek(i, m, sc)) {
+                    continue;
+                }
+                if (sc >> 63) {
+                    const Cand c{sc & ~(1ull << 63), m};
+                    if (cand_gt(thr, c)) tl.push(c);
+                }
+            }
+            thr = emit(tl, r0, min(EMIT_W, C.pi - r0));
+        }
+        for (int32_t i = first; i < n; i += stride) tab.clear(i);
+    }
+    return cnt;
+}
+
+// The tables as list_best reads them: slot h of entry i, its neighbour, and
+// whether it is in use.  Words lo and it carry the scores of the later rounds.
+template <bool WIDE> struct DenseTab {
+    Tab T;
+    Fmt f;
+    __device__ __forceinline__ bool get(int32_t i, int32_t &m, uint64_t &eta, int32_t &inter) const {
+        m = i;
+        tab_read<WIDE>(T, f, i, eta, inter);
+        return eta != 0;
+    }
+    __device__ __forceinline__ void put(int32_t i, uint64_t x) const {
+        T.lo[i] = (uint32_t)x;
+        T.it[i] = (uint32_t)(x >> 32);
+    }
+    __device__ __forceinline__ bool peek(int32_t i, int32_t &m, uint64_t &x) const {
+        m = i;
+        x = ((uint64_t)T.it[i] << 32) | T.lo[i];
+        return x != 0;
+    }
+    __device__ __forceinline__ void clear(int32_t i) const {
+        T.lo[i] = T.it[i] = 0;
+        if constexpr (WIDE) T.hi[i] = 0;
+    }
+};
+// slots: the list of used slots, or null: every slot of the table
+template <bool WIDE, class Slot> struct HashTab {
+    Tab T;
+    Fmt f;
+    const Slot *slots;
+    __device__ __forceinline__ uint32_t at(int32_t i) const { return slots ? (uint32_t)slots[i] : (uint32_t)i; }
+    __device__ __forceinline__ bool get(int32_t i, int32_t &m, uint64_t &eta, int32_t &inter) const {
+        const uint32_t h = at(i);
+        m = T.keys[h];
+        if (m < 0) return false;
+        tab_read<WIDE>(T, f, h, eta, inter);
+        return true;
+    }
+    __device__ __forceinline__ void put(int32_t i, uint64_t x) const {
+        const uint32_t h = at(i);
+        T.lo[h] = (uint32_t)x;
+        T.it[h] = (uint32_t)(x >> 32);
+    }
+    __device__ __forceinline__ bool peek(int32_t i, int32_t &m, uint64_t &x) const {
+        const uint32_t h = at(i);
+        m = T.keys[h];
+        x = ((uint64_t)T.it[h] << 32) | T.lo[h];
+        return m >= 0;
+    }
+    __device__ __forceinline__ void clear(int32_t i) const {
+        const uint32_t h = at(i);
+        T.keys[h] = -1;
+        T.lo[h] = T.it[h] = 0;
+        if constexpr (WIDE) T.hi[h] = 0;
+    }
+};
+
 // ---------------------------------------------------------------- dense table
 // eta[m], inter[m] for every node of the level in shared memory (levels of at
 // most DENSE_N nodes, nodes with large neighbourhoods).
+template <int PIMAX, int BT, bool WIDE>
+__device__ void propose_dense_node(const PropCtx &C, int32_t v, const Tab &T, ListQueue<BT> &Q, Cand *s_top,
+                                   int32_t *s_tmp) {
+    const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0;
+    const Fmt f = fmt_of(deg);
+    const Self S = self_of(C, v);
+    cta_walk(C, v, i0, deg, S.nin, nullptr, Q, DenseIns<WIDE>{T, f});
+    const int32_t cnt = list_best<PIMAX>(C, S, C.n, threadIdx.x, BT, DenseTab<WIDE>{T, f}, [&](auto &tl, int r0, int nr) {
+        if constexpr (PIMAX <= EMIT_W) block_emit_top<PIMAX>(tl, C, v, s_top);
+        else return block_emit_range(tl, C, v, s_top, r0, nr, &s_top[32 * EMIT_W]);
+    });
+    const int32_t tot = block_sum_i32(cnt, s_tmp);
+    if (threadIdx.x == 0) C.nbcnt[v] = tot;
+}
 template <int PIMAX, int BT>
 __global__ void __launch_bounds__(BT) k_propose_dense(PropCtx C, const int32_t *list, const int32_t *count_p) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long *eta = reinterpret_cast<unsigned long long *>(smem);
-    uint32_t *inter = reinterpret_cast<uint32_t *>(eta + C.n);
-    __shared__ Cand s_top[32 * PIMAX];
-    __shared__ int32_t s_qe[BT];
-    __shared__ unsigned long long s_qq[BT];
-    __shared__ uint32_t s_qc[BT];
-    __shared__ int32_t s_nbig;
+    uint32_t *w = reinterpret_cast<uint32_t *>(smem);
+    const Tab T{nullptr, w, w + 2 * C.n, w + C.n};
+    __shared__ ListQueue<BT> Q;
+    __shared__ Cand s_top[32 * EMIT_W + 1];
     __shared__ int32_t s_tmp[32];
     const int32_t count = *count_p;
-    if (count == 0) return;
-    for (int32_t i = threadIdx.x; i < C.n; i += BT) {
-        eta[i] = 0;
-        inter[i] = 0;
-    }
-    if (threadIdx.x == 0) s_nbig = 0;
+    if ((int32_t)blockIdx.x >= count) return;
+    for (int32_t i = threadIdx.x; i < 3 * C.n; i += BT) w[i] = 0;
+    if (threadIdx.x < 2) Q.n[threadIdx.x] = Q.next[threadIdx.x] = 0;
     __syncthreads();
-    const uint64_t cap = *C.cap;
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
         const int32_t v = list[k];
-        const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0, nin_v = C.nin[v];
-        cta_walk(C, v, i0, deg, nin_v, nullptr, BigQueue{s_qe, s_qq, s_qc, &s_nbig},
-                 [&](int32_t m, unsigned long long eq, uint32_t ic) {
-            add_u64_split(&eta[m], eq);
-            if (ic) atomicAdd(&inter[m], ic);
-        });
-        __syncthreads();
-        if constexpr (PIMAX <= EMIT_W) {
-            TopList<PIMAX> tl;
-            tl.init();
-            int32_t cnt = 0;
-            for (int32_t m = threadIdx.x; m < C.n; m += BT) {
-                unsigned long long em = eta[m];
-                if (em) {
-                    cnt++;
-                    int32_t it = (int32_t)inter[m];
-                    if (pair_valid(C, v, m, it)) tl.push(Cand{em + pair_noise(C.level_key, v, m, cap), m});
-                    eta[m] = 0;
-                    inter[m] = 0;
-                }
-            }
-            int32_t tot = block_sum_i32(cnt, s_tmp);
-            if (threadIdx.x == 0) C.nbcnt[v] = tot;
-            block_emit_top<PIMAX>(tl, C, v, s_top);
-        } else {
-            Cand thr{~0ull, INT32_MAX};
-            for (int r0 = 0; r0 < C.pi; r0 += EMIT_W) {
-                TopList<EMIT_W> tl;
-                tl.init();
-                for (int32_t m = threadIdx.x; m < C.n; m += BT) {
-                    const unsigned long long em = eta[m];
-                    if (em && pair_valid(C, v, m, (int32_t)inter[m])) {
-                        const Cand c{em + pair_noise(C.level_key, v, m, cap), m};
-                        if (cand_gt(thr, c)) tl.push(c);
-                    }
-                }
-                thr = block_emit_range(tl, C, v, s_top, r0, min(EMIT_W, C.pi - r0), &s_top[32 * PIMAX - 1]);
-            }
-            int32_t cnt = 0;
-            for (int32_t m = threadIdx.x; m < C.n; m += BT) {
-                if (eta[m]) {
-                    cnt++;
-                    eta[m] = 0;
-                    inter[m] = 0;
-                }
-            }
-            int32_t tot = block_sum_i32(cnt, s_tmp);
-            if (threadIdx.x == 0) C.nbcnt[v] = tot;
-        }
+        if (C.ioff[v + 1] - C.ioff[v] <= C.deg_narrow) propose_dense_node<PIMAX, BT, false>(C, v, T, Q, s_top, s_tmp);
+        else propose_dense_node<PIMAX, BT, true>(C, v, T, Q, s_top, s_tmp);
     }
 }
 
 // ---------------------------------------------------------------- warp per node
 // Nodes whose neighbourhood bound is at most half the per-warp table: one
-// warp per node, no block barriers.  Incident hyperedges of up to 32 pins are
-// spread over the lanes (one hyperedge per lane), larger ones lane per pin.
+// warp per node, no block barriers, two-word counters only.
 constexpr int WP_T = 256;
-__device__ __forceinline__ uint32_t hslot_w(int32_t m, uint32_t mask) {
-    return mask ? ((uint32_t)m * 0x9E3779B1u) >> __clz(mask) : 0u;   // top bits (Fibonacci hashing)
-}
-__device__ __forceinline__ void warp_insert(int32_t *keys, unsigned long long *eta, uint32_t *inter, uint32_t mask,
-                                            uint32_t cap, int32_t m, unsigned long long qe, uint32_t ninter) {
-    uint32_t h = hslot_w(m, mask);
-    for (uint32_t probe = 0; probe < cap; probe++) {
-        int32_t k = ((volatile int32_t *)keys)[h];
-        if (k == -1) {
-            int32_t old = atomicCAS(&keys[h], -1, m);
-            k = old == -1 ? m : old;
-        }
-        if (k == m) {
-            add_u64_split(&eta[h], qe);
-            if (ninter) atomicAdd(&inter[h], ninter);
-            return;
-        }
-        h = (h + 1) & mask;
-    }
-}
 template <int PIMAX>
 __global__ void __launch_bounds__(WP_T) k_propose_warp(PropCtx C, const int32_t *list, const int32_t *count_p,
                                                        uint32_t cap) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) unsigned char smem[];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwb = WP_T / 32;
-    unsigned long long *eta = reinterpret_cast<unsigned long long *>(smem) + (size_t)wid * cap;
-    uint32_t *inter = reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(smem) + (size_t)nwb * cap) +
-                      (size_t)wid * cap;
-    int32_t *keys = reinterpret_cast<int32_t *>(reinterpret_cast<uint32_t *>(reinterpret_cast<unsigned long long *>(
-                                                    smem) + (size_t)nwb * cap) + (size_t)nwb * cap) +
-                    (size_t)wid * cap;
+    uint32_t *w = reinterpret_cast<uint32_t *>(smem);
+    const Tab T{reinterpret_cast<int32_t *>(w) + (size_t)wid * cap, w + (size_t)(nwb + wid) * cap, nullptr,
+                w + (size_t)(2 * nwb + wid) * cap};
     const int32_t count = *count_p;
-    if (count == 0) return;
-    const uint32_t mask = cap - 1;
-    for (uint32_t i = lane; i < cap; i += 32) {
-        keys[i] = -1;
-        eta[i] = 0;
-        inter[i] = 0;
-    }
-    __syncwarp();
-    const uint64_t capn = *C.cap;
     const int64_t gw = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    if (gw >= count) return;
+    for (uint32_t i = lane; i < cap; i += 32) {
+        T.keys[i] = -1;
+        T.lo[i] = 0;
+        T.it[i] = 0;
+    }
+    __syncwarp();
     for (int64_t k = gw; k < count; k += nw) {
         const int32_t v = list[k];
-        const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0, nin_v = C.nin[v];
-        // all incident hyperedges, one per lane, combined across the warp
-        warp_walk(C, v, i0, deg, nin_v, [&](int32_t m, unsigned long long eq, uint32_t ic) {
-            warp_insert(keys, eta, inter, mask, cap, m, eq, ic);
-        });
+        const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0;
+        const Fmt f = fmt_of(deg);
+        const Self S = self_of(C, v);
+        warp_walk(C, v, i0, deg, S.nin, WarpIns{T, f, cap - 1});
         __syncwarp();
-        // the warp's best entries r0.. of v's list from the lanes' lists
-        auto emit = [&](auto &tl, int r0, int nr) {
+        int32_t cnt = list_best<PIMAX>(C, S, (int32_t)cap, lane, 32, HashTab<false, uint32_t>{T, f, nullptr},
+                                       [&](auto &tl, int r0, int nr) {
             Cand last{0, -1};
             for (int r = 0; r < nr; r++) {
-                Cand best = tl.c[0];
-                int owner = lane;
-                for (int o = 16; o > 0; o >>= 1) {
-                    Cand ob{__shfl_xor_sync(0xffffffffu, best.eta, o), __shfl_xor_sync(0xffffffffu, best.id, o)};
-                    int oo = __shfl_xor_sync(0xffffffffu, owner, o);
-                    if (cand_gt(ob, best)) {
-                        best = ob;
-                        owner = oo;
-                    }
-                }
+                last = warp_pop_best(tl);
                 if (lane == 0) {
-                    C.cand[(int64_t)v * C.pi + r0 + r] = best.id;
-                    C.cscore[(int64_t)v * C.pi + r0 + r] = best.id >= 0 ? best.eta : 0;
+                    C.cand[(int64_t)v * C.pi + r0 + r] = last.id;
+                    C.cscore[(int64_t)v * C.pi + r0 + r] = last.id >= 0 ? last.eta : 0;
                 }
-                if (best.id >= 0 && lane == owner) tl.pop();
-                last = best;
             }
             return last;
-        };
-        int32_t cnt = 0;
-        if constexpr (PIMAX <= EMIT_W) {
-            TopList<PIMAX> tl;
-            tl.init();
-            for (uint32_t h = lane; h < cap; h += 32) {
-                const int32_t m = keys[h];
-                if (m >= 0) {
-                    cnt++;
-                    if (pair_valid(C, v, m, (int32_t)inter[h])) tl.push(Cand{eta[h] + pair_noise(C.level_key, v, m, capn), m});
-                    keys[h] = -1;
-                    eta[h] = 0;
-                    inter[h] = 0;
-                }
-            }
-            __syncwarp();
-            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            if (lane == 0) C.nbcnt[v] = cnt;
-            emit(tl, 0, C.pi);
-        } else {
-            // rounds of four, each below the last entry of the round before
-            // the first round stores each neighbour's noised score in its eta
-            // slot and its validity in its inter slot, the later rounds only
-            // compare
-            Cand thr{~0ull, INT32_MAX};
-            for (int r0 = 0; r0 < C.pi; r0 += EMIT_W) {
-                TopList<EMIT_W> tl;
-                tl.init();
-                for (uint32_t h = lane; h < cap; h += 32) {
-                    const int32_t m = keys[h];
-                    if (m < 0) continue;
-                    unsigned long long sc = eta[h];
-                    bool ok = inter[h] != 0;
-                    if (r0 == 0) {
-                        ok = pair_valid(C, v, m, (int32_t)inter[h]);
-                        if (ok) sc += pair_noise(C.level_key, v, m, capn);
-                        eta[h] = sc;
-                        inter[h] = ok ? 1u : 0u;
-                    }
-                    if (ok) {
-                        const Cand c{sc, m};
-                        if (cand_gt(thr, c)) tl.push(c);
-                    }
-                }
-                thr = emit(tl, r0, min(EMIT_W, C.pi - r0));
-            }
-            for (uint32_t h = lane; h < cap; h += 32) {
-                if (keys[h] >= 0) {
-                    cnt++;
-                    keys[h] = -1;
-                    eta[h] = 0;
-                    inter[h] = 0;
-                }
-            }
-            __syncwarp();
-            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-            if (lane == 0) C.nbcnt[v] = cnt;
-        }
+        });
+        __syncwarp();
+        cnt = __reduce_add_sync(0xffffffffu, cnt);
+        if (lane == 0) C.nbcnt[v] = cnt;
     }
 }
 
 // ---------------------------------------------------------------- hashed table
-__device__ __forceinline__ uint32_t hslot(int32_t m, uint32_t mask) {
-    return mask ? ((uint32_t)m * 0x9E3779B1u) >> __clz(mask) : 0u;   // top bits (Fibonacci hashing)
-}
-
-// Table of `cap` slots at keys/eta/inter (shared or global).  Nodes from
-// list[0..count) are processed; a node whose distinct neighbours exceed
-// limit is appended to ovf (and its table cleared).
-template <int PIMAX>
-__device__ void propose_hashed_node(const PropCtx &C, int32_t v, int32_t *keys, unsigned long long *eta,
-                                    uint32_t *inter, uint32_t cap, uint32_t limit, int32_t *slots, int32_t *ovf,
-                                    int32_t *ovf_n, int *s_flag, int32_t *s_cnt, Cand *s_top,
-                                    int32_t *s_tmp, BigQueue BQ) {
-    const uint32_t mask = cap - 1;
-    const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0, nin_v = C.nin[v];
-    auto insert_n = [&](int32_t m, unsigned long long qe, uint32_t ninter) {
-        uint32_t h = hslot(m, mask);
-        for (uint32_t probe = 0; probe < cap; probe++) {
-            int32_t k = ((volatile int32_t *)keys)[h];
-            if (k == -1) {
-                int32_t old = atomicCAS(&keys[h], -1, m);
-                if (old == -1) {
-                    const uint32_t slot = (uint32_t)atomicAdd(s_cnt, 1);
-                    if (slot < limit) slots[slot] = (int32_t)h;
-                    else *(volatile int *)s_flag = 1;
-                    k = m;
-                } else {
-                    k = old;
-                }
-            }
-            if (k == m) {
-                add_u64_split(&eta[h], qe);
-                if (ninter) atomicAdd(&inter[h], ninter);
-                return;
-            }
-            h = (h + 1) & mask;
-        }
-    };
-    cta_walk(C, v, i0, deg, nin_v, s_flag, BQ, insert_n);
-    __syncthreads();
-    const int overflow = *s_flag;
-    const uint64_t capn = *C.cap;
-    if (overflow) {
+// Table of mask + 1 slots (shared or global); a node whose distinct neighbours
+// exceed `limit` is appended to ovf (and its table cleared).
+template <int PIMAX, int BT, bool WIDE, class Slot>
+__device__ void propose_hashed_node(const PropCtx &C, int32_t v, const Tab &T, uint32_t mask, uint32_t limit,
+                                    Slot *slots, int32_t *ovf, int32_t *ovf_n, int *s_flag, int32_t *s_cnt,
+                                    Cand *s_top, ListQueue<BT> &Q) {
+    const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0;
+    const Fmt f = fmt_of(deg);
+    const Self S = self_of(C, v);
+    cta_walk(C, v, i0, deg, S.nin, s_flag, Q, HashIns<WIDE, Slot>{T, f, mask, limit, slots, s_cnt, s_flag});
+    if (*(volatile int *)s_flag) {
         // the slot list is incomplete: clear the whole table, redo the node in a larger one
-        for (uint32_t h = threadIdx.x; h < cap; h += blockDim.x) {
-            keys[h] = -1;
-            eta[h] = 0;
-            inter[h] = 0;
+        for (uint32_t h = threadIdx.x; h <= mask; h += BT) {
+            T.keys[h] = -1;
+            T.lo[h] = T.it[h] = 0;
+            if constexpr (WIDE) T.hi[h] = 0;
         }
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -795,98 +866,53 @@ __device__ void propose_hashed_node(const PropCtx &C, int32_t v, int32_t *keys, 
     }
     // only the occupied slots, from the slot list
     const int32_t used = *(volatile int32_t *)s_cnt;
-    if constexpr (PIMAX <= EMIT_W) {
-        TopList<PIMAX> tl;
-        tl.init();
-        for (int32_t i = threadIdx.x; i < used; i += blockDim.x) {
-            const int32_t h = slots[i];
-            const int32_t m = keys[h];
-            if (pair_valid(C, v, m, (int32_t)inter[h])) tl.push(Cand{eta[h] + pair_noise(C.level_key, v, m, capn), m});
-            keys[h] = -1;
-            eta[h] = 0;
-            inter[h] = 0;
-        }
-        int32_t tot = used;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            C.nbcnt[v] = tot;
-            *s_cnt = 0;
-        }
-        block_emit_top<PIMAX>(tl, C, v, s_top);
-    } else {
-        // rounds of four over the slot list, each below the last entry of the round before
-        // (the first round stores the noised scores in eta and the validity
-        // in inter)
-        Cand thr{~0ull, INT32_MAX};
-        for (int r0 = 0; r0 < C.pi; r0 += EMIT_W) {
-            TopList<EMIT_W> tl;
-            tl.init();
-            for (int32_t i = threadIdx.x; i < used; i += blockDim.x) {
-                const int32_t h = slots[i];
-                const int32_t m = keys[h];
-                unsigned long long sc = eta[h];
-                bool ok = inter[h] != 0;
-                if (r0 == 0) {
-                    ok = pair_valid(C, v, m, (int32_t)inter[h]);
-                    if (ok) sc += pair_noise(C.level_key, v, m, capn);
-                    eta[h] = sc;
-                    inter[h] = ok ? 1u : 0u;
-                }
-                if (ok) {
-                    const Cand c{sc, m};
-                    if (cand_gt(thr, c)) tl.push(c);
-                }
-            }
-            thr = block_emit_range(tl, C, v, s_top, r0, min(EMIT_W, C.pi - r0), &s_top[32 * PIMAX - 1]);
-        }
-        for (int32_t i = threadIdx.x; i < used; i += blockDim.x) {
-            const int32_t h = slots[i];
-            keys[h] = -1;
-            eta[h] = 0;
-            inter[h] = 0;
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            C.nbcnt[v] = used;
-            *s_cnt = 0;
-        }
-        __syncthreads();
+    list_best<PIMAX>(C, S, used, threadIdx.x, BT, HashTab<WIDE, Slot>{T, f, slots}, [&](auto &tl, int r0, int nr) {
+        if constexpr (PIMAX <= EMIT_W) block_emit_top<PIMAX>(tl, C, v, s_top);
+        else return block_emit_range(tl, C, v, s_top, r0, nr, &s_top[32 * EMIT_W]);
+    });
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        C.nbcnt[v] = used;
+        *s_cnt = 0;
     }
+    __syncthreads();
 }
 
-template <int PIMAX, int BT>
+// bytes of a shared-memory table of cap slots and its slot list
+__host__ __device__ constexpr size_t hash_smem(uint32_t cap, bool wide) {
+    return (size_t)cap * (wide ? 16 : 12) + (size_t)(cap * 3 / 4) * sizeof(uint16_t);
+}
+// BOTH: nodes of any number of hyperedges; else only those with two-word counters
+template <int PIMAX, int BT, bool BOTH>
 __global__ void __launch_bounds__(BT) k_propose_smem(PropCtx C, const int32_t *list, const int32_t *count_p,
                                                      uint32_t cap, uint32_t limit, int32_t *ovf, int32_t *ovf_n) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) unsigned char smem[];
-    unsigned long long *eta = reinterpret_cast<unsigned long long *>(smem);
-    uint32_t *inter = reinterpret_cast<uint32_t *>(eta + cap);
-    int32_t *keys = reinterpret_cast<int32_t *>(inter + cap);
-    int32_t *slots = keys + cap;
-    __shared__ Cand s_top[32 * PIMAX];
-    __shared__ int32_t s_qe[BT];
-    __shared__ unsigned long long s_qq[BT];
-    __shared__ uint32_t s_qc[BT];
-    __shared__ int32_t s_nbig;
-    __shared__ int32_t s_tmp[32];
+    uint32_t *w = reinterpret_cast<uint32_t *>(smem);
+    const Tab T{reinterpret_cast<int32_t *>(w), w + cap, BOTH ? w + 3 * cap : nullptr, w + 2 * cap};
+    uint16_t *slots = reinterpret_cast<uint16_t *>(w + (BOTH ? 4 : 3) * cap);
+    __shared__ ListQueue<BT> Q;
+    __shared__ Cand s_top[32 * EMIT_W + 1];
     __shared__ int s_flag;
     __shared__ int32_t s_cnt;
     const int32_t count = *count_p;
-    if (count == 0) return;
-    for (uint32_t i = threadIdx.x; i < cap; i += BT) {
-        keys[i] = -1;
-        eta[i] = 0;
-        inter[i] = 0;
-    }
+    if ((int32_t)blockIdx.x >= count) return;
+    for (uint32_t i = threadIdx.x; i < (BOTH ? 4 : 3) * cap; i += BT) w[i] = i < cap ? 0xffffffffu : 0u;
+    if (threadIdx.x < 2) Q.n[threadIdx.x] = Q.next[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         s_flag = 0;
         s_cnt = 0;
-        s_nbig = 0;
     }
     __syncthreads();
-    for (int32_t k = blockIdx.x; k < count; k += gridDim.x)
-        propose_hashed_node<PIMAX>(C, list[k], keys, eta, inter, cap, limit, slots, ovf, ovf_n, &s_flag, &s_cnt,
-                                   s_top, s_tmp, BigQueue{s_qe, s_qq, s_qc, &s_nbig});
+    for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
+        const int32_t v = list[k];
+        bool wide = false;
+        if constexpr (BOTH) wide = C.ioff[v + 1] - C.ioff[v] > C.deg_narrow;
+        if (!wide)
+            propose_hashed_node<PIMAX, BT, false>(C, v, T, cap - 1, limit, slots, ovf, ovf_n, &s_flag, &s_cnt, s_top, Q);
+        else if constexpr (BOTH)
+            propose_hashed_node<PIMAX, BT, true>(C, v, T, cap - 1, limit, slots, ovf, ovf_n, &s_flag, &s_cnt, s_top, Q);
+    }
 }
 
 // one CTA region of gcap slots in global memory per CTA (clean on entry and
@@ -897,39 +923,46 @@ __global__ void __launch_bounds__(PT) k_propose_global(PropCtx C, const int32_t 
                                                        uint32_t *ginter, int32_t *gslots, int32_t *err_list,
                                                        int32_t *err_n) {
     HP_KERNEL_ENTER();
-    __shared__ Cand s_top[32 * PIMAX];
-    __shared__ int32_t s_qe[PT];
-    __shared__ unsigned long long s_qq[PT];
-    __shared__ uint32_t s_qc[PT];
-    __shared__ int32_t s_nbig;
-    __shared__ int32_t s_tmp[32];
+    __shared__ ListQueue<PT> Q;
+    __shared__ Cand s_top[32 * EMIT_W + 1];
     __shared__ int s_flag;
     __shared__ int32_t s_cnt;
     const int32_t count = *count_p;
-    if (count == 0) return;
+    if ((int32_t)blockIdx.x >= count) return;
     const int64_t o = (int64_t)blockIdx.x * gcap;
+    uint32_t *eta = reinterpret_cast<uint32_t *>(geta + o);
+    const Tab T{gkeys + o, eta, eta + gcap, ginter + o};
+    if (threadIdx.x < 2) Q.n[threadIdx.x] = Q.next[threadIdx.x] = 0;
     if (threadIdx.x == 0) {
         s_flag = 0;
         s_cnt = 0;
-        s_nbig = 0;
     }
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x)
-        propose_hashed_node<PIMAX>(C, list[k], gkeys + o, geta + o, ginter + o, gcap, gcap - 1, gslots + o, err_list,
-                                   err_n, &s_flag, &s_cnt, s_top, s_tmp, BigQueue{s_qe, s_qq, s_qc, &s_nbig});
+        propose_hashed_node<PIMAX, PT, true>(C, list[k], T, gcap - 1, gcap - 1, gslots + o, err_list, err_n, &s_flag,
+                                             &s_cnt, s_top, Q);
 }
 
 // ---------------------------------------------------------------- node tiers
-// warp tier: small neighbourhood bound and little traversal work; hub
-// tier: traversals (pin visits or incidence entries) large enough to keep a
-// 1024-thread CTA busy
-// dense tier (level of at most DENSE_N nodes): neighbourhood bound above
-// dense_bound; the others use hashed tables
-constexpr long long WARP_VISITS = 4096, HUB_VISITS = 262144;
-constexpr int32_t HUB_INCIDENCE = 4096;   // incidence entries: chunks of a 512-thread walk
-__global__ void k_tiers(const int32_t *bound, const long long *vis, const int32_t *ioff, int32_t n,
-                        uint32_t warp_limit, int32_t dense_bound, int32_t *lW, int32_t *lB, int32_t *lH, int32_t *lD,
-                        int32_t *lDH, int32_t *cnt, int32_t pi, int32_t *cand, uint64_t *cscore) {
+// warp tier: small neighbourhood bound and little traversal work, and two-word
+// counters; hub tier: traversals (pin visits or incidence entries) large
+// enough to keep a 1024-thread CTA busy, and the nodes that need the wide
+// counters.  Dense tiers (level of at most DENSE_N nodes): neighbourhood bound
+// above dense_bound, by the same split; the others use hashed tables.  On
+// levels of at most DENSE_ALL nodes there are too few nodes to fill the GPU a
+// warp each: only walks of up to WARP_VISITS_FEW pins stay with a warp, and
+// every other node takes a dense table, which costs it no probes.
+constexpr long long WARP_VISITS = 4096, WARP_VISITS_FEW = 512, HUB_VISITS = 262144, HUB_VISITS_FEW = 16384;
+constexpr int32_t HUB_INCIDENCE = 4096;   // incidence entries: chunks of a walk
+constexpr int32_t DENSE_ALL = 4096;
+struct TierRule {
+    uint32_t warp_limit;
+    int32_t dense_bound, deg_narrow;
+    long long warp_visits, hub_visits;
+};
+__global__ void k_tiers(const int32_t *bound, const long long *vis, const int32_t *ioff, int32_t n, TierRule R,
+                        int32_t *lW, int32_t *lB, int32_t *lH, int32_t *lD, int32_t *lDH, int32_t *cnt, int32_t pi,
+                        int32_t *cand, uint64_t *cscore) {
     HP_KERNEL_ENTER();
     GRID_STRIDE(v, (int64_t)n) {
         if (bound[v] == 0) {
@@ -940,9 +973,10 @@ __global__ void k_tiers(const int32_t *bound, const long long *vis, const int32_
             }
             continue;
         }
-        const bool hub = vis[v] > HUB_VISITS || ioff[v + 1] - ioff[v] > HUB_INCIDENCE;
-        if ((uint32_t)bound[v] <= warp_limit && vis[v] <= WARP_VISITS) lW[atomicAdd(&cnt[0], 1)] = (int32_t)v;
-        else if (bound[v] > dense_bound) {
+        const int32_t deg = ioff[v + 1] - ioff[v];
+        const bool wide = deg > R.deg_narrow, hub = vis[v] > R.hub_visits || deg > HUB_INCIDENCE || wide;
+        if ((uint32_t)bound[v] <= R.warp_limit && vis[v] <= R.warp_visits && !wide) lW[atomicAdd(&cnt[0], 1)] = (int32_t)v;
+        else if (bound[v] > R.dense_bound) {
             if (hub) lDH[atomicAdd(&cnt[7], 1)] = (int32_t)v;
             else lD[atomicAdd(&cnt[6], 1)] = (int32_t)v;
         } else if (hub) lH[atomicAdd(&cnt[5], 1)] = (int32_t)v;
@@ -987,63 +1021,85 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
     const int32_t dbg = P.o.debug_table_cap;
     const uint32_t wcap = dbg > 0 ? std::min<uint32_t>(512, (uint32_t)dbg) : 512;
     uint32_t capB = 4096, capC = 8192;
-    if (dbg > 0) capB = capC = (uint32_t)dbg;
+    if (dbg > 0) capB = capC = (uint32_t)std::min(dbg, 8192);
+    TierRule R;
+    R.warp_limit = wcap / 2;
+    R.deg_narrow = C.deg_narrow;
+    R.warp_visits = C.n <= DENSE_ALL ? WARP_VISITS_FEW : WARP_VISITS;
+    R.hub_visits = HUB_VISITS;
     // dense tables only on small levels, for neighbourhoods too large for the first hashed table
-    const int32_t dense_bound = (C.n <= DENSE_N && dbg == 0) ? (int32_t)(capB / 2) : 0x7fffffff;
-    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.vis, L.ioff, C.n, wcap / 2, dense_bound, W.lW, W.lB, W.lH,
-                                              W.lD, W.lDH, W.cnt, C.pi, C.cand, C.cscore);
+    R.dense_bound = 0x7fffffff;
+    if (C.n <= DENSE_N && dbg == 0) R.dense_bound = (int32_t)(capB / 2);
+    if (C.n <= DENSE_ALL && dbg == 0) {
+        R.dense_bound = 0;
+        R.hub_visits = HUB_VISITS_FEW;
+    }
+    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.vis, L.ioff, C.n, R, W.lW, W.lB, W.lH, W.lD, W.lDH, W.cnt,
+             C.pi, C.cand, C.cscore);
     HP_LAUNCH_CHECK();
     // the tiers take disjoint node lists, so they run side by side: the warp
     // tier, the dense tier and the hub tier each on a side stream, tier B on
     // the main one; tier C (overflows of B and the hubs) waits for the hubs,
     // and the global tier (whose error list reuses the warp list) for all
     cudaStream_t sw = W.side[0], sd = W.side[1], sh = W.side[2];
+    const bool dense = R.dense_bound != 0x7fffffff, hashed = R.dense_bound != 0;
     HPC(cudaEventRecord(W.ev[0], s));
-    for (cudaStream_t x : {sw, sd, sh}) HPC(cudaStreamWaitEvent(x, W.ev[0], 0));
+    HPC(cudaStreamWaitEvent(sw, W.ev[0], 0));
+    if (dense) HPC(cudaStreamWaitEvent(sd, W.ev[0], 0));
+    if (hashed) HPC(cudaStreamWaitEvent(sh, W.ev[0], 0));
     {
-        size_t sm = (size_t)wcap * 16 * (WP_T / 32);
+        size_t sm = (size_t)wcap * 12 * (WP_T / 32);
         int occ = prepare_kernel((const void *)k_propose_warp<PIMAX>, WP_T, sm);
         int grid = (int)std::min<int64_t>(cdiv(C.n, WP_T / 32), (int64_t)sms * occ);
         launch_k(k_propose_warp<PIMAX>, std::max(grid, 1), WP_T, sm, sw, C, W.lW, W.cnt + 0, wcap);
         HP_LAUNCH_CHECK();
+        HPC(cudaEventRecord(W.ev[1], sw));
     }
-    if (dense_bound != 0x7fffffff) {
+    if (dense) {
+        // hubs first; the other nodes by CTAs of 256 threads, of 1024 where
+        // the tables leave room for few CTAs on an SM
         size_t sm = (size_t)C.n * 12;
-        int occ = prepare_kernel((const void *)k_propose_dense<PIMAX, PT>, PT, sm);
-        launch_k(k_propose_dense<PIMAX, PT>, std::max(1, std::min<int>(C.n, sms * occ)), PT, sm, sd, C, W.lD, W.cnt + 6);
+        const int occ_h = prepare_kernel((const void *)k_propose_dense<PIMAX, 1024>, 1024, sm);
+        cudaStream_t sdh = hashed ? sd : s;   // (no hashed tiers: the main stream is free)
+        launch_k(k_propose_dense<PIMAX, 1024>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sdh, C, W.lDH,
+                 W.cnt + 7);
         HP_LAUNCH_CHECK();
-        prepare_kernel((const void *)k_propose_dense<PIMAX, 1024>, 1024, sm);
-        launch_k(k_propose_dense<PIMAX, 1024>, sms, 1024, sm, sd, C, W.lDH, W.cnt + 7);
+        const int occ = prepare_kernel((const void *)k_propose_dense<PIMAX, PT>, PT, sm);
+        if (occ * PT >= occ_h * 1024)
+            launch_k(k_propose_dense<PIMAX, PT>, std::max(1, std::min<int>(C.n, sms * occ)), PT, sm, sd, C, W.lD, W.cnt + 6);
+        else
+            launch_k(k_propose_dense<PIMAX, 1024>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sd, C, W.lD,
+                     W.cnt + 6);
         HP_LAUNCH_CHECK();
+        HPC(cudaEventRecord(W.ev[2], sd));
     }
-    auto smem_of = [](uint32_t cap) { return (size_t)cap * 16 + (size_t)(cap * 3 / 4) * 4; };
-    {
-        size_t sm = smem_of(capB);
-        prepare_kernel((const void *)k_propose_smem<PIMAX, 1024>, 1024, sm);
-        launch_k(k_propose_smem<PIMAX, 1024>, sms, 1024, sm, sh, C, W.lH, W.cnt + 5, capB, capB * 3 / 4, W.lC, W.cnt + 2);
+    if (hashed) {
+        size_t sm = hash_smem(capB, true);
+        const int occ_h = prepare_kernel((const void *)k_propose_smem<PIMAX, 1024, true>, 1024, sm);
+        launch_k(k_propose_smem<PIMAX, 1024, true>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sh, C, W.lH,
+                 W.cnt + 5, capB, capB * 3 / 4, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
-        int occ = prepare_kernel((const void *)k_propose_smem<PIMAX, 512>, 512, sm);
-        launch_k(k_propose_smem<PIMAX, 512>, std::max(1, std::min<int>(C.n, sms * occ)), 512, sm, s,
+        HPC(cudaEventRecord(W.ev[3], sh));
+        sm = hash_smem(capB, false);
+        int occ = prepare_kernel((const void *)k_propose_smem<PIMAX, PT, false>, PT, sm);
+        launch_k(k_propose_smem<PIMAX, PT, false>, std::max(1, std::min<int>(C.n, sms * occ)), PT, sm, s,
             C, W.lB, W.cnt + 1, capB, capB * 3 / 4, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
-    }
-    HPC(cudaEventRecord(W.ev[3], sh));
-    HPC(cudaStreamWaitEvent(s, W.ev[3], 0));
-    {
+        HPC(cudaStreamWaitEvent(s, W.ev[3], 0));
         // nodes whose neighbourhood outgrew the first table (the bound can be far above the truth)
-        size_t sm = smem_of(capC);
-        int occ = prepare_kernel((const void *)k_propose_smem<PIMAX, PT>, PT, sm);
-        launch_k(k_propose_smem<PIMAX, PT>, std::max(1, std::min<int>(C.n, sms * occ)), PT, sm, s,
+        sm = hash_smem(capC, true);
+        occ = prepare_kernel((const void *)k_propose_smem<PIMAX, 1024, true>, 1024, sm);
+        launch_k(k_propose_smem<PIMAX, 1024, true>, std::max(1, std::min<int>(C.n, sms * occ)), 1024, sm, s,
             C, W.lC, W.cnt + 2, capC, capC * 3 / 4, W.lG, W.cnt + 3);
         HP_LAUNCH_CHECK();
     }
-    HPC(cudaEventRecord(W.ev[1], sw));
-    HPC(cudaEventRecord(W.ev[2], sd));
     HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
-    HPC(cudaStreamWaitEvent(s, W.ev[2], 0));
-    launch_k(k_propose_global<PIMAX>, W.gnb, PT, 0, s, C, W.lG, W.cnt + 3, W.gcap, W.gkeys, W.geta, W.ginter, W.gslots,
-                                                  W.lW, W.cnt + 4);
-    HP_LAUNCH_CHECK();
+    if (dense) HPC(cudaStreamWaitEvent(s, W.ev[2], 0));
+    if (hashed) {
+        launch_k(k_propose_global<PIMAX>, W.gnb, PT, 0, s, C, W.lG, W.cnt + 3, W.gcap, W.gkeys, W.geta, W.ginter, W.gslots,
+                                                      W.lW, W.cnt + 4);
+        HP_LAUNCH_CHECK();
+    }
 }
 
 // ---------------------------------------------------------------- best-effort pairing
@@ -1581,7 +1637,9 @@ static void propose_lists(Level &L, int32_t level, const int32_t *w, const Param
     C.inc = L.inc;
     C.nin = L.nin;
     C.q = W.q;
-    C.cap = &box->cap;
+    C.cap = &box->cap;   // (cap_inv follows it)
+    // q(e) = w 2^24 / |e| with |e| >= 2 has at most bits(max w) + 23 bits
+    C.deg_narrow = (1 << ((64 - 23 - bits_for((uint64_t)P.wmax)) / 3)) - 1;
     {
         // the level key folds seed and level exactly as the oracle's noise
         uint64_t z = P.seed + 0x9E3779B97F4A7C15ull * (uint64_t)(level + 1);

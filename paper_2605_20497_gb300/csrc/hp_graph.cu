@@ -2,6 +2,8 @@
 // hypergraph construction (Sec. V-E).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "hp_cluster.cuh"
 #include "hp_internal.cuh"
 
@@ -27,8 +29,10 @@ __global__ void k_check_offsets(const int32_t *off, int32_t e, uint32_t *err) {
 }
 
 __global__ void k_edges_level0(const int32_t *off, int32_t e, const int32_t *src_counts, const int32_t *weights,
-                               int32_t kind, int32_t *nsrc, int32_t *w, unsigned long long *wsum, uint32_t *err) {
+                               int32_t kind, int32_t *nsrc, int32_t *w, unsigned long long *wsum, int32_t *wmax,
+                               uint32_t *err) {
     HP_KERNEL_ENTER();
+    int32_t mx = 0;
     GRID_STRIDE(i, (int64_t)e) {
         int32_t sz = off[i + 1] - off[i];
         int32_t s = src_counts ? src_counts[i] : 1;
@@ -38,7 +42,10 @@ __global__ void k_edges_level0(const int32_t *off, int32_t e, const int32_t *src
         if (wi < 1 || wi > 65536) atomicOr(err, E_WEIGHT);
         w[i] = wi;
         if (weights) atomicAdd(wsum, (unsigned long long)(wi < 0 ? 0 : wi));
+        mx = max(mx, wi);
     }
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(wmax, mx);
 }
 
 // pedge[j] = hyperedge of pin position j (one warp per hyperedge)
@@ -149,7 +156,7 @@ uint32_t validate_and_build_level0(const int32_t *pins, const int32_t *offsets, 
     struct Box {
         uint32_t err, pad;
         unsigned long long wsum;
-        int32_t np;
+        int32_t np, wmax;
     };
     Box *box = A.get<Box>(1);
     HPC(cudaMemsetAsync(box, 0, sizeof(Box), s));
@@ -176,7 +183,7 @@ uint32_t validate_and_build_level0(const int32_t *pins, const int32_t *offsets, 
     L.pedge = A.get<int32_t>(L.np);
     if (e > 0) {
         launch_k(k_edges_level0, grid_of(e, 256), 256, 0, s, L.off, e, src_counts, weights, P.o.count_kind, L.nsrc, w,
-                 &box->wsum, &box->err);
+                 &box->wsum, &box->wmax, &box->err);
         HP_LAUNCH_CHECK();
         launch_k(k_pin_edges, grid_of((int64_t)e * 32, 256), 256, 0, s, L.off, e, L.pedge);
         HP_LAUNCH_CHECK();
@@ -200,6 +207,7 @@ uint32_t validate_and_build_level0(const int32_t *pins, const int32_t *offsets, 
     fetch_bytes(&hb, box, sizeof(Box), s);
     if (hb.wsum > (1ull << 37)) hb.err |= E_WSUM;
     P.wsum = weights ? (int64_t)hb.wsum : (int64_t)e;
+    P.wmax = std::min(std::max(hb.wmax, 1), 65536);
     A.release(box);
     return hb.err;
 }

@@ -378,6 +378,7 @@ struct Params {
     uint64_t seed;
     hp_options o;
     int64_t wsum = 0;   // sum of hyperedge weights (bounds any gain)
+    int32_t wmax = 65536;   // no weight is above
 };
 
 // graph construction (hp_graph.cu)
@@ -392,6 +393,7 @@ void make_level(int32_t n, int32_t e, const int32_t *off, const int32_t *pins, c
 struct LevelBox {
     unsigned long long qsum, visits, pairs, iso, nbrs;
     uint64_t cap;      // noise cap of the level
+    uint64_t cap_inv;  // floor((2^64 - 1) / (cap + 1)), next to it
     int32_t cn, cnp;   // nodes and pins of the coarse level
     uint32_t err;      // error bits raised by the level's matching
     int32_t isolist;   // nodes without a valid neighbour (the best-effort pairing's list)
