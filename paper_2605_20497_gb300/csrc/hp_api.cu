@@ -166,6 +166,7 @@ static hp_status run(const int32_t *pins, const int32_t *offsets, int32_t e, int
                            std::to_string(hb.err) + ")";
             return status_of(hb.err);
         }
+        coarsen_note(CW, lv[L], hb);
         st.pin_visits += (int64_t)hb.visits;
         {
             // algorithmic bytes of the level (see hp_stats.alg_bytes)

@@ -400,6 +400,8 @@ struct LevelBox {
     int32_t ntargets;  // distinct targets of the first proposal graph
     int32_t maxin;     // largest in-degree of the first proposal graph
     unsigned long long pairs1;   // pairs of the first matching round
+    int32_t ngroups;   // groups of equal destination lists (0: not looked for)
+    int32_t pad;
 };
 // Contraction (Sec. V-E): computes the coarse sizes into box_dev, reads the
 // box once into box_host; returns false and builds nothing when the level
@@ -415,6 +417,8 @@ struct CoarsenWs;
 CoarsenWs *coarsen_workspace(int32_t n, int32_t e, const Params &P, Arena &A);
 void coarsen_workspace_free(CoarsenWs *W, Arena &A);
 LevelBox *coarsen_box(CoarsenWs *W);
+// what the host keeps of a finished level's counters for the next ones
+void coarsen_note(CoarsenWs *W, const Level &L, const LevelBox &hb);
 // One level on the device, no host synchronisation; counters in the box.
 // prop_events (optional): two events recorded around the proposal launches
 void coarsen_level(Level &L, int32_t level, const int32_t *w, const Params &P, int32_t *mate, CoarsenWs &W, Arena &A,

@@ -38,18 +38,20 @@ def test_windows(torch, window, weights):
     check(g, 500, 10 ** 6, chain_window=window)
 
 
+# 45,056 moves is the most one cluster sorts
+@pytest.mark.parametrize("n,least,most", [(12000, 4097, 45056), (70000, 45057, 70000)])
 @pytest.mark.parametrize("window", [1, 33, 256])
 @pytest.mark.parametrize("weights", [False, True])
-def test_one_repetition_device_wide(torch, window, weights):
-    # a random part vector: nearly every node proposes a move, more than one cluster sequences on a step call
+def test_one_repetition_device_wide(torch, n, least, most, window, weights):
+    # a random part vector: most nodes propose a move, more than one cluster sequences on a step call
     from test_gpu_steps import gpu_refine
-    g = inputs.random_hypergraph(12000, 18000, 6, seed=5, weights=weights, max_weight=9)
+    g = inputs.random_hypergraph(n, 3 * n // 2, 6, seed=5, weights=weights, max_weight=9)
     rng = np.random.default_rng(window)
     size = rng.integers(1, 4, size=g.num_nodes).astype(np.int32)
     rho = rng.integers(0, 7, size=g.num_nodes).astype(np.int32)
-    omega, delta = 6000, 10 ** 6
+    omega, delta = n, 10 ** 6
     r = gpu_refine(torch, g, size, rho, 7, False, omega, delta, chain_window=window)
-    assert r["m"] > 4096
+    assert least <= r["m"] <= most
     seq = oracle.sequence(g, size, 7, r["node"], r["src"], r["dst"], r["gain"], window=window)
     assert np.array_equal(r["seq"], seq)
 
