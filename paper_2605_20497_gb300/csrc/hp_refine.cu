@@ -292,7 +292,8 @@ constexpr int GN_T = 128;
 
 // gain(v,p) = saving(v) - loss(v,p) with loss = W(v) - conn(v,p), conn(v,p) =
 // sum of w(e) over e in I(v) with pins(p,e) > 0 (singleton hyperedges cancel).
-__device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, const int32_t *inc, const int32_t *w,
+__device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, const int32_t *cutn, const int32_t *inc,
+                           const int32_t *w,
                            const int32_t *rho, const int32_t *size, const long long *psize, const long long *saving,
                            const long long *wns, Plist PL, int32_t omega, int second_half, int32_t *keys,
                            long long *conn, int32_t *slots, uint32_t cap, uint32_t limit, int32_t *s_cnt, int *s_flag,
@@ -328,7 +329,7 @@ __device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, c
     // before one table update per distinct part, so that the few parts a
     // node touches are not hammered by every lane.
     {
-        const int32_t c0 = ioff[v], c1 = ioff[v + 1];
+        const int32_t c0 = ioff[v], c1 = c0 + cutn[v];
         for (int32_t base = c0; base < c1; base += blockDim.x) {
             if (__any_sync(0xffffffffu, *(volatile int *)s_flag)) break;
             const int32_t t = base + (int32_t)threadIdx.x;
@@ -418,7 +419,7 @@ __device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, c
 }
 
 struct GainArgs {
-    const int32_t *off, *ioff, *inc, *w, *rho, *size;
+    const int32_t *off, *ioff, *cutn, *inc, *w, *rho, *size;   // cut hyperedges of v: inc[ioff[v] .. ioff[v] + cutn[v])
     const long long *psize, *saving, *wns;
     Plist PL;
     int32_t omega;
@@ -449,7 +450,7 @@ __global__ void __launch_bounds__(BT) k_gains_smem(GainArgs G, const int32_t *li
     }
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x)
-        gains_node(list[k], G.off, G.ioff, G.inc, G.w, G.rho, G.size, G.psize, G.saving, G.wns, G.PL, G.omega,
+        gains_node(list[k], G.off, G.ioff, G.cutn, G.inc, G.w, G.rho, G.size, G.psize, G.saving, G.wns, G.PL, G.omega,
                    G.second_half, keys, conn, slots, cap, cap * 3 / 4, &s_cnt, &s_flag, G.M, ovf, ovf_n, s_rg, s_rp);
 }
 
@@ -476,7 +477,7 @@ __global__ void __launch_bounds__(GN_T) k_gains_global(GainArgs G, const int32_t
     }
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x)
-        gains_node(list[k], G.off, G.ioff, G.inc, G.w, G.rho, G.size, G.psize, G.saving, G.wns, G.PL, G.omega,
+        gains_node(list[k], G.off, G.ioff, G.cutn, G.inc, G.w, G.rho, G.size, G.psize, G.saving, G.wns, G.PL, G.omega,
                    G.second_half, keys, conn, slots, cap, cap - 1, &s_cnt, &s_flag, G.M, bad, bad_n, s_rg, s_rp);
 }
 
@@ -507,7 +508,7 @@ __global__ void __launch_bounds__(GW_T) k_gains_warp(GainArgs G, const int32_t *
     for (int64_t k = gw; k < count; k += nw) {
         const int32_t v = list[k];
         const int32_t s = G.rho[v];
-        const int32_t c0 = G.ioff[v], c1 = G.ioff[v + 1];
+        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
         for (int32_t base = c0; base < c1; base += 32) {
             if (*(volatile int32_t *)&s_used[wid] > (int32_t)limit) break;   // same value for the whole warp
             const int32_t t = base + lane;
@@ -647,7 +648,7 @@ __global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
         const int32_t v = list[k], s = G.rho[v];
-        const int32_t c0 = G.ioff[v], c1 = G.ioff[v + 1];
+        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
         uint32_t acc[WQ * 4];
 #pragma unroll
         for (int q = 0; q < WQ * 4; q++) acc[q] = 0;
@@ -874,7 +875,7 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
 
 // counters of one repetition (device)
 enum { C_CAND, C_MOVES, C_OVF, C_BAD, C_NH, C_BAD0, C_APPLIED, C_NV, C_HUB, C_CW, C_TOUCH, C_TTOUCH,
-       C_ACC,          // three 64-bit byte counters (even index: 8-byte aligned), see k_cut_flags
+       C_ACC,          // three 64-bit byte counters (even index: 8-byte aligned), see k_cut_bits
        C_N = C_ACC + 6 };
 
 // moves of at most SMALLM are validated by one CTA (k_val_small) with the
@@ -894,6 +895,7 @@ struct RepArrays {
     int32_t *cnt, *linked;
     int32_t *D0;
     long long *psize, *saving;
+    int32_t *cutn;   // cut hyperedges of every candidate node
     int32_t *pc;
     int32_t *pred, *succ, *chain, *mvpos;
     long long *cgain;
@@ -915,7 +917,10 @@ __global__ void k_rep_zero(RepArrays R, int keep) {
         }
         if (i <= R.nparts) R.pc[i] = 0;
         if (i < R.n) {
-            if (!keep) R.saving[i] = 0;
+            if (!keep) {
+                R.saving[i] = 0;
+                R.cutn[i] = 0;
+            }
             R.pred[i] = -1;
             R.succ[i] = -1;
             R.chain[i] = -1;
@@ -932,35 +937,63 @@ __global__ void k_rep_zero(RepArrays R, int keep) {
     }
 }
 
-__global__ void k_rep_nodes(const int32_t *rho, const int32_t *size, const int32_t *singin, int32_t n,
-                            long long *psize, int32_t *D0) {
+// |p| and the single-pin hyperedges' share of D(p).  Up to RN_PARTS parts are
+// summed per CTA first: a million nodes over a few hundred parts otherwise
+// queue on as many addresses.
+constexpr int32_t RN_PARTS = 2048;
+__global__ void __launch_bounds__(256) k_rep_nodes(const int32_t *rho, const int32_t *size, const int32_t *singin,
+                                                   int32_t n, int32_t nparts, long long *psize, int32_t *D0) {
     HP_KERNEL_ENTER();
+    __shared__ uint32_t s_size[RN_PARTS], s_d[RN_PARTS];   // sizes sum to the level-0 node count: 32 bits
+    if (nparts > RN_PARTS) {
+        GRID_STRIDE(v, (int64_t)n) {
+            const int32_t p = rho[v];
+            atomicAdd((unsigned long long *)&psize[p], (unsigned long long)size[v]);
+            if (singin[v]) atomicAdd(&D0[p], singin[v]);
+        }
+        return;
+    }
+    for (int32_t p = threadIdx.x; p < nparts; p += blockDim.x) s_size[p] = s_d[p] = 0;
+    __syncthreads();
     GRID_STRIDE(v, (int64_t)n) {
-        int32_t p = rho[v];
-        atomicAdd((unsigned long long *)&psize[p], (unsigned long long)size[v]);
-        if (singin[v]) atomicAdd(&D0[p], singin[v]);
+        const int32_t p = rho[v];
+        atomicAdd(&s_size[p], (uint32_t)size[v]);
+        if (singin[v]) atomicAdd(&s_d[p], (uint32_t)singin[v]);
+    }
+    __syncthreads();
+    for (int32_t p = threadIdx.x; p < nparts; p += blockDim.x) {
+        if (s_size[p]) atomicAdd((unsigned long long *)&psize[p], (unsigned long long)s_size[p]);
+        if (s_d[p]) atomicAdd(&D0[p], (int32_t)s_d[p]);
     }
 }
 
-// Cut incident hyperedges (|e| >= 2 and more than one part): the only ones
-// that add to conn(v, p) for p != rho(v).  Compacted per node, in incidence
-// order, for the gain kernels.
-// Also counts, for the step's algorithmic bytes, the pins-list entries of
-// the level (sum of lambda(e), once per hyperedge: at the entry of its first
-// pin), the cut incidence entries and the list entries the gain kernels walk
-// for them (sum of lambda(e) over cut entries), into acc[0..2].
-__global__ void k_cut_flags(const int32_t *off, const int32_t *pin, const int32_t *inc, const int32_t *inode,
-                            const int32_t *lam, int64_t np, int32_t *flag, unsigned long long *acc) {
+// Cut hyperedges (|e| >= 2 and more than one part), one bit each: the only
+// ones that add to conn(v, p) for p != rho(v).  Also counts, for the step's
+// algorithmic bytes, the pins-list entries of the level (sum of lambda(e)),
+// the cut incidence entries (sum of |e| over cut hyperedges) and the list
+// entries the gain kernels walk for them (sum of |e| lambda(e)), into acc[0..2].
+__global__ void k_cut_bits(const int32_t *off, const int32_t *lam, int32_t e, uint32_t *bits, unsigned long long *acc) {
     HP_KERNEL_ENTER();
+    const int lane = threadIdx.x & 31;
     unsigned long long lsum = 0, cuts = 0, clam = 0;
-    GRID_STRIDE(t, np) {
-        const int32_t e = inc[t];
-        const bool listed = off[e + 1] - off[e] >= 2;   // single-pin hyperedges have no pins list
-        const int32_t f = (listed && lam[e] >= 2) ? 1 : 0;
-        flag[t] = f;
-        if (listed && inode[t] == pin[off[e]]) lsum += (unsigned long long)lam[e];
-        cuts += (unsigned long long)f;
-        if (f) clam += (unsigned long long)lam[e];
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); base < e; base += step) {
+        const int64_t i = base + lane;
+        bool cut = false;
+        if (i < e) {
+            const int32_t sz = off[i + 1] - off[i];
+            if (sz >= 2) {   // single-pin hyperedges have no pins list
+                const int32_t l = lam[i];
+                cut = l >= 2;
+                lsum += (unsigned long long)l;
+                if (cut) {
+                    cuts += (unsigned long long)sz;
+                    clam += (unsigned long long)sz * (unsigned long long)l;
+                }
+            }
+        }
+        const uint32_t word = __ballot_sync(0xffffffffu, cut);
+        if (lane == 0) bits[base >> 5] = word;
     }
     // one update of each counter per CTA (all CTAs hit the same three words)
     __shared__ unsigned long long s_acc[3];
@@ -971,7 +1004,7 @@ __global__ void k_cut_flags(const int32_t *off, const int32_t *pin, const int32_
         cuts += __shfl_down_sync(0xffffffffu, cuts, o);
         clam += __shfl_down_sync(0xffffffffu, clam, o);
     }
-    if ((threadIdx.x & 31) == 0 && (lsum | cuts | clam)) {
+    if (lane == 0 && (lsum | cuts | clam)) {
         atomicAdd(&s_acc[0], lsum);
         atomicAdd(&s_acc[1], cuts);
         atomicAdd(&s_acc[2], clam);
@@ -979,24 +1012,52 @@ __global__ void k_cut_flags(const int32_t *off, const int32_t *pin, const int32_
     __syncthreads();
     if (threadIdx.x < 3 && s_acc[threadIdx.x]) atomicAdd(&acc[threadIdx.x], s_acc[threadIdx.x]);
 }
-__global__ void k_cut_fill(const int32_t *inc, const int32_t *flag, const int32_t *cpos, const int32_t *ioff,
-                           int64_t np, int32_t n, int32_t *cut, int32_t *cut_off) {
+// The cut hyperedges of every candidate (saving(v) > 0), gathered at the front
+// of v's own incidence segment (in no particular order: the gains are sums):
+// one pass over the incidence, a warp's entries of one node taking their
+// places by one atomic.  Bound by the reads of the incidence (8 B an entry, 4
+// where no node of a warp is a candidate).  Flagging, scanning and filling
+// lists of all nodes took 166 + 45 + 62 us a repetition on the 1M Gaussian net.
+__global__ void k_cut_lists(const int32_t *ioff, const int32_t *inc, const int32_t *inode, int64_t np,
+                            const long long *saving, const uint32_t *bits, int32_t *cut, int32_t *cutn) {
     HP_KERNEL_ENTER();
-    GRID_STRIDE(t, np) {
-        if (flag[t]) cut[cpos[t]] = inc[t];
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31u); base < np; base += step) {
+        const int64_t t = base + lane;
+        const int32_t v = t < np ? inode[t] : -1;
+        const bool cand = v >= 0 && saving[v] > 0;
+        if (!__any_sync(FULL, cand)) continue;
+        int32_t e = 0;
+        bool f = false;
+        if (cand) {
+            e = inc[t];
+            f = (bits[e >> 5] >> (e & 31)) & 1u;
+        }
+        // the lanes of v: from the last head up to this lane to the one before the next head
+        const int32_t pv = __shfl_up_sync(FULL, v, 1);
+        const unsigned heads = __ballot_sync(FULL, lane == 0 || pv != v), fm = __ballot_sync(FULL, f);
+        const unsigned upto = (2u << lane) - 1u;
+        const int first = 31 - __clz((int)(heads & upto));
+        const unsigned later = heads & ~upto;
+        const unsigned run = fm & ~((1u << first) - 1u) & (later ? (later & (0u - later)) - 1u : FULL);
+        int32_t at = 0;
+        if (lane == first && run) at = atomicAdd(&cutn[v], __popc(run));
+        at = __shfl_sync(FULL, at, first);
+        if (f) cut[ioff[v] + at + __popc(run & ((1u << lane) - 1u))] = e;
     }
-    GRID_STRIDE(v, (int64_t)n + 1) cut_off[v] = cpos[ioff[v]];
 }
 
 // candidates: nodes that can spare a cut, by number of cut hyperedges:
 // up to GW_DEG a warp each, up to HUB_DEG a CTA each, more a large CTA each
 constexpr int32_t HUB_DEG = 1024, GW_DEG = 256;
-__global__ void k_candidates(const long long *saving, const int32_t *cut_off, int32_t n, int32_t *list, int32_t *cnt,
+__global__ void k_candidates(const long long *saving, const int32_t *cutn, int32_t n, int32_t *list, int32_t *cnt,
                              int32_t *hubs, int32_t *hcnt, int32_t *wlist, int32_t *wcnt) {
     HP_KERNEL_ENTER();
     GRID_STRIDE(v, (int64_t)n) {
         if (saving[v] > 0) {
-            const int32_t d = cut_off[v + 1] - cut_off[v];
+            const int32_t d = cutn[v];
             if (d > HUB_DEG) hubs[atomicAdd(hcnt, 1)] = (int32_t)v;
             else if (d <= GW_DEG) wlist[atomicAdd(wcnt, 1)] = (int32_t)v;
             else list[atomicAdd(cnt, 1)] = (int32_t)v;
@@ -2286,7 +2347,8 @@ struct LevelWs {
     Plist PL;
     RepArrays R;
     int32_t *cl, *hubs, *cw;
-    int32_t *cflag, *cpos, *cut, *cut_off;   // cut incident hyperedges per node
+    uint32_t *cutbits;                       // a bit per cut hyperedge
+    int32_t *cut;                            // cut hyperedges of the candidates (k_cut_lists)
     int32_t *tiny, n_tiny;                   // hyperedges of 2..8 pins
     int32_t *mid, n_mid;                     // hyperedges of 9..small_max pins
     int32_t parts_used;                      // parts holding a node at the level's start
@@ -2383,10 +2445,9 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->cl = A.get<int32_t>(n);
     W->hubs = A.get<int32_t>(n);
     W->cw = A.get<int32_t>(n);
-    W->cflag = A.get<int32_t>(np);
-    W->cpos = A.get<int32_t>(np + 1);
+    W->cutbits = A.get<uint32_t>(e / 32 + 1);
     W->cut = A.get<int32_t>(np);
-    W->cut_off = A.get<int32_t>(n + 1);
+    R.cutn = A.get<int32_t>(n);
     W->tiny = A.get<int32_t>(e);
     W->mid = A.get<int32_t>(e);
     W->touched = A.get<int32_t>(e);
@@ -2469,7 +2530,7 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
     for (void *p : std::initializer_list<void *>{
              W->act, W->big, W->wns, W->singin, W->PL.p, W->PL.cnt, W->PL.cin, W->PL.lam, W->R.cnt, W->R.linked,
              W->R.D0, W->R.psize, W->R.saving, W->R.pc, W->R.pred, W->R.succ, W->R.chain, W->R.mvpos, W->R.cgain,
-             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cflag, W->cpos, W->cut, W->cut_off, W->tiny, W->mid, W->touched, W->ttouched, W->M.node, W->M.src, W->M.dst, W->M.gain,
+             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->ttouched, W->M.node, W->M.src, W->M.dst, W->M.gain,
              W->S.node, W->S.src, W->S.dst, W->S.gain, W->keys, W->idx, W->msz, W->mni, W->first, W->choice, W->accnode, W->pen,
              W->minpen, W->acc1, W->acc2, W->pos, W->clen, W->lens, W->starts, W->cstart, W->seqmove, W->heads, W->hkeys,
              W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
@@ -2592,7 +2653,9 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
     HP_LAUNCH_CHECK();
     if (!reuse) {
         W.bits_valid = false;
-        launch_k(k_rep_nodes, grid_of(n, 256), 256, 0, s, rho, L.size, W.singin, n, R.psize, R.D0);
+        // (a few CTAs an SM: each ends with a pass over the parts; the step call takes any sizes)
+        launch_k(k_rep_nodes, std::min(grid_of(n, 256), 4 * num_sms()), 256, 0, s, rho, L.size, W.singin, n, dbg ? RN_PARTS + 1 : nparts,
+                 R.psize, R.D0);
         HP_LAUNCH_CHECK();
         // pins(p,e), pins_in(p,e), D(p), saving(v)
         if (W.n_mid > 0) {
@@ -2626,19 +2689,18 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         }
         // moves in isolation (Eq. 13)
         if (L.np > 0) {
-            launch_k(k_cut_flags, grid_of(L.np, 256), 256, 0, s, L.off, L.pin, L.inc, L.inode, W.PL.lam, L.np, W.cflag,
+            launch_k(k_cut_bits, grid_of(L.e, 256), 256, 0, s, L.off, W.PL.lam, L.e, W.cutbits,
                      reinterpret_cast<unsigned long long *>(cnt + C_ACC));
             HP_LAUNCH_CHECK();
+            launch_k(k_cut_lists, grid_of(L.np, 256), 256, 0, s, L.ioff, L.inc, L.inode, L.np, R.saving, W.cutbits, W.cut,
+                     R.cutn);
+            HP_LAUNCH_CHECK();
         }
-        scan_excl(W.cflag, W.cpos, L.np, W.cpos + L.np, A);
-        launch_k(k_cut_fill, grid_of(std::max<int64_t>(L.np, (int64_t)n + 1), 256), 256, 0, s, L.inc, W.cflag, W.cpos, L.ioff,
-                 L.np, n, W.cut, W.cut_off);
-        HP_LAUNCH_CHECK();
     }
-    launch_k(k_candidates, grid_of(n, 256), 256, 0, s, R.saving, W.cut_off, n, W.cl, cnt + C_CAND, W.hubs, cnt + C_HUB,
+    launch_k(k_candidates, grid_of(n, 256), 256, 0, s, R.saving, R.cutn, n, W.cl, cnt + C_CAND, W.hubs, cnt + C_HUB,
              W.cw, cnt + C_CW);
     HP_LAUNCH_CHECK();
-    GainArgs G{L.off, W.cut_off, W.cut, w, rho, L.size, R.psize, R.saving, W.wns, W.PL, P.omega, second_half, W.M};
+    GainArgs G{L.off, L.ioff, R.cutn, W.cut, w, rho, L.size, R.psize, R.saving, W.wns, W.PL, P.omega, second_half, W.M};
     if (bits_pay(L, W)) {
         if (!reuse || !W.bits_valid) {
             launch_k(k_part_bits, grid_of((int64_t)L.e * 32, PB_T), PB_T, 0, s, L.off, W.PL, L.e, W.wq, W.bits);
