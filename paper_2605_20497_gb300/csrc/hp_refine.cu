@@ -2306,6 +2306,102 @@ __global__ void __launch_bounds__(IS_T) k_inseq_small(SeqSim Q, const int32_t *l
         if (sz > lo && sz <= emax) inseq_edge<32>(Q, e, lane, bk, bd, ord, tp, tc, tci, gc);
     }
 }
+// The same for up to PB_PARTS parts: the running counts of every part sit in
+// a table indexed by part (pins in the low half word, inbound pins in the high
+// one), loaded from the pins list.  The moves are taken 32 sequence ranks at a
+// time, a lane each: a lane's counts are the table's plus what the chunk's
+// earlier lanes change at its two parts (32 broadcasts); the table then takes
+// the chunk's changes.  Against counting over all earlier ranks from the list:
+// work c instead of c^2 / 2 a hyperedge with c moved pins, and no binary
+// searches.  A warp per hyperedge of lo < |e| <= emax <= 512 pins.
+__host__ __device__ inline size_t inseq_parts_smem(int32_t nparts, int32_t emax) {
+    return 4 * (size_t)(IS_T / 32) * (nparts + 2 * (size_t)emax + 1);
+}
+__global__ void __launch_bounds__(IS_T) k_inseq_parts(SeqSim Q, const int32_t *list, const int32_t *count_p,
+                                                      int32_t emax, int32_t nparts, const int32_t *mcount, int32_t lo) {
+    HP_KERNEL_ENTER();
+    if (*mcount == 0) return;
+    const int32_t count = *count_p;
+    extern __shared__ __align__(16) uint32_t smw[];
+    const unsigned FULL = 0xffffffffu;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    // running counts; moved pins (sequence position << 1 | destination pin) as found, then by rank
+    uint32_t *tab = smw + (size_t)wid * (nparts + 2 * emax + 1), *mv = tab + nparts, *srt = mv + emax;
+    for (int32_t p = lane; p < nparts; p += 32) tab[p] = 0;
+    __syncwarp();
+    const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t x = w0; x < count; x += nw) {
+        const int32_t e = list[x];
+        const int32_t a = Q.off[e], b = Q.off[e + 1], sz = b - a;
+        if (sz <= lo || sz > emax) continue;
+        const int32_t dst0 = a + Q.nsrc[e], lam = Q.PL.lam[e];
+        const long long we = Q.w[e];
+        int32_t c = 0;
+        for (int32_t j0 = a; j0 < b; j0 += 32) {
+            const int32_t j = j0 + lane;
+            const int32_t k = j < b ? Q.mvpos[Q.pin[j]] : -1;
+            const unsigned m = __ballot_sync(FULL, k >= 0);
+            if (k >= 0) mv[c + __popc(m & lt)] = ((uint32_t)k << 1) | (j >= dst0 ? 1u : 0u);
+            c += __popc(m);
+        }
+        if (c == 0) continue;
+        for (int32_t k = lane; k < lam; k += 32)
+            tab[Q.PL.p[a + k]] = (uint32_t)Q.PL.cnt[a + k] | ((uint32_t)Q.PL.cin[a + k] << 16);
+        __syncwarp();
+        for (int32_t i = lane; i < c; i += 32) {   // positions are distinct
+            const uint32_t k = mv[i];
+            int32_t r = 0;
+            for (int32_t t = 0; t < c; t++) r += mv[t] < k;
+            srt[r] = k;
+        }
+        __syncwarp();
+        for (int32_t r0 = 0; r0 < c; r0 += 32) {
+            const bool on = r0 + lane < c;
+            const int n = min(32, c - r0);
+            int32_t k = 0, ps = -1, pd = -1;
+            uint32_t dv = 0, cs = 0, cd = 0;
+            if (on) {
+                const uint32_t y = srt[r0 + lane];
+                k = (int32_t)(y >> 1);
+                dv = (y & 1u) ? 0x10001u : 1u;
+                const int32_t mi = Q.seqmove[k];
+                ps = Q.src[mi];
+                pd = Q.dst[mi];
+                cs = tab[ps];
+                cd = tab[pd];
+            }
+            __syncwarp();
+            for (int t = 0; t + 1 < n; t++) {
+                const int32_t xs = __shfl_sync(FULL, ps, t), xd = __shfl_sync(FULL, pd, t);
+                const uint32_t xv = __shfl_sync(FULL, dv, t);
+                if (lane > t) {
+                    if (xd == ps) cs += xv;
+                    if (xs == ps) cs -= xv;
+                    if (xd == pd) cd += xv;
+                    if (xs == pd) cd -= xv;
+                }
+            }
+            if (on) {
+                long long g = 0;
+                if ((cs & 0xffffu) == 1u) g += we;
+                if ((cd & 0xffffu) == 0u) g -= we;
+                if (g) atomicAdd(&Q.gseq[k], (unsigned long long)g);
+                if (dv >> 16) {
+                    if ((cs >> 16) == 1u) atomicAdd(&Q.dDs[k], -1);
+                    if ((cd >> 16) == 0u) atomicAdd(&Q.dDd[k], 1);
+                }
+                atomicAdd(&tab[ps], 0u - dv);
+                atomicAdd(&tab[pd], dv);
+            }
+            __syncwarp();
+        }
+        // clean the table: the list's parts and the parts moved to
+        for (int32_t k = lane; k < lam; k += 32) tab[Q.PL.p[a + k]] = 0;
+        for (int32_t i = lane; i < c; i += 32) tab[Q.dst[Q.seqmove[srt[i] >> 1]]] = 0;
+        __syncwarp();
+    }
+}
 __global__ void __launch_bounds__(256) k_inseq_big(SeqSim Q, const int32_t *list, int32_t count, int32_t emax,
                                                    int32_t *gbuf, const int32_t *mcount) {
     HP_KERNEL_ENTER();
@@ -3006,6 +3102,15 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         launch_k(k_inseq_tiny, grid_of(W.n_act, IST_T), IST_T, 0, s, Z, W.ttouched, cnt + C_TTOUCH, cnt + C_MOVES);
         HP_LAUNCH_CHECK();
         auto inseq_mid = [&](int32_t lo, int32_t emax) {
+            if (nparts <= PB_PARTS) {
+                const size_t sm = inseq_parts_smem(nparts, emax);
+                const int occ = prepare_kernel((const void *)k_inseq_parts, IS_T, sm);
+                const int grid = (int)std::min<int64_t>(cdiv(W.n_act, IS_T / 32), (int64_t)num_sms() * occ);
+                launch_k(k_inseq_parts, std::max(grid, 1), IS_T, sm, s, Z, W.touched, cnt + C_TOUCH, emax, nparts,
+                         cnt + C_MOVES, lo);
+                HP_LAUNCH_CHECK();
+                return;
+            }
             size_t sm = (size_t)(9 * emax + 1) * 4 * (IS_T / 32);
             int occ = prepare_kernel((const void *)k_inseq_small, IS_T, sm);
             int grid = (int)std::min<int64_t>(cdiv(W.n_act, IS_T / 32), (int64_t)num_sms() * occ);
