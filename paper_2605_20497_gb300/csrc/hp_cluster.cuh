@@ -103,7 +103,10 @@ template <class K> __host__ __device__ constexpr int sq_chunk() {
     return (int)(SQ_SMEM / (2 * sizeof(K) + 3 * sizeof(uint32_t))) / 32 * 32;
 }
 template <class K> __host__ __device__ constexpr int sq_max() { return SQ_CS * sq_chunk<K>(); }
-constexpr int SQ_RANK_MAX = 256;                // up to this many items one CTA ranks them directly
+// items are ranked directly where n^2 <= passes << SQ_RANK_LOG (1,448 at four
+// passes): a ranking compares n^2 pairs on eight SMs, about 4.5 us at 1,448
+// items, a radix pass takes 3.3 us whatever the size
+constexpr int SQ_RANK_LOG = 19;
 
 // the sort buffers of key type K in the dynamic shared memory
 template <class K> struct SqBuf {
@@ -124,7 +127,7 @@ template <class K> struct SqBuf {
 // ranks its items by digit (stable: warp-major, slot-major, lane-minor, as
 // the items lie in global order), publishes its per-digit counts, reads the
 // other CTAs' counts, and writes each item into the shared-memory buffer of
-// the CTA that holds its destination position.
+// the CTA that holds its destination position.  Few items are ranked directly.
 template <class K>
 __device__ __forceinline__ void cluster_radix_sort(cg::cluster_group &cl, K *keys, uint32_t *vals, int32_t n,
                                                    int passes, SqBuf<K> B, uint32_t *s_wc, uint32_t *s_tot,
@@ -133,23 +136,23 @@ __device__ __forceinline__ void cluster_radix_sort(cg::cluster_group &cl, K *key
     uint32_t *va = B.va, *vb = B.vb, *rk = B.rk;
     if (n <= 1 || passes <= 0) return;   // uniform over the cluster
     const int r = (int)cl.block_rank(), t = threadIdx.x, T = blockDim.x, lane = t & 31, w = t >> 5;
-    if (n <= SQ_RANK_MAX) {
-        // few items: CTA 0 ranks them directly (stable: ties by position) on
-        // the sorted bits, the other CTAs wait at the barrier
-        if (r == 0) {
-            const K mask = 8 * passes >= (int)(8 * sizeof(K)) ? ~K(0) : ((K(1) << (8 * passes)) - 1);
-            for (int32_t i = t; i < n; i += T) {
-                ka[i] = keys[i];
-                va[i] = vals[i];
+    if ((int64_t)n * n <= (int64_t)passes << SQ_RANK_LOG) {
+        // few items: every CTA reads them all and ranks its share directly, a
+        // warp per item (stable: ties by position), on the sorted bits
+        const K mask = 8 * passes >= (int)(8 * sizeof(K)) ? ~K(0) : ((K(1) << (8 * passes)) - 1);
+        for (int32_t i = t; i < n; i += T) ka[i] = keys[i];
+        const int32_t share = (n + SQ_CS - 1) / SQ_CS, lo = min(n, r * share), hi = min(n, lo + share);
+        for (int32_t i = lo + t; i < hi; i += T) va[i] = vals[i];
+        cl.sync();   // read by every CTA before any item moves
+        for (int32_t i = lo + w; i < hi; i += T >> 5) {
+            const K ki = ka[i] & mask;
+            uint32_t rank = 0;
+            for (int32_t j = lane; j < n; j += 32) {
+                const K kj = ka[j] & mask;
+                rank += (kj < ki || (kj == ki && j < i)) ? 1u : 0u;
             }
-            __syncthreads();
-            for (int32_t i = t; i < n; i += T) {
-                const K ki = ka[i] & mask;
-                int32_t rank = 0;
-                for (int32_t j = 0; j < n; j++) {
-                    const K kj = ka[j] & mask;
-                    rank += (kj < ki || (kj == ki && j < i)) ? 1 : 0;
-                }
+            rank = __reduce_add_sync(0xffffffffu, rank);
+            if (lane == 0) {
                 keys[rank] = ka[i];
                 vals[rank] = va[i];
             }

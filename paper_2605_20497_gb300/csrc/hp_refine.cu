@@ -1840,6 +1840,109 @@ __device__ void ph_first_of(const int32_t *src, int32_t m, int32_t nparts, int32
     }
 }
 
+// The chaining rounds of at most CHAIN_SMEM_M moves by one cluster (packed
+// acceptance).  Every CTA keeps a copy of what the window scans read: gain,
+// size and |in| of each move, and a bit per move with a predecessor, to which
+// each round adds the moves chosen in the one before; a thread keeps its own
+// moves' state in registers, so a round reads nothing but the previous
+// round's slots: one trip to L2, the scans, one cluster barrier.  Keeping that
+// state in global memory cost four dependent trips a round (8.6 us a round of
+// 1,800 moves on the 262k layered net; 6.2 this way).
+__device__ __forceinline__ void chain_rounds_smem(const ChainCtx &C, const Moves &S, int rounds, int32_t m,
+                                                  cg::cluster_group &cl, unsigned char *smem, uint32_t *s_taken) {
+    constexpr int NS = (CHAIN_SMEM_M + SQ_CS * SQ_T - 1) / (SQ_CS * SQ_T);   // moves a thread owns
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int gw = (int)cl.block_rank() * (SQ_T / 32) + wid, nw = SQ_CS * (SQ_T / 32);
+    long long *c_gain = reinterpret_cast<long long *>(smem);
+    int2 *c_sn = reinterpret_cast<int2 *>(c_gain + CHAIN_SMEM_M);
+    for (int32_t j = threadIdx.x; j < m; j += SQ_T) {
+        c_gain[j] = S.gain[j];
+        c_sn[j] = make_int2(C.msz[j], C.mni[j]);
+    }
+    for (int32_t x = threadIdx.x; x < (m + 31) / 32; x += SQ_T) s_taken[x] = 0;
+    // the free ends are dealt to the warps a lane at a time (a warp of few
+    // moves otherwise scans for 32 of them one after another)
+    int32_t j0[NS], jend[NS], vi[NS], choice[NS];
+    uint32_t pen[NS];
+    bool free_end[NS];
+#pragma unroll
+    for (int q = 0; q < NS; q++) {
+        const int32_t i = q * (32 * nw) + lane * nw + gw;
+        j0[q] = jend[q] = vi[q] = 0;
+        choice[q] = -1;
+        pen[q] = 0;
+        free_end[q] = i < m;
+        if (i < m) {
+            const int32_t d = S.dst[i];
+            j0[q] = C.first[d];
+            jend[q] = C.first[d + 1];
+            vi[q] = S.node[i];
+        }
+    }
+    __syncthreads();
+    // links the winners of the round whose slots are acc
+    auto link = [&](const unsigned long long *acc) {
+#pragma unroll
+        for (int q = 0; q < NS; q++) {
+            const int32_t i = q * (32 * nw) + lane * nw + gw, j = choice[q];
+            if (j >= 0 && acc[j] == chain_key(pen[q], vi[q])) {
+                C.pred[j] = i;
+                C.succ[i] = j;
+                free_end[q] = false;
+            }
+        }
+    };
+    int rr = 0;
+    for (; rr < rounds; rr++) {
+        unsigned long long *accr = C.acc[rr % 3], *accp = C.acc[(rr + 2) % 3], *accn = C.acc[(rr + 1) % 3];
+        if (rr > 0) {
+            const int32_t go = *(volatile int32_t *)&C.linked[rr - 1];
+            for (int32_t x = wid; x < (m + 31) / 32; x += SQ_T / 32) {
+                const int32_t j = 32 * x + lane;
+                const unsigned b = __ballot_sync(FULL, j < m && accp[j] != 0ull);
+                if (lane == 0) s_taken[x] |= b;
+            }
+            if (!go) break;   // the same for the whole cluster
+            link(accp);
+            __syncthreads();
+        }
+        bool any = false;
+#pragma unroll
+        for (int q = 0; q < NS; q++) {
+            const int32_t i = q * (32 * nw) + lane * nw + gw;
+            if (i < m) accn[i] = 0;
+            choice[q] = -1;
+            int2 sn = make_int2(0, 0);
+            if (i < m) sn = c_sn[i];
+            unsigned todo = __ballot_sync(FULL, free_end[q] && j0[q] < jend[q]);
+            while (todo) {
+                const int l = __ffs(todo) - 1;
+                todo &= todo - 1;
+                uint32_t p = 0;
+                const int32_t x = warp_pick(__shfl_sync(FULL, i, l), __shfl_sync(FULL, j0[q], l),
+                                            __shfl_sync(FULL, jend[q], l), C.window, __shfl_sync(FULL, sn.x, l),
+                                            __shfl_sync(FULL, sn.y, l),
+                                            [&](int32_t j) { return (s_taken[j >> 5] >> (j & 31)) & 1u; },
+                                            [&](int32_t j) { return c_gain[j]; }, [&](int32_t j) { return c_sn[j]; }, p);
+                if (lane == l) {
+                    choice[q] = x;
+                    pen[q] = p;
+                }
+            }
+            if (choice[q] >= 0) {
+                atomicMax(&accr[choice[q]], chain_key(pen[q], vi[q]));
+                any = true;
+            }
+        }
+        if (__any_sync(FULL, any) && lane == 0) C.linked[rr] = 1;
+        cl.sync();
+    }
+    // the links of the last round run (rounds cut off by the limit)
+    if (rr == rounds && rounds > 0) link(C.acc[(rounds - 1) % 3]);
+    cl.sync();
+}
+
 __global__ void __cluster_dims__(SQ_CS, 1, 1) __launch_bounds__(SEQ_T) k_seq_cluster(ClusterSeqArgs A) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) unsigned char smem[];
@@ -1891,60 +1994,36 @@ __global__ void __cluster_dims__(SQ_CS, 1, 1) __launch_bounds__(SEQ_T) k_seq_clu
     cl.sync();
     ph_first_of(A.S.src, m, A.nparts, A.first, t0, nt);
     cl.sync();
-    // chaining rounds (Sec. VI-C).  Up to CHAIN_SMEM_M moves, every CTA keeps
-    // a copy of what the window scans read: gain, size and |in| of each move,
-    // and a bit per move with a predecessor, to which each round adds the
-    // moves chosen in the one before.
-    const bool in_smem = A.packed && m <= CHAIN_SMEM_M;
-    long long *c_gain = reinterpret_cast<long long *>(smem);
-    int2 *c_sn = reinterpret_cast<int2 *>(c_gain + CHAIN_SMEM_M);
-    uint32_t *c_taken = s_wc;
-    if (in_smem) {
-        for (int32_t j = threadIdx.x; j < m; j += blockDim.x) {
-            c_gain[j] = A.S.gain[j];
-            c_sn[j] = make_int2(A.C.msz[j], A.C.mni[j]);
-        }
-        for (int32_t x = threadIdx.x; x < (m + 31) / 32; x += blockDim.x) c_taken[x] = 0;
-        __syncthreads();
-    }
+    // chaining rounds (Sec. VI-C)
     const int gw = (int)(t0 >> 5), nwarps = (int)(nt >> 5);
-    for (int rr = 0; rr < A.rounds; rr++) {
-        if (rr > 0 && !*(volatile int32_t *)&A.C.linked[rr - 1]) break;
-        if (A.packed) {
+    if (A.packed && m <= CHAIN_SMEM_M) {
+        chain_rounds_smem(A.C, A.S, A.rounds, m, cl, smem, s_wc);
+    } else if (A.packed) {
+        for (int rr = 0; rr < A.rounds; rr++) {
+            if (rr > 0 && !*(volatile int32_t *)&A.C.linked[rr - 1]) break;
             const unsigned long long *accp = A.C.acc[(rr + 2) % 3];
-            if (in_smem) {
-                if (rr > 0) {
-                    for (int32_t x = threadIdx.x >> 5; x < (m + 31) / 32; x += blockDim.x >> 5) {
-                        const int32_t j = 32 * x + (threadIdx.x & 31);
-                        const unsigned b = __ballot_sync(0xffffffffu, j < m && accp[j] != 0ull);
-                        if ((threadIdx.x & 31) == 0) c_taken[x] |= b;
-                    }
-                    __syncthreads();
-                }
-                ph_round(A.C, rr, m, gw, nwarps,
-                         [&](int32_t j) { return (c_taken[j >> 5] >> (j & 31)) & 1u; },
-                         [&](int32_t j) { return c_gain[j]; }, [&](int32_t j) { return c_sn[j]; });
-            } else {
-                ph_round(A.C, rr, m, gw, nwarps,
-                         [&](int32_t j) { return A.C.pred[j] >= 0 || (rr > 0 && accp[j] != 0ull); },
-                         [&](int32_t j) { return A.S.gain[j]; },
-                         [&](int32_t j) { return make_int2(A.C.msz[j], A.C.mni[j]); });
-            }
+            ph_round(A.C, rr, m, gw, nwarps,
+                     [&](int32_t j) { return A.C.pred[j] >= 0 || (rr > 0 && accp[j] != 0ull); },
+                     [&](int32_t j) { return A.S.gain[j]; },
+                     [&](int32_t j) { return make_int2(A.C.msz[j], A.C.mni[j]); });
             cl.sync();
-            continue;
         }
-        ph_choose(A.C, m, t0, nt);
-        cl.sync();
-        ph_accept_min(A.C, m, t0, nt);
-        cl.sync();
-        ph_accept_id(A.C, m, t0, nt);
-        cl.sync();
-        ph_link(A.C, rr, 0, m, t0, nt);
-        cl.sync();
-    }
-    if (A.packed && A.rounds > 0 && *(volatile int32_t *)&A.C.linked[A.rounds - 1]) {
-        ph_link_last(A.C, A.rounds - 1, m, t0, nt);
-        cl.sync();
+        if (A.rounds > 0 && *(volatile int32_t *)&A.C.linked[A.rounds - 1]) {
+            ph_link_last(A.C, A.rounds - 1, m, t0, nt);
+            cl.sync();
+        }
+    } else {
+        for (int rr = 0; rr < A.rounds; rr++) {
+            if (rr > 0 && !*(volatile int32_t *)&A.C.linked[rr - 1]) break;
+            ph_choose(A.C, m, t0, nt);
+            cl.sync();
+            ph_accept_min(A.C, m, t0, nt);
+            cl.sync();
+            ph_accept_id(A.C, m, t0, nt);
+            cl.sync();
+            ph_link(A.C, rr, 0, m, t0, nt);
+            cl.sync();
+        }
     }
     // chains, ordered by (total gain desc, head node asc)
     ph_path_heads(A.Q, m, t0, nt);
