@@ -92,32 +92,12 @@ __device__ __forceinline__ bool size_ok(const PropCtx &C, int32_t slack, int32_t
     return !C.size_filter || C.size[m] <= slack;
 }
 
-// ---------------------------------------------------------------- per-level weights
-__global__ void k_level_q(const int32_t *off, const int32_t *w, int32_t e, uint64_t *q, unsigned long long *sum) {
-    HP_KERNEL_ENTER();
-    __shared__ unsigned long long s;
-    if (threadIdx.x == 0) s = 0;
-    __syncthreads();
-    unsigned long long loc = 0;
-    GRID_STRIDE(i, (int64_t)e) {
-        // floor(w 2^24 / |e|): the numerator is below 2^41 and the divisor
-        // below 2^31, so the correctly rounded double quotient of a
-        // non-integer ratio is never rounded across an integer
-        const double num = (double)((uint64_t)w[i] << 24), den = (double)(off[i + 1] - off[i]);
-        const uint64_t qi = (uint64_t)floor(num / den);
-        q[i] = qi;
-        loc += qi;
-    }
-    for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s, loc);
-    __syncthreads();
-    if (threadIdx.x == 0) atomicAdd(sum, s);
-}
-
+// ---------------------------------------------------------------- per-level sums
 // the level's counters, node sums and tier counts start at zero (one launch
 // instead of four memsets, which would each end the overlap of a launch with
 // its predecessor)
-__global__ void k_level_start(LevelBox *box, long long *nsum, long long *vis, int32_t n, int32_t *cnt) {
+// (mate, where given: nobody is paired yet)
+__global__ void k_level_start(LevelBox *box, long long *nsum, long long *vis, int32_t n, int32_t *cnt, int32_t *mate) {
     HP_KERNEL_ENTER();
     const int64_t t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (t0 < (int64_t)(sizeof(LevelBox) / sizeof(uint32_t))) reinterpret_cast<uint32_t *>(box)[t0] = 0u;
@@ -125,27 +105,42 @@ __global__ void k_level_start(LevelBox *box, long long *nsum, long long *vis, in
     GRID_STRIDE(v, (int64_t)n) {
         nsum[v] = 0;
         vis[v] = 0;
+        if (mate) mate[v] = -1;
     }
 }
 
-// per incidence entry (e, v): sums over I(v) of |e| - 1 (bound on |N(v)|)
-// and |e| (pins the traversal of v visits), reduced per run of equal v
-// inside a warp, so hub nodes with huge incidence lists spread over threads
-__global__ void k_node_sums(const int32_t *off, const int32_t *inc, const int32_t *inode, int64_t np,
-                            long long *nsum, long long *vis, unsigned long long *visits) {
+// q(e) and their sum; and per incidence entry (e, v) the sums over I(v) of
+// |e| - 1 (bound on |N(v)|) and |e| (pins the traversal of v visits), reduced
+// per run of equal v inside a warp, so hub nodes with huge incidence lists
+// spread over threads
+__global__ void k_level_sums(const int32_t *off, const int32_t *w, int32_t e, uint64_t *q, unsigned long long *qsum,
+                             const int32_t *inc, const int32_t *inode, int64_t np, long long *nsum, long long *vis,
+                             unsigned long long *visits) {
     HP_KERNEL_ENTER();
+    __shared__ unsigned long long s[2];
+    if (threadIdx.x < 2) s[threadIdx.x] = 0;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
+    unsigned long long qloc = 0, loc = 0;
+    GRID_STRIDE(i, (int64_t)e) {
+        // floor(w 2^24 / |e|): the numerator is below 2^41 and the divisor
+        // below 2^31, so the correctly rounded double quotient of a
+        // non-integer ratio is never rounded across an integer
+        const double num = (double)((uint64_t)w[i] << 24), den = (double)(off[i + 1] - off[i]);
+        const uint64_t qi = (uint64_t)floor(num / den);
+        q[i] = qi;
+        qloc += qi;
+    }
     const int64_t wbase = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) << 5;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long loc = 0;
     for (int64_t base = wbase; base < np; base += stride) {
         const int64_t t = base + lane;
         const bool valid = t < np;
         const int32_t v = valid ? inode[t] : -1 - lane;
         long long sz = 0;
         if (valid) {
-            const int32_t e = inc[t];
-            sz = off[e + 1] - off[e];
+            const int32_t x = inc[t];
+            sz = off[x + 1] - off[x];
             loc += (unsigned long long)sz;
         }
         long long a = valid ? sz - 1 : 0, b = sz;
@@ -156,24 +151,18 @@ __global__ void k_node_sums(const int32_t *off, const int32_t *inc, const int32_
             atomicAdd((unsigned long long *)&vis[v], (unsigned long long)b);
         }
     }
-    for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
-    if (lane == 0) atomicAdd(visits, loc);
-}
-
-__global__ void k_node_bounds(const long long *nsum, int32_t n, int32_t *bound, LevelBox *box, int32_t e,
-                              int32_t permille) {
-    HP_KERNEL_ENTER();
-    // the noise cap of the level from the sum of q (complete: k_level_q ran before)
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        box->cap = e > 0 ? (uint64_t)((box->qsum / (unsigned long long)e) * (unsigned long long)permille / 1000ull)
-                         : 0ull;
-        box->cap_inv = ~0ull / (box->cap + 1);
+    for (int o = 16; o > 0; o >>= 1) {
+        qloc += __shfl_down_sync(0xffffffffu, qloc, o);
+        loc += __shfl_down_sync(0xffffffffu, loc, o);
     }
-    GRID_STRIDE(v, (int64_t)n) {
-        long long b = bound[v];
-        if (nsum[v] < b) b = nsum[v];
-        if (n - 1 < b) b = n - 1;
-        bound[v] = (int32_t)b;
+    if (lane == 0) {
+        if (qloc) atomicAdd(&s[0], qloc);
+        if (loc) atomicAdd(&s[1], loc);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s[0]) atomicAdd(qsum, s[0]);
+        if (s[1]) atomicAdd(visits, s[1]);
     }
 }
 
@@ -964,12 +953,22 @@ struct TierRule {
     int32_t dense_bound, deg_narrow;
     long long warp_visits, hub_visits;
 };
-__global__ void k_tiers(const int32_t *bound, const long long *vis, const int32_t *ioff, int32_t n, TierRule R,
+// First the bound on |N(v)| (its old value, the sum over I(v), the level's
+// other nodes) and the level's noise cap, from the sum of q.
+__global__ void k_tiers(int32_t *bound, const long long *nsum, LevelBox *box, int32_t e, int32_t permille,
+                        const long long *vis, const int32_t *ioff, int32_t n, TierRule R,
                         int32_t *lW, int32_t *lB, int32_t *lH, int32_t *lD, int32_t *lDH, int32_t *cnt, int32_t pi,
                         int32_t *cand, uint64_t *cscore) {
     HP_KERNEL_ENTER();
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        box->cap = e > 0 ? (uint64_t)((box->qsum / (unsigned long long)e) * (unsigned long long)permille / 1000ull)
+                         : 0ull;
+        box->cap_inv = ~0ull / (box->cap + 1);
+    }
     GRID_STRIDE(v, (int64_t)n) {
-        if (bound[v] == 0) {
+        const int32_t bv = (int32_t)min(min((long long)bound[v], nsum[v]), (long long)(n - 1));
+        bound[v] = bv;
+        if (bv == 0) {
             // no (size-valid) neighbour: an empty candidate list, no walk
             for (int32_t r = 0; r < pi; r++) {
                 cand[v * (int64_t)pi + r] = -1;
@@ -979,8 +978,8 @@ __global__ void k_tiers(const int32_t *bound, const long long *vis, const int32_
         }
         const int32_t deg = ioff[v + 1] - ioff[v];
         const bool wide = deg > R.deg_narrow, hub = vis[v] > R.hub_visits || deg > HUB_INCIDENCE || wide;
-        if ((uint32_t)bound[v] <= R.warp_limit && vis[v] <= R.warp_visits && !wide) lW[atomicAdd(&cnt[0], 1)] = (int32_t)v;
-        else if (bound[v] > R.dense_bound) {
+        if ((uint32_t)bv <= R.warp_limit && vis[v] <= R.warp_visits && !wide) lW[atomicAdd(&cnt[0], 1)] = (int32_t)v;
+        else if (bv > R.dense_bound) {
             if (hub) lDH[atomicAdd(&cnt[7], 1)] = (int32_t)v;
             else lD[atomicAdd(&cnt[6], 1)] = (int32_t)v;
         } else if (hub) lH[atomicAdd(&cnt[5], 1)] = (int32_t)v;
@@ -1039,7 +1038,7 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
         R.dense_bound = 0;
         R.hub_visits = HUB_VISITS_FEW;
     }
-    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.vis, L.ioff, C.n, R, W.lW, W.lB, W.lH, W.lD, W.lDH, W.cnt,
+    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.nsum, W.box, L.e, P.o.noise_permille, W.vis, L.ioff, C.n, R, W.lW, W.lB, W.lH, W.lD, W.lDH, W.cnt,
              C.pi, C.cand, C.cscore);
     HP_LAUNCH_CHECK();
     // the tiers take disjoint node lists, so they run side by side: the warp
@@ -1415,6 +1414,7 @@ struct MatchArgs {
     int32_t *target, *ccount;   // the writable views of D's arrays
     uint64_t *score;
     DpCtx D;
+    const int32_t *nbcnt, *bad;   // neighbours of every node (summed into the box); nodes no table held
 };
 __global__ void __cluster_dims__(SQ_CS, 1, 1) __launch_bounds__(SQ_T) k_match_cluster(MatchArgs A) {
     HP_KERNEL_ENTER();
@@ -1428,6 +1428,13 @@ __global__ void __cluster_dims__(SQ_CS, 1, 1) __launch_bounds__(SQ_T) k_match_cl
     const int64_t t0 = (int64_t)cl.block_rank() * blockDim.x + threadIdx.x, nt = (int64_t)SQ_CS * blockDim.x;
     const SqBuf<uint32_t> B(smem);
     const int32_t n = A.n;
+    {
+        unsigned long long loc = 0;
+        CSTRIDE(v, n, t0, nt) loc += (unsigned long long)A.nbcnt[v];
+        for (int o = 16; o > 0; o >>= 1) loc += __shfl_down_sync(0xffffffffu, loc, o);
+        if ((threadIdx.x & 31) == 0 && loc) atomicAdd(&A.box->nbrs, loc);
+        if (t0 == 0 && *A.bad) atomicOr(A.D.err, E_INTERNAL);
+    }
     // best-effort pairing (Sec. V-C): nodes with no valid neighbour, by (size, id)
     ph_iso_flags(A.candK, A.K, n, A.flag, t0, nt);
     cl.sync();
@@ -1618,26 +1625,21 @@ static void dst_groups(const Level &L, int32_t *canon, int32_t *canon_on, LevelB
 
 // The top-K valid neighbours by (eta, id) of every node of the level into
 // W.cand / W.cscore (Sec. V-C, Eq. 5-6), and the level's counters into the
-// box.  The level must have at least one node.
+// box; mate (where given) is set to -1.  The level must have at least one node.
 static void propose_lists(Level &L, int32_t level, const int32_t *w, const Params &P, int32_t K, CoarsenWs &W,
-                          Arena &A, cudaEvent_t *prop_events) {
+                          Arena &A, cudaEvent_t *prop_events, int32_t *mate) {
     cudaStream_t s = A.stream();
     const int32_t n = L.n;
     LevelBox *box = W.box;
     static_assert(sizeof(LevelBox) % sizeof(uint32_t) == 0 && sizeof(LevelBox) / sizeof(uint32_t) <= 256,
                   "the level box is zeroed by the first block of k_level_start");
-    launch_k(k_level_start, grid_of(std::max<int64_t>(n, 256), 256), 256, 0, s, box, W.nsum, W.vis, n, W.cnt);
+    launch_k(k_level_start, grid_of(std::max<int64_t>(n, 256), 256), 256, 0, s, box, W.nsum, W.vis, n, W.cnt, mate);
     HP_LAUNCH_CHECK();
     if (L.e > 0) {
-        launch_k(k_level_q, grid_of(L.e, 256), 256, 0, s, L.off, w, L.e, W.q, &box->qsum);
+        launch_k(k_level_sums, grid_of(std::max<int64_t>(L.e, L.np), 256), 256, 0, s, L.off, w, L.e, W.q, &box->qsum, L.inc,
+                 L.inode, L.np, W.nsum, W.vis, &box->visits);
         HP_LAUNCH_CHECK();
     }
-    if (L.np > 0) {
-        launch_k(k_node_sums, grid_of(L.np, 256), 256, 0, s, L.off, L.inc, L.inode, L.np, W.nsum, W.vis, &box->visits);
-        HP_LAUNCH_CHECK();
-    }
-    launch_k(k_node_bounds, grid_of(n, 256), 256, 0, s, W.nsum, n, L.nbnd, box, L.e, P.o.noise_permille);
-    HP_LAUNCH_CHECK();
     PropCtx C;
     C.n = n;
     C.pi = K;
@@ -1713,7 +1715,7 @@ void level_features(Level &L, const int32_t *w, const Params &P, CoarsenWs &W, A
     cudaStream_t s = A.stream();
     const int32_t K = P.o.learned_k;
     if (L.n == 0) return;
-    propose_lists(L, 0, w, P, K, W, A, nullptr);
+    propose_lists(L, 0, w, P, K, W, A, nullptr, nullptr);
     launch_k(k_flag_if_nonzero, 1, 1, 0, s, W.cnt + 4, err_dev);
     HP_LAUNCH_CHECK();
     LearnIn X = learn_in(L, 0, P, K, W);
@@ -1730,12 +1732,11 @@ void coarsen_level(Level &L, int32_t level, const int32_t *w, const Params &P, i
     const bool learned = P.o.learned_k > 0 && (P.o.learned_levels == 0 || level < P.o.learned_levels);
     const int32_t K = learned ? P.o.learned_k : pi;   // length of the proposal's lists
     LevelBox *box = W.box;
-    fill_i32(mate, n, -1, s);
     if (n == 0) {
         HPC(cudaMemsetAsync(box, 0, sizeof(LevelBox), s));
         return;
     }
-    propose_lists(L, level, w, P, K, W, A, prop_events);
+    propose_lists(L, level, w, P, K, W, A, prop_events, mate);
     // C(n) and its matching weights
     int32_t *cand = W.cand;
     uint64_t *cscore = W.cscore;
@@ -1746,10 +1747,6 @@ void coarsen_level(Level &L, int32_t level, const int32_t *w, const Params &P, i
         learned_candidates(X, P.o.node_batch, s);
     }
     if (prop_events) HPC(cudaEventRecord(prop_events[1], s));
-    launch_k(k_flag_if_nonzero, 1, 1, 0, s, W.cnt + 4, err_dev);
-    HP_LAUNCH_CHECK();
-    launch_k(k_sum_i32, grid_of(n, 256), 256, 0, s, L.nbnd, n, &box->nbrs);
-    HP_LAUNCH_CHECK();
     if (cand_out) {
         HPC(cudaMemcpyAsync(cand_out, cand, sizeof(int32_t) * n * pi, cudaMemcpyDeviceToDevice, s));
         HPC(cudaMemcpyAsync(score_out, cscore, sizeof(uint64_t) * n * pi, cudaMemcpyDeviceToDevice, s));
@@ -1772,13 +1769,17 @@ void coarsen_level(Level &L, int32_t level, const int32_t *w, const Params &P, i
     if (n <= sq_max<uint32_t>()) {
         // small level: pairing and matching by one cluster, one launch
         MatchArgs M{W.cand, K, cand, cscore, pi, n, P.omega, P.delta, L.size, L.nin, W.flag, W.pos, W.ikeys, W.iids,
-                    bits_for((uint64_t)P.omega), mate, box, W.target, W.ccount, W.score, D};
+                    bits_for((uint64_t)P.omega), mate, box, W.target, W.ccount, W.score, D, L.nbnd, W.cnt + 4};
         prepare_kernel((const void *)k_match_cluster, SQ_T, SQ_SMEM);
         launch_k(k_match_cluster, SQ_CS, SQ_T, SQ_SMEM, s, M);
         HP_LAUNCH_CHECK();
         return;
     }
 
+    launch_k(k_flag_if_nonzero, 1, 1, 0, s, W.cnt + 4, err_dev);
+    HP_LAUNCH_CHECK();
+    launch_k(k_sum_i32, grid_of(n, 256), 256, 0, s, L.nbnd, n, &box->nbrs);
+    HP_LAUNCH_CHECK();
     // best-effort pairing of nodes with no valid neighbour (Sec. V-C)
     launch_k(k_iso_flags, grid_of(n, 256), 256, 0, s, W.cand, K, n, W.flag);
     HP_LAUNCH_CHECK();

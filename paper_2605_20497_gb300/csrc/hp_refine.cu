@@ -812,28 +812,91 @@ __global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 
 }
 
 // ---------------------------------------------------------------- per level constants
-// Per node: Wns(v) = sum of w(e) over incident hyperedges with |e| >= 2, and
-// the number of singleton hyperedges {v} that hold v as a destination.
-// Singleton hyperedges cancel in every gain (they are spared and re-created
-// by any move) and change only the distinct-inbound count, by one per
-// singleton at p_s (-) and at p_d (+): they are handled per node.
-__global__ void k_level_nodes(const int32_t *off, const int32_t *ioff, const int32_t *inc, const int32_t *inode,
-                              const int32_t *nin, const int32_t *w, int64_t np, long long *wns, int32_t *singin) {
+// The level's classes and constants, in one pass over its nodes, hyperedges
+// and incidence (all independent of one another):
+// - parts holding at least one node (lambda(e) never exceeds their number
+//   within a level: moves only go to parts that exist);
+// - hyperedges of 2..TINY_E pins (one thread each), up to SMALL_EDGE (a warp
+//   each) and larger ones (a CTA each), and the largest;
+// - per node, Wns(v) = sum of w(e) over incident hyperedges with |e| >= 2, and
+//   the number of singleton hyperedges {v} that hold v as a destination.
+//   Singleton hyperedges cancel in every gain (they are spared and re-created
+//   by any move) and change only the distinct-inbound count, by one per
+//   singleton at p_s (-) and at p_d (+): they are handled per node.
+// Appends take one atomic per CTA and list: 229,376 hyperedges a warp at a
+// time queued 7,000 atomics on one word, most of the 12 us that took.
+constexpr int TINY_E = 8;
+constexpr int32_t SMALL_EDGE = 512;
+// largest hyperedge handled a warp each: the level's largest, at least 2, at most SMALL_EDGE
+inline int32_t level_small_max(int32_t max_e) { return max_e < 2 ? 2 : (max_e > SMALL_EDGE ? SMALL_EDGE : max_e); }
+// counters of a level: larger hyperedges, the largest, tiny ones, middle ones, parts in use
+enum { V_BIG, V_MAX, V_TINY, V_MID, V_PARTS, V_N };
+constexpr int LP_T = 256;
+__global__ void __launch_bounds__(LP_T) k_level_prep(Level L, const int32_t *w, const int32_t *rho, int32_t *pmark,
+                                                     int32_t *big, int32_t *tiny, int32_t *mid, int32_t *cnt,
+                                                     long long *wns, int32_t *singin) {
     HP_KERNEL_ENTER();
-    const int lane = threadIdx.x & 31;
-    const int64_t wbase = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) << 5;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = wbase; base < np; base += stride) {
+    __shared__ int32_t s_n[3][LP_T / 32], s_max, s_used;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const uint32_t lt = (1u << lane) - 1u;
+    if (threadIdx.x == 0) s_max = s_used = 0;
+    __syncthreads();
+    const int64_t step = (int64_t)gridDim.x * LP_T;
+    int32_t used = 0, mx = 0;
+    GRID_STRIDE(v, (int64_t)L.n) {
+        if (pmark[rho[v]] == 0 && atomicExch(&pmark[rho[v]], 1) == 0) used++;
+    }
+    for (int64_t base = (int64_t)blockIdx.x * LP_T; base < L.e; base += step) {
+        const int64_t i = base + threadIdx.x;
+        const int32_t sz = i < L.e ? L.off[i + 1] - L.off[i] : 0;
+        mx = max(mx, sz);
+        const int cls = sz < 2 ? -1 : sz <= TINY_E ? 0 : sz <= SMALL_EDGE ? 1 : 2;
+        unsigned m[3];
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            m[c] = __ballot_sync(FULL, cls == c);
+            if (lane == 0) s_n[c][wid] = __popc(m[c]);
+        }
+        __syncthreads();
+        if (threadIdx.x < 3) {   // the warps' places in their lists
+            int32_t tot = 0;
+            for (int x = 0; x < LP_T / 32; x++) tot += s_n[threadIdx.x][x];
+            int32_t at = tot ? atomicAdd(&cnt[threadIdx.x == 0 ? V_TINY : threadIdx.x == 1 ? V_MID : V_BIG], tot) : 0;
+            for (int x = 0; x < LP_T / 32; x++) {
+                const int32_t k = s_n[threadIdx.x][x];
+                s_n[threadIdx.x][x] = at;
+                at += k;
+            }
+        }
+        __syncthreads();
+        if (cls == 0) tiny[s_n[0][wid] + __popc(m[0] & lt)] = (int32_t)i;
+        if (cls == 1) mid[s_n[1][wid] + __popc(m[1] & lt)] = (int32_t)i;
+        if (cls == 2) big[s_n[2][wid] + __popc(m[2] & lt)] = (int32_t)i;
+        __syncthreads();
+    }
+    mx = __reduce_max_sync(FULL, mx);
+    used = __reduce_add_sync(FULL, used);
+    if (lane == 0) {
+        atomicMax(&s_max, mx);
+        if (used) atomicAdd(&s_used, used);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        if (s_max) atomicMax(&cnt[V_MAX], s_max);
+        if (s_used) atomicAdd(&cnt[V_PARTS], s_used);
+    }
+    for (int64_t base = (int64_t)blockIdx.x * LP_T + (threadIdx.x & ~31u); base < L.np; base += step) {
         const int64_t t = base + lane;
-        const bool valid = t < np;
-        const int32_t v = valid ? inode[t] : -1 - lane;
+        const bool valid = t < L.np;
+        const int32_t v = valid ? L.inode[t] : -1 - lane;
         long long a = 0;
         int32_t c = 0;
         if (valid) {
-            const int32_t e = inc[t];
-            const int32_t sz = off[e + 1] - off[e];
+            const int32_t e = L.inc[t];
+            const int32_t sz = L.off[e + 1] - L.off[e];
             if (sz >= 2) a = w[e];
-            else if (t < ioff[v] + nin[v]) c = 1;
+            else if (t < L.ioff[v] + L.nin[v]) c = 1;
         }
         bool tail = warp_run_sum(v, a);
         warp_run_sum(v, c);
@@ -841,26 +904,6 @@ __global__ void k_level_nodes(const int32_t *off, const int32_t *ioff, const int
             if (a) atomicAdd((unsigned long long *)&wns[v], (unsigned long long)a);
             if (c) atomicAdd(&singin[v], c);
         }
-    }
-}
-
-// hyperedges with >= 2 pins: up to TINY_E pins (one thread each), up to
-// small_max (a warp each), larger (a CTA each).  All of them form `act`
-// (the in-sequence pass); tiny ones are also listed apart.
-constexpr int TINY_E = 8;
-// largest hyperedge handled a warp each: the level's largest, at least 2, at most 512
-__host__ __device__ inline int32_t level_small_max(int32_t max_e) { return max_e < 2 ? 2 : (max_e > 512 ? 512 : max_e); }
-__global__ void k_level_edges(const int32_t *off, int32_t e, const int32_t *max_e, int32_t *act, int32_t *big,
-                              int32_t *tiny, int32_t *mid, int32_t *cnt) {
-    HP_KERNEL_ENTER();
-    const int32_t small_max = level_small_max(*max_e);
-    GRID_STRIDE(i, (int64_t)e) {
-        int32_t sz = off[i + 1] - off[i];
-        if (sz >= 2 && sz <= small_max) {
-            act[atomicAdd(&cnt[0], 1)] = (int32_t)i;
-            if (sz <= TINY_E) tiny[atomicAdd(&cnt[3], 1)] = (int32_t)i;
-            else mid[atomicAdd(&cnt[4], 1)] = (int32_t)i;
-        } else if (sz > small_max) big[atomicAdd(&cnt[1], 1)] = (int32_t)i;
     }
 }
 
@@ -961,7 +1004,7 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
 }
 
 // counters of one repetition (device)
-enum { C_CAND, C_MOVES, C_OVF, C_BAD, C_NH, C_BAD0, C_APPLIED, C_NV, C_HUB, C_CW, C_TOUCH, C_TTOUCH,
+enum { C_CAND, C_MOVES, C_OVF, C_BAD, C_NH, C_BAD0, C_APPLIED, C_NV, C_HUB, C_CW, C_TOUCH, C_PAD,
        C_ACC,          // three 64-bit byte counters (even index: 8-byte aligned), see k_cut_bits
        C_N = C_ACC + 6 };
 
@@ -2326,8 +2369,7 @@ __device__ void inseq_edge(const SeqSim &Q, int32_t e, int gt, int32_t *bk, int3
 // The hyperedges of `list` that hold a moved pin (lanes take one hyperedge
 // each; those of more than 32 pins are scanned by the whole warp).
 __global__ void k_touched(const int32_t *off, const int32_t *pin, const int32_t *mvpos, const int32_t *list,
-                          int32_t count, int32_t *out, int32_t *out_n, int32_t *tout, int32_t *tout_n,
-                          const int32_t *mcount) {
+                          int32_t count, int32_t *out, int32_t *out_n, const int32_t *mcount) {
     HP_KERNEL_ENTER();
     if (*mcount == 0) return;
     const unsigned FULL = 0xffffffffu;
@@ -2359,10 +2401,7 @@ __global__ void k_touched(const int32_t *off, const int32_t *pin, const int32_t 
             }
             if (lane == l) hit = found;
         }
-        if (hit) {
-            if (b - a <= TINY_E) tout[atomicAdd(tout_n, 1)] = e;
-            else out[atomicAdd(out_n, 1)] = e;
-        }
+        if (hit) out[atomicAdd(out_n, 1)] = e;
     }
 }
 
@@ -2494,14 +2533,15 @@ __global__ void __launch_bounds__(256) k_inseq_big(SeqSim Q, const int32_t *list
 }
 
 
-// In-sequence gains of hyperedges of at most TINY_E pins, one thread each:
+// In-sequence gains of hyperedges of at most TINY_E pins (all of the level's:
+// listing the ones with a moved pin first reads what this reads), one thread each:
 // the moved pins are taken in sequence order (ranks among at most TINY_E
 // distinct positions) and the parts they leave or enter are tracked in a
 // per-thread table of 2 TINY_E entries in shared memory.  The r-th moves of
 // a warp's hyperedges are combined by sequence position (match_any) before
 // their atomics: a moved node with many hyperedges is one position.
 constexpr int IST_T = 128;
-__global__ void __launch_bounds__(IST_T) k_inseq_tiny(SeqSim Q, const int32_t *list, const int32_t *count_p,
+__global__ void __launch_bounds__(IST_T) k_inseq_tiny(SeqSim Q, const int32_t *list, int32_t count,
                                                        const int32_t *mcount) {
     HP_KERNEL_ENTER();
     __shared__ int32_t s_tab[IST_T * 6 * TINY_E];
@@ -2509,20 +2549,16 @@ __global__ void __launch_bounds__(IST_T) k_inseq_tiny(SeqSim Q, const int32_t *l
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
-    const int32_t count = *count_p;
     int32_t *tp = s_tab + threadIdx.x * 6 * TINY_E, *tc = tp + 2 * TINY_E, *tci = tc + 2 * TINY_E;
     const int64_t step = (int64_t)gridDim.x * IST_T;
     for (int64_t base = blockIdx.x * (int64_t)IST_T + (threadIdx.x & ~31u); base < count; base += step) {
         const int64_t i = base + lane;
-        int32_t a = 0, sz = 0, d0 = 0, lam = 0;
+        int32_t e = 0, a = 0, sz = 0, d0 = 0, lam = 0;
         long long we = 0;
         if (i < count) {
-            const int32_t e = list[i];
+            e = list[i];
             a = Q.off[e];
             sz = Q.off[e + 1] - a;
-            d0 = Q.nsrc[e];
-            we = Q.w[e];
-            lam = Q.PL.lam[e];
         }
         int32_t kk[TINY_E];
         int nm = 0;
@@ -2538,6 +2574,11 @@ __global__ void __launch_bounds__(IST_T) k_inseq_tiny(SeqSim Q, const int32_t *l
             }
         }
         const int rmax = (int)__reduce_max_sync(FULL, (unsigned)nm);
+        if (nm > 0) {
+            d0 = Q.nsrc[e];
+            we = Q.w[e];
+            lam = Q.PL.lam[e];
+        }
         int nt = 0;
         for (int r = 0; r < rmax; r++) {
             int32_t k = -1;
@@ -2601,9 +2642,9 @@ struct LevelWs {
     int32_t cn, ce, nparts, cmax_e;
     int64_t cnp;
     // per level
-    int32_t n, max_e, small_max, n_act, n_big;
+    int32_t n, max_e, small_max, n_big;
     uint32_t pcap;
-    int32_t *act, *big;
+    int32_t *big;
     long long *wns;
     int32_t *singin;
     Plist PL;
@@ -2622,7 +2663,7 @@ struct LevelWs {
     bool bits_valid = false;
     uint4 *bits = nullptr;   // [ce][wq] parts of every cut hyperedge (k_part_bits), or none
     int wq = 0;
-    int32_t *touched, *ttouched;             // hyperedges with a moved pin (more than / at most 8 pins)
+    int32_t *touched;                        // hyperedges of mid with a moved pin
     Moves M, S;
     uint64_t *keys;
     uint32_t *idx;
@@ -2677,7 +2718,6 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->ce = e;
     W->nparts = nparts;
     W->cmax_e = max_e;
-    W->act = A.get<int32_t>(e);
     W->big = A.get<int32_t>(e);
     W->wns = A.get<long long>(n);
     W->singin = A.get<int32_t>(n);
@@ -2713,7 +2753,6 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->tiny = A.get<int32_t>(e);
     W->mid = A.get<int32_t>(e);
     W->touched = A.get<int32_t>(e);
-    W->ttouched = A.get<int32_t>(e);
     for (Moves *m : {&W->M, &W->S}) {
         m->node = A.get<int32_t>(n);
         m->src = A.get<int32_t>(n);
@@ -2750,7 +2789,7 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->edd = A.get<long long>(2 * (int64_t)n);
     W->vhead = A.get<int32_t>(std::max<int64_t>(nparts, 1));
     W->bgain = A.get<long long>(1);
-    W->lvl = A.get<int32_t>(6);
+    W->lvl = A.get<int32_t>(V_N);
     W->pmark = A.get<int32_t>(std::max(nparts, 1));
     // overflow tables of the gain kernel, one per CTA of its fallback grid
     W->gcap = pow2_at_least(2 * (int64_t)nparts + 2);
@@ -2770,7 +2809,7 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     // hyperedges above 512 pins: tables and buffers in global memory
     W->ptab = W->ibuf = nullptr;
     W->pnb = 0;
-    if (max_e > 512) {
+    if (max_e > SMALL_EDGE) {
         W->bcap = pow2_at_least(2 * (int64_t)max_e);
         W->pnb = num_sms() * 2;
         W->ptab = A.get<int32_t>((int64_t)W->pnb * (3 * (int64_t)W->bcap + 4 * (int64_t)max_e));
@@ -2790,9 +2829,9 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
     for (cudaEvent_t x : W->ev)
         if (x) cudaEventDestroy(x);
     for (void *p : std::initializer_list<void *>{
-             W->act, W->big, W->wns, W->singin, W->PL.p, W->PL.cnt, W->PL.cin, W->PL.lam, W->R.cnt, W->R.linked,
+             W->big, W->wns, W->singin, W->PL.p, W->PL.cnt, W->PL.cin, W->PL.lam, W->R.cnt, W->R.linked,
              W->R.D0, W->R.psize, W->R.saving, W->R.pc, W->R.pred, W->R.succ, W->R.chain, W->R.mvpos, W->R.cgain,
-             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->ttouched, W->M.node, W->M.src, W->M.dst, W->M.gain,
+             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->M.node, W->M.src, W->M.dst, W->M.gain,
              W->S.node, W->S.src, W->S.dst, W->S.gain, W->keys, W->idx, W->msz, W->mni, W->first, W->choice, W->accnode, W->pen,
              W->minpen, W->acc1, W->acc2, W->pos, W->clen, W->lens, W->starts, W->cstart, W->seqmove, W->heads, W->hkeys,
              W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
@@ -2800,28 +2839,18 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
     delete W;
 }
 
-// per level: hyperedge classes and per-node constants
-// parts holding at least one node (lambda(e) never exceeds it within a level:
-// moves only go to parts that exist)
 // the level's counters and per-part / per-node sums start at zero (one
 // launch instead of four memsets, which would each end the overlap of a
 // launch with its predecessor)
 __global__ void k_prep_zero(int32_t *lvl, int32_t *pmark, int32_t nparts, long long *wns, int32_t *singin, int32_t n) {
     HP_KERNEL_ENTER();
-    GRID_STRIDE(i, (int64_t)max(max(n, nparts), 6)) {
-        if (i < 6) lvl[i] = 0;
+    GRID_STRIDE(i, (int64_t)max(max(n, nparts), (int32_t)V_N)) {
+        if (i < V_N) lvl[i] = 0;
         if (i < nparts) pmark[i] = 0;
         if (i < n) {
             wns[i] = 0;
             singin[i] = 0;
         }
-    }
-}
-
-__global__ void k_used_parts(const int32_t *rho, int32_t n, int32_t *mark, int32_t *count) {
-    HP_KERNEL_ENTER();
-    GRID_STRIDE(v, (int64_t)n) {
-        if (atomicExch(&mark[rho[v]], 1) == 0) atomicAdd(count, 1);
     }
 }
 
@@ -2831,38 +2860,22 @@ static void level_prepare(const Level &L, const int32_t *w, const int32_t *rho, 
     W.n = n;
     W.R.n = n;
     W.R.e = e;
-    launch_k(k_prep_zero, grid_of(std::max(std::max(n, W.nparts), 6), 256), 256, 0, s, W.lvl, W.pmark, W.nparts, W.wns,
-             W.singin, n);
+    launch_k(k_prep_zero, grid_of(std::max(std::max(n, W.nparts), (int32_t)V_N), 256), 256, 0, s, W.lvl, W.pmark, W.nparts,
+             W.wns, W.singin, n);
     HP_LAUNCH_CHECK();
-    if (e > 0) {
-        launch_k(k_max_edge, grid_of(e, 256), 256, 0, s, L.off, e, W.lvl + 2);
-        HP_LAUNCH_CHECK();
-    }
-    if (n > 0) {
-        launch_k(k_used_parts, grid_of(n, 256), 256, 0, s, rho, n, W.pmark, W.lvl + 5);
-        HP_LAUNCH_CHECK();
-    }
-    if (e > 0) {
-        // the size classes take the largest hyperedge from the device (no read-back here)
-        launch_k(k_level_edges, grid_of(e, 256), 256, 0, s, L.off, e, W.lvl + 2, W.act, W.big, W.tiny, W.mid, W.lvl);
-        HP_LAUNCH_CHECK();
-    }
-    if (L.np > 0) {
-        launch_k(k_level_nodes, grid_of(L.np, 256), 256, 0, s, L.off, L.ioff, L.inc, L.inode, L.nin, w, L.np, W.wns,
-                 W.singin);
-        HP_LAUNCH_CHECK();
-    }
-    int32_t hc[6];
+    launch_k(k_level_prep, grid_of(std::max<int64_t>(std::max(n, e), L.np), LP_T), LP_T, 0, s, L, w, rho, W.pmark, W.big,
+             W.tiny, W.mid, W.lvl, W.wns, W.singin);
+    HP_LAUNCH_CHECK();
+    int32_t hc[V_N];
     fetch_bytes(hc, W.lvl, sizeof hc, s);
-    W.max_e = hc[2];
+    W.max_e = hc[V_MAX];
     W.small_max = level_small_max(W.max_e);
-    W.n_act = hc[0];
-    W.n_big = hc[1];
-    W.n_tiny = hc[3];
-    W.n_mid = hc[4];
-    W.parts_used = hc[5];
+    W.n_big = hc[V_BIG];
+    W.n_tiny = hc[V_TINY];
+    W.n_mid = hc[V_MID];
+    W.parts_used = hc[V_PARTS];
     // pins lists of the level hold at most min(small_max, parts in use) entries
-    W.pcap = pow2_at_least(2 * (int64_t)std::max<int32_t>(2, std::min<int32_t>(W.small_max, hc[5])));
+    W.pcap = pow2_at_least(2 * (int64_t)std::max<int32_t>(2, std::min<int32_t>(W.small_max, W.parts_used)));
     if (W.n_big > 0 && !W.ptab) throw Error(HP_ERR_INTERNAL, "large hyperedge buffers missing");
 }
 
@@ -3174,17 +3187,19 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
 
     // in-sequence gains and distinct-inbound changes per move
     SeqSim Z{L.off, L.pin, L.nsrc, w, R.mvpos, W.seqmove, W.S.src, W.S.dst, W.PL, R.gseq, R.dDs, R.dDd};
-    if (W.n_act > 0) {
-        launch_k(k_touched, grid_of(W.n_act, 256), 256, 0, s, L.off, L.pin, R.mvpos, W.act, W.n_act, W.touched,
-                 cnt + C_TOUCH, W.ttouched, cnt + C_TTOUCH, cnt + C_MOVES);
+    if (W.n_tiny > 0) {
+        launch_k(k_inseq_tiny, grid_of(W.n_tiny, IST_T), IST_T, 0, s, Z, W.tiny, W.n_tiny, cnt + C_MOVES);
         HP_LAUNCH_CHECK();
-        launch_k(k_inseq_tiny, grid_of(W.n_act, IST_T), IST_T, 0, s, Z, W.ttouched, cnt + C_TTOUCH, cnt + C_MOVES);
+    }
+    if (W.n_mid > 0) {
+        launch_k(k_touched, grid_of(W.n_mid, 256), 256, 0, s, L.off, L.pin, R.mvpos, W.mid, W.n_mid, W.touched, cnt + C_TOUCH,
+                 cnt + C_MOVES);
         HP_LAUNCH_CHECK();
         auto inseq_mid = [&](int32_t lo, int32_t emax) {
             if (nparts <= PB_PARTS) {
                 const size_t sm = inseq_parts_smem(nparts, emax);
                 const int occ = prepare_kernel((const void *)k_inseq_parts, IS_T, sm);
-                const int grid = (int)std::min<int64_t>(cdiv(W.n_act, IS_T / 32), (int64_t)num_sms() * occ);
+                const int grid = (int)std::min<int64_t>(cdiv(W.n_mid, IS_T / 32), (int64_t)num_sms() * occ);
                 launch_k(k_inseq_parts, std::max(grid, 1), IS_T, sm, s, Z, W.touched, cnt + C_TOUCH, emax, nparts,
                          cnt + C_MOVES, lo);
                 HP_LAUNCH_CHECK();
@@ -3192,7 +3207,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
             }
             size_t sm = (size_t)(9 * emax + 1) * 4 * (IS_T / 32);
             int occ = prepare_kernel((const void *)k_inseq_small, IS_T, sm);
-            int grid = (int)std::min<int64_t>(cdiv(W.n_act, IS_T / 32), (int64_t)num_sms() * occ);
+            int grid = (int)std::min<int64_t>(cdiv(W.n_mid, IS_T / 32), (int64_t)num_sms() * occ);
             launch_k(k_inseq_small, std::max(grid, 1), IS_T, sm, s, Z, W.touched, cnt + C_TOUCH, emax, cnt + C_MOVES, lo);
             HP_LAUNCH_CHECK();
         };
