@@ -2687,7 +2687,17 @@ struct LevelWs {
     long long *bgain;
     int32_t *lvl;   // per-level counters
     int32_t *pmark; // [nparts] parts in use
+    int32_t *pnew;  // [nparts] their ranks
 };
+
+// rows of part bits (16 * wq bytes per hyperedge) for the current number of
+// parts, where every sum of weights fits their 32-bit counters and they take
+// at most PB_BYTES
+static void part_bits_rows(LevelWs &W, const Params &P, Arena &A) {
+    if (W.nparts > PB_PARTS || P.wsum >= (1ll << 32) || P.o.debug_table_cap != 0) return;
+    W.wq = (int)pow2_at_least(std::max<int64_t>(cdiv(W.nparts, 128), 1));
+    if (!W.bits && (int64_t)W.ce * W.wq * 16 <= PB_BYTES) W.bits = A.get<uint4>((int64_t)W.ce * W.wq);
+}
 
 static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t e, int32_t nparts, int32_t max_e,
                                       const Params &P, Arena &A);
@@ -2791,6 +2801,7 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->bgain = A.get<long long>(1);
     W->lvl = A.get<int32_t>(V_N);
     W->pmark = A.get<int32_t>(std::max(nparts, 1));
+    W->pnew = A.get<int32_t>(std::max(nparts, 1));
     // overflow tables of the gain kernel, one per CTA of its fallback grid
     W->gcap = pow2_at_least(2 * (int64_t)nparts + 2);
     W->gnb = (int)std::min<int64_t>(num_sms(), std::max<int64_t>(1, ((int64_t)1 << 27) / ((int64_t)W->gcap * 12)));
@@ -2799,13 +2810,7 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->gc = A.get<long long>((int64_t)W->gnb * W->gcap);
     fill_i32(W->gk, (int64_t)W->gnb * 2 * W->gcap, -1, s);
     HPC(cudaMemsetAsync(W->gc, 0, sizeof(long long) * W->gnb * W->gcap, s));
-    // rows of part bits (16 * wq bytes per hyperedge) where every sum of
-    // weights fits their 32-bit counters and they take at most PB_BYTES
-    W->wq = (int)cdiv(nparts, 128);
-    if (nparts <= PB_PARTS && P.wsum < (1ll << 32) && P.o.debug_table_cap == 0) {
-        W->wq = (int)pow2_at_least(std::max(W->wq, 1));
-        if ((int64_t)e * W->wq * 16 <= PB_BYTES) W->bits = A.get<uint4>((int64_t)e * W->wq);
-    }
+    part_bits_rows(*W, P, A);
     // hyperedges above 512 pins: tables and buffers in global memory
     W->ptab = W->ibuf = nullptr;
     W->pnb = 0;
@@ -2834,7 +2839,7 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
              W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->M.node, W->M.src, W->M.dst, W->M.gain,
              W->S.node, W->S.src, W->S.dst, W->S.gain, W->keys, W->idx, W->msz, W->mni, W->first, W->choice, W->accnode, W->pen,
              W->minpen, W->acc1, W->acc2, W->pos, W->clen, W->lens, W->starts, W->cstart, W->seqmove, W->heads, W->hkeys,
-             W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
+             W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->pnew, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
         A.release(p);
     delete W;
 }
@@ -3290,11 +3295,30 @@ int32_t refine_rep_debug(const Level &L, const int32_t *w, int32_t nparts, const
     return k;
 }
 
+__global__ void k_relabel(const int32_t *newid, int32_t n, int32_t *rho) {
+    HP_KERNEL_ENTER();
+    GRID_STRIDE(v, (int64_t)n) rho[v] = newid[rho[v]];
+}
+// Parts that have emptied never hold a node again, so once half of the ids
+// are out of use the parts in use are renumbered in ascending order, which no
+// decision can tell from the old ids (ties go by their order).  A net that
+// stops coarsening at ten thousand nodes and ends in a hundred parts then has
+// the tables, keys and part-indexed kernels of a hundred parts.
+static void renumber_parts(const Level &L, const Params &P, int32_t *rho, LevelWs &W, Arena &A) {
+    if (2 * (int64_t)W.parts_used > W.nparts) return;
+    scan_excl(W.pmark, W.pnew, W.nparts, nullptr, A);
+    launch_k(k_relabel, grid_of(L.n, 256), 256, 0, A.stream(), W.pnew, L.n, rho);
+    HP_LAUNCH_CHECK();
+    W.nparts = W.R.nparts = W.parts_used;
+    part_bits_rows(W, P, A);
+}
+
 RefineOut refine_level(const Level &L, const int32_t *w, const Params &P, int32_t *rho, LevelWs *W, Arena &A,
                        uint32_t *err_dev) {
     RefineOut out;
     if (L.n == 0 || P.o.theta == 0) return out;
     level_prepare(L, w, rho, *W, A);
+    renumber_parts(L, P, rho, *W, A);
     const int64_t bytes0 = W->alg_bytes;
     const int32_t half = P.o.theta / 2;
     bool same_rho = false;   // the previous repetition applied nothing

@@ -86,3 +86,17 @@ def test_cut_degrees(torch, hub):
     g = graph(1500, [5] * 3100, hub, hub)
     check(torch, g, 20, hub)
     check(torch, g, 1200, hub)
+
+
+# few coarsening levels: many parts at the start, most of them empty soon, so that the rest is renumbered
+@pytest.mark.parametrize("max_levels", [0, 1, 3])
+@pytest.mark.parametrize("omega", [40, 700])
+def test_renumbered_parts(torch, max_levels, omega):
+    g = inputs.random_hypergraph(1500, 2600, 7, seed=omega, multi_src=True, weights=True)
+    r = hp.partition(g, omega, 10 ** 5, seed=4, trace=True, max_levels=max_levels)
+    o = oracle.partition(g, omega, 10 ** 5, seed=4, trace=True, max_levels=max_levels)
+    assert r.status == o.status == hp.HP_OK, hp.hp_last_error()
+    assert np.array_equal(r.part, o.part)
+    for k, v in o.stats.items():
+        assert r.stats[k] == v, k
+    assert [t["moves"] for t in r.trace] == [t["moves"] for t in o.trace]
