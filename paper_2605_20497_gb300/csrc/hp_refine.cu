@@ -2655,8 +2655,8 @@ struct LevelWs {
     int32_t *tiny, n_tiny;                   // hyperedges of 2..8 pins
     int32_t *mid, n_mid;                     // hyperedges of 9..small_max pins
     int32_t parts_used;                      // parts holding a node at the level's start
-    cudaStream_t side = nullptr;             // side stream of the hub gains
-    cudaEvent_t ev[2] = {nullptr, nullptr};
+    cudaStream_t side = nullptr, side2 = nullptr;   // side streams of the gain kernels
+    cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
     // algorithmic bytes of the repetitions (host): running total, and the cut
     // entries and their list entries of the last rebuilt repetition
     int64_t alg_bytes = 0, cuts = 0, cut_lam = 0;
@@ -2710,7 +2710,8 @@ LevelWs *refine_workspace(int32_t n, int64_t np, int32_t e, int32_t nparts, int3
     try {
         return refine_workspace_body(W, n, np, e, nparts, max_e, P, A);
     } catch (...) {
-        if (W->side) cudaStreamDestroy(W->side);
+        for (cudaStream_t x : {W->side, W->side2})
+            if (x) cudaStreamDestroy(x);
         for (cudaEvent_t x : W->ev)
             if (x) cudaEventDestroy(x);
         delete W;
@@ -2721,7 +2722,7 @@ LevelWs *refine_workspace(int32_t n, int64_t np, int32_t e, int32_t nparts, int3
 static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t e, int32_t nparts, int32_t max_e,
                                       const Params &P, Arena &A) {
     cudaStream_t s = A.stream();
-    HPC(cudaStreamCreateWithFlags(&W->side, cudaStreamNonBlocking));
+    for (cudaStream_t *x : {&W->side, &W->side2}) HPC(cudaStreamCreateWithFlags(x, cudaStreamNonBlocking));
     for (cudaEvent_t &x : W->ev) HPC(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
     W->cn = n;
     W->cnp = np;
@@ -2827,10 +2828,11 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
     if (!W) return;
     // side-stream work must be done before the arena hands its memory back
     // (it is, unless the call is ending early on an error)
-    if (W->side) {
-        (void)cudaStreamSynchronize(W->side);
-        cudaStreamDestroy(W->side);
-    }
+    for (cudaStream_t x : {W->side, W->side2})
+        if (x) {
+            (void)cudaStreamSynchronize(x);
+            cudaStreamDestroy(x);
+        }
     for (cudaEvent_t x : W->ev)
         if (x) cudaEventDestroy(x);
     for (void *p : std::initializer_list<void *>{
@@ -2896,6 +2898,147 @@ static bool bits_pay(const Level &L, const LevelWs &W) {
     if (!W.bits) return false;
     if (W.cuts == 0) return L.np >= 16 * (int64_t)L.e;
     return W.cut_lam >= W.cuts * 4 * W.wq;
+}
+
+// ---------------------------------------------------------------- gains by part
+// The list form for up to PB_PARTS parts and weight sums below 2^32: the
+// node's conn(v, p) in 32-bit counters indexed by part, so no table can
+// overflow and the node classes need not wait for one another.  NW warps per
+// node (one: several nodes a CTA); the k-th list entries of a warp's 32
+// hyperedges are combined by part before one update per distinct part, the
+// next entries and the next hyperedges loaded ahead.  Bound by the latency of
+// those loads.  Hashed tables with a spill from class to class took 100, 83
+// and 53 ms of kernel time (the last two one after the other) in the 466
+// repetitions of the 1M Gaussian net; these 48, 38 and 54, side by side.
+template <int NW>
+__global__ void __launch_bounds__(NW == 1 ? 256 : NW * 32)
+    k_gains_parts(GainArgs G, int32_t nparts, const int32_t *list, const int32_t *count_p) {
+    HP_KERNEL_ENTER();
+    extern __shared__ __align__(16) uint32_t smw[];
+    __shared__ long long s_rg[32];
+    __shared__ int32_t s_rp[32];
+    constexpr int GROUPS = NW == 1 ? 8 : 1;   // nodes a CTA has in hand
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int grp = NW == 1 ? wid : 0, gt = NW == 1 ? lane : (int)threadIdx.x;
+    const int words = (nparts + 31) / 32;
+    uint32_t *conn = smw + (size_t)grp * (words * 32 + 32), *used = conn + words * 32;
+    const int32_t count = *count_p;
+    if ((int64_t)blockIdx.x * GROUPS >= count) return;
+    for (int i = gt; i < words * 32 + 32; i += NW * 32) conn[i] = 0;
+    gsync<NW * 32>();
+    for (int64_t x = (int64_t)blockIdx.x * GROUPS + grp; x < count; x += (int64_t)gridDim.x * GROUPS) {
+        const int32_t v = list[x], s = G.rho[v];
+        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
+        auto hedge = [&](int32_t t, int32_t &a, int32_t &lam, uint32_t &we) {
+            a = lam = 0;
+            we = 0;
+            if (t < c1) {
+                const int32_t e = G.inc[t];
+                lam = G.PL.lam[e];
+                a = G.off[e];
+                we = (uint32_t)G.w[e];
+            }
+        };
+        int32_t na, nlam;
+        uint32_t nwe;
+        hedge(c0 + gt, na, nlam, nwe);
+        const int w32 = NW == 1 ? 0 : wid * 32;
+        for (int32_t base = c0 + w32; base < c1; base += NW * 32) {
+            const int32_t a = na, lam = nlam;
+            const uint32_t we = nwe;
+            if (base + NW * 32 < c1) hedge(base + NW * 32 + lane, na, nlam, nwe);
+            const int kmax = (int)__reduce_max_sync(FULL, (unsigned)lam);
+            int32_t pn = lam > 0 ? G.PL.p[a] : -1;
+            for (int k = 0; k < kmax; k++) {
+                int32_t p = pn;
+                pn = k + 1 < lam ? G.PL.p[a + k + 1] : -1;
+                if (p == s) p = -1;
+                const unsigned m = __match_any_sync(FULL, p);
+                uint32_t sw[1] = {we};
+                group_sum(m, p >= 0, sw);
+                if (p >= 0 && lane == __ffs(m) - 1) {
+                    atomicAdd(&conn[p], sw[0]);
+                    atomicOr(&used[p >> 5], 1u << (p & 31));
+                }
+            }
+        }
+        gsync<NW * 32>();
+        // the best part: the largest gain, the larger id on ties
+        long long bg = 0;
+        int32_t bp = -1;
+        const long long basev = G.saving[v] - G.wns[v];
+        const long long room = (long long)G.omega - G.size[v];
+        auto look = [&](int32_t p) {
+            const uint32_t c = conn[p];
+            conn[p] = 0;
+            if (G.second_half && G.psize[p] > room) return;
+            const long long g = basev + (long long)c;
+            if (bp < 0 || g > bg || (g == bg && p > bp)) {
+                bg = g;
+                bp = p;
+            }
+        };
+        if (NW == 1) {
+            for (uint32_t b = used[lane]; b; b &= b - 1) look(32 * lane + __ffs(b) - 1);
+            used[lane] = 0;
+        } else {
+            for (int32_t p = threadIdx.x; p < nparts; p += NW * 32)
+                if ((used[p >> 5] >> (p & 31)) & 1u) look(p);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const long long og = __shfl_down_sync(FULL, bg, o);
+            const int32_t op = __shfl_down_sync(FULL, bp, o);
+            if (op >= 0 && (bp < 0 || og > bg || (og == bg && op > bp))) {
+                bg = og;
+                bp = op;
+            }
+        }
+        if (NW > 1) {
+            if (lane == 0) {
+                s_rg[wid] = bg;
+                s_rp[wid] = bp;
+            }
+            __syncthreads();
+            if (threadIdx.x < 32) used[threadIdx.x] = 0;
+            if (threadIdx.x == 0)
+                for (int q = 1; q < NW; q++)
+                    if (s_rp[q] >= 0 && (bp < 0 || s_rg[q] > bg || (s_rg[q] == bg && s_rp[q] > bp))) {
+                        bg = s_rg[q];
+                        bp = s_rp[q];
+                    }
+        }
+        if (gt == 0 && bp >= 0 && bg > 0) {
+            const int32_t i = atomicAdd(G.M.count, 1);
+            G.M.node[i] = v;
+            G.M.src[i] = s;
+            G.M.dst[i] = bp;
+            G.M.gain[i] = bg;
+        }
+        gsync<NW * 32>();
+    }
+}
+// the three node classes side by side
+static void gains_parts(const GainArgs &G, const LevelWs &W, const int32_t *cnt, int32_t n, cudaStream_t s) {
+    const size_t sm = 4 * (size_t)(cdiv(W.nparts, 32) * 32 + 32);
+    HPC(cudaEventRecord(W.ev[0], s));
+    for (int q = 0; q < 2; q++) HPC(cudaStreamWaitEvent(q ? W.side2 : W.side, W.ev[0], 0));
+    const int occ_h = prepare_kernel((const void *)k_gains_parts<32>, 1024, sm);
+    launch_k(k_gains_parts<32>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 1024, sm, W.side, G, W.nparts, W.hubs,
+             cnt + C_HUB);
+    HP_LAUNCH_CHECK();
+    HPC(cudaEventRecord(W.ev[1], W.side));
+    const int occ_m = prepare_kernel((const void *)k_gains_parts<8>, 256, sm);
+    launch_k(k_gains_parts<8>, std::max(1, std::min<int>(n, num_sms() * occ_m)), 256, sm, W.side2, G, W.nparts, W.cl,
+             cnt + C_CAND);
+    HP_LAUNCH_CHECK();
+    HPC(cudaEventRecord(W.ev[2], W.side2));
+    const int occ = prepare_kernel((const void *)k_gains_parts<1>, 256, 8 * sm);
+    launch_k(k_gains_parts<1>, std::max(1, std::min<int>((int)cdiv(n, 8), num_sms() * occ)), 256, 8 * sm, s, G, W.nparts,
+             W.cw, cnt + C_CW);
+    HP_LAUNCH_CHECK();
+    HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
+    HPC(cudaStreamWaitEvent(s, W.ev[2], 0));
 }
 
 template <int WQ>
@@ -2998,6 +3141,8 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         else if (W.wq == 2) gains_bits<2>(G, W, cnt, n, s);
         else if (W.wq == 4) gains_bits<4>(G, W, cnt, n, s);
         else gains_bits<8>(G, W, cnt, n, s);
+    } else if (nparts <= PB_PARTS && P.wsum < (1ll << 32) && P.o.debug_table_cap == 0) {
+        gains_parts(G, W, cnt, n, s);
     } else {
         uint32_t gcap_smem = 2048;
         if (P.o.debug_table_cap > 0) gcap_smem = (uint32_t)P.o.debug_table_cap;
