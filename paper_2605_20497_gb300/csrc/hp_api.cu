@@ -407,10 +407,7 @@ hp_status hp_merge_scores(const uint8_t *feat, int64_t count, const hp_merge_mod
             return HP_ERR_INVALID_ARG;
         if (count == 0) return HP_OK;
         cudaStream_t s = static_cast<cudaStream_t>(stream);
-        hp::Arena A(s);
-        hp_merge_model *dm = A.get<hp_merge_model>(1);
-        HPC(cudaMemcpyAsync(dm, model, sizeof(hp_merge_model), cudaMemcpyHostToDevice, s));
-        hp::merge_scores(feat, count, dm, score_out, s);
+        hp::merge_scores(feat, count, *model, score_out, s);
         HPC(cudaStreamSynchronize(s));
         return HP_OK;
     });

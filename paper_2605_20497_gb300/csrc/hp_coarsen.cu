@@ -998,7 +998,7 @@ struct CoarsenWs {
     int32_t *cand;      // [n*K] top-K lists of the proposal (K = learned_k, else Pi)
     uint64_t *cscore;
     // learned merge priority (learned_k > 0)
-    hp_merge_model *model = nullptr;
+    const hp_merge_model *model = nullptr;   // the caller's (host)
     uint8_t *feat = nullptr;
     int32_t *rank = nullptr, *lscore = nullptr, *lcand = nullptr;
     uint64_t *lcs = nullptr;
@@ -1513,11 +1513,7 @@ static CoarsenWs *coarsen_workspace_body(CoarsenWs *W, int32_t n, int32_t e, con
     W->cand = A.get<int32_t>((int64_t)n * K);
     W->cscore = A.get<uint64_t>((int64_t)n * K);
     if (P.o.learned_k > 0) {
-        // no model: the workspace of the feature extraction alone
-        if (P.o.merge_model) {
-            W->model = A.get<hp_merge_model>(1);
-            HPC(cudaMemcpyAsync(W->model, P.o.merge_model, sizeof(hp_merge_model), cudaMemcpyHostToDevice, s));
-        }
+        W->model = P.o.merge_model;   // none: the workspace of the feature extraction alone
         // per-pair rows of one pass of node_batch nodes (all nodes without it)
         const int64_t rows = (int64_t)(P.o.node_batch > 0 ? std::min(P.o.node_batch, std::max(n, 1)) : n) * K;
         W->feat = A.get<uint8_t>(rows * 16);
@@ -1581,7 +1577,7 @@ void coarsen_workspace_free(CoarsenWs *W, Arena &A) {
                     (void *)W->score, (void *)W->ccount, (void *)W->fillpos,
                     (void *)W->best, (void *)W->ss0, (void *)W->ss10, (void *)W->sum0, (void *)W->kmax, (void *)W->box})
         A.release(p);
-    for (void *p : {(void *)W->model, (void *)W->feat, (void *)W->rank, (void *)W->lscore, (void *)W->lcand,
+    for (void *p : {(void *)W->feat, (void *)W->rank, (void *)W->lscore, (void *)W->lcand,
                     (void *)W->lcs})
         if (p) A.release(p);
     delete W;

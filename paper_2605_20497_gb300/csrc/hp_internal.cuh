@@ -435,7 +435,7 @@ struct LearnIn {
     const int32_t *size, *ioff, *inc, *nin;   // the level graph
     const int32_t *candK;                     // [n*K] top-K valid neighbours by (eta, id), -1 padded
     const uint64_t *csK;                      // [n*K] their eta (with noise)
-    const hp_merge_model *model;              // device copy
+    const hp_merge_model *model;              // host pointer, read during the call
     uint8_t *feat;                            // [(v1-v0)*K][16] scratch, 16-byte aligned
     int32_t *rank;                            // [(v1-v0)*K] scratch
     int32_t *score;                           // [(v1-v0)*K] scratch
@@ -455,7 +455,7 @@ double merge_grad(const uint8_t *feat, const float *label, int64_t count, const 
 void merge_adam(float *p, const float *g, float *m, float *v, int64_t step, float lr, float b1, float b2, float eps,
                 float wd, cudaStream_t s);
 void merge_quantize(const float *params, const uint8_t *calib, int64_t count, hp_merge_model &M);
-void merge_scores(const uint8_t *feat, int64_t count, const hp_merge_model *dmodel, int32_t *out, cudaStream_t s);
+void merge_scores(const uint8_t *feat, int64_t count, const hp_merge_model &model, int32_t *out, cudaStream_t s);
 
 // refinement (hp_refine.cu)
 // optional copies of the intermediate results of one repetition (device

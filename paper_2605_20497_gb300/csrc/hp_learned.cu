@@ -8,11 +8,12 @@
 // candidate relation keep the proposal graph free of cycles longer than two,
 // which the matching of Sec. V-D relies on.
 //
-// The MLP runs on the tensor cores: bf16 operands, fp32 accumulation
-// (mma.sync m16n8k16).  Weight codes lie in [-127, 127] and activations in
-// 0..255, so every operand is an exact bf16 and every product and partial
-// sum an integer below 2^21: the fp32 accumulation is exact and the score is
-// the same integer on any hardware and in any summation order.
+// The MLP runs on the tensor cores: fp16 (or bf16) operands, fp32
+// accumulation (mma.sync m16n8k16).  Weight codes lie in [-127, 127] and
+// activations in 0..255, so every operand is exact in either type and every
+// product and partial sum an integer below 2^21: the fp32 accumulation is
+// exact and the score is the same integer on any hardware and in any
+// summation order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -225,8 +226,10 @@ constexpr int W2_STRIDE = 36;   // words per row of the packed W2 (32 + 4: confl
 // so the layer-1 outputs of n-tiles 2c and 2c+1 are, as they stand in the
 // registers, the A operand of layer 2 for k-chunk c.
 __global__ void __launch_bounds__(MLP_WARPS * 32) k_merge_mlp(const uint8_t *feat, int64_t count,
-                                                               const hp_merge_model *M, int32_t *out) {
+                                                               const __grid_constant__ hp_merge_model MV,
+                                                               int32_t *out) {
     HP_KERNEL_ENTER();
+    const hp_merge_model *M = &MV;
     __shared__ uint32_t s_w1[64 * 8];           // [hidden j][feature pair]
     __shared__ uint32_t s_w2[64 * W2_STRIDE];   // [hidden k][hidden pair]
     __shared__ int32_t s_b1[64], s_b2[64], s_w3[64];
@@ -300,6 +303,171 @@ __global__ void __launch_bounds__(MLP_WARPS * 32) k_merge_mlp(const uint8_t *fea
         if (t == 0) {
             if (in0) out[r0] = b3 + acc0;
             if (in1) out[r1] = b3 + acc1;
+        }
+    }
+}
+
+// The form that nearly every model takes: fp16 operands (weight codes and
+// activations are exact in it too), and an epilogue of three instructions a
+// value instead of eight.  With c = b 2^-s + 1024, fma.rm(d, 2^-s, c) is the
+// pre-activation (d + b) / 2^s + 1024 rounded down to fp32.  Between 1024 and
+// 2048 both fp32 and, rounded towards zero, fp16 hold every integer, so the
+// conversion of two values to packed fp16 gives their floor; values outside
+// are cut to the limits 1024 and 1279 by a packed maximum and minimum, and
+// 1024 comes off exactly: clamp((d + b) >> s, 0, 255).  It needs every c to be
+// a float (mlp_exact); the scores are then the same integers.  The output
+// layer is a third matrix product with one column.  A warp takes 32 rows a
+// step, so that a weight fragment serves two products, and a lane reads its
+// four features of a row as one word (the k order of both operands is
+// permuted alike).  Bound by the mma.sync rate: 8,388,608 rows in 310 us,
+// 540 us in the general form above, which spent 67 % of its time on integer
+// instructions.
+__device__ __forceinline__ void mma_16816_f16(float (&d)[4], const uint32_t (&a)[4], uint2 b) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+__device__ __forceinline__ uint32_t act_pair(float d0, float d1, float scale, float2 c) {
+    uint32_t x;
+    asm("{\n\t.reg .f32 u, v;\n\t.reg .b32 lo, hi;\n\t"
+        "fma.rm.f32 u, %1, %3, %4;\n\t"
+        "fma.rm.f32 v, %2, %3, %5;\n\t"
+        "cvt.rz.f16x2.f32 %0, v, u;\n\t"
+        "mov.b32 lo, 0x64006400;\n\t"    // 1024, 1024
+        "mov.b32 hi, 0x64FF64FF;\n\t"    // 1279, 1279
+        "max.f16x2 %0, %0, lo;\n\t"
+        "min.f16x2 %0, %0, hi;\n\t"
+        "sub.f16x2 %0, %0, lo;\n\t}"
+        : "=&r"(x)
+        : "f"(d0), "f"(d1), "f"(scale), "f"(c.x), "f"(c.y));
+    return x;
+}
+// two bytes of w as packed fp16 (1024 + byte, less 1024)
+template <int SEL> __device__ __forceinline__ uint32_t bytes_f16(uint32_t w) {
+    uint32_t x;
+    asm("{\n\t.reg .b32 k;\n\tmov.b32 k, 0x64006400;\n\tprmt.b32 %0, %1, 0x64646464, %2;\n\tsub.f16x2 %0, %0, k;\n\t}"
+        : "=&r"(x)
+        : "r"(w), "n"(SEL));
+    return x;
+}
+__device__ __forceinline__ uint32_t pack_f16(int32_t lo, int32_t hi) {
+    uint32_t x;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(x) : "f"((float)hi), "f"((float)lo));
+    return x;
+}
+static float mlp_offset(int32_t b, int shift) { return (float)std::ldexp((double)b + std::ldexp(1024.0, shift), -shift); }
+static bool mlp_exact(const hp_merge_model &m) {
+    // b 2^-s + 1024 is exact in double (at most 42 significant bits)
+    auto ok = [](int32_t b, int shift) {
+        return (double)mlp_offset(b, shift) == std::ldexp((double)b + std::ldexp(1024.0, shift), -shift);
+    };
+    for (int i = 0; i < 64; i++)
+        if (!ok(m.b1[i], m.shift1) || !ok(m.b2[i], m.shift2)) return false;
+    return true;
+}
+
+constexpr int MF16_WARPS = 8;
+__global__ void __launch_bounds__(MF16_WARPS * 32, 2)
+    k_merge_mlp_f16(const uint8_t *feat, int64_t count, const __grid_constant__ hp_merge_model M, int32_t *out) {
+    HP_KERNEL_ENTER();
+    __shared__ uint2 s_w1[8 * 32], s_w2[32 * 32], s_w3[4 * 32];   // B fragments as a lane reads them
+    __shared__ float2 s_c1[32], s_c2[32];                          // offsets of columns 2q, 2q + 1
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    for (int i = threadIdx.x; i < 8 * 32; i += blockDim.x) {
+        const int j = (i >> 5) * 8 + ((i & 31) >> 2), f = 4 * (i & 3);   // hidden unit, first feature
+        s_w1[i] = make_uint2(pack_f16(M.w1[j][f], M.w1[j][f + 1]), pack_f16(M.w1[j][f + 2], M.w1[j][f + 3]));
+    }
+    for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
+        const int l = i & 31, c = (i >> 5) & 3, k = (i >> 7) * 8 + (l >> 2), j = 16 * c + 2 * (l & 3);
+        s_w2[i] = make_uint2(pack_f16(M.w2[k][j], M.w2[k][j + 1]), pack_f16(M.w2[k][j + 8], M.w2[k][j + 9]));
+    }
+    for (int i = threadIdx.x; i < 4 * 32; i += blockDim.x) {
+        const int l = i & 31, j = 16 * (i >> 5) + 2 * (l & 3);
+        s_w3[i] = (l >> 2) ? make_uint2(0u, 0u)   // one column
+                           : make_uint2(pack_f16(M.w3[j], M.w3[j + 1]), pack_f16(M.w3[j + 8], M.w3[j + 9]));
+    }
+    // 2^-s is a normal float for s <= 30; the offsets are exact (mlp_exact)
+    const float sc1 = __int_as_float((127 - M.shift1) << 23), sc2 = __int_as_float((127 - M.shift2) << 23);
+    for (int i = threadIdx.x; i < 32; i += blockDim.x) {
+        auto off = [](int32_t b, int sh) { return (float)(((double)b + (double)(1024ll << sh)) / (double)(1ll << sh)); };
+        s_c1[i] = make_float2(off(M.b1[2 * i], M.shift1), off(M.b1[2 * i + 1], M.shift1));
+        s_c2[i] = make_float2(off(M.b2[2 * i], M.shift2), off(M.b2[2 * i + 1], M.shift2));
+    }
+    __syncthreads();
+    const int32_t b3 = M.b3;
+    const int64_t steps = (count + 31) / 32, stride = (int64_t)gridDim.x * MF16_WARPS;
+    const int64_t s0 = (int64_t)blockIdx.x * MF16_WARPS + (threadIdx.x >> 5);
+    auto word = [&](int64_t step, int k) -> uint32_t {   // features 4t..4t+3 of row 8k + g of the step
+        const int64_t r = step * 32 + 8 * k + g;
+        return r < count ? __ldg(reinterpret_cast<const uint32_t *>(feat + r * 16) + t) : 0u;
+    };
+    uint32_t nx[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) nx[k] = s0 < steps ? word(s0, k) : 0u;
+    // warp-uniform loop: all 32 lanes take part in every MMA
+    for (int64_t step = s0; step < steps; step += stride) {
+        uint32_t x[2][4];
+#pragma unroll
+        for (int m = 0; m < 2; m++) {
+            x[m][0] = bytes_f16<0x4140>(nx[2 * m]);
+            x[m][1] = bytes_f16<0x4140>(nx[2 * m + 1]);
+            x[m][2] = bytes_f16<0x4342>(nx[2 * m]);
+            x[m][3] = bytes_f16<0x4342>(nx[2 * m + 1]);
+        }
+        if (step + stride < steps) {
+#pragma unroll
+            for (int k = 0; k < 4; k++) nx[k] = word(step + stride, k);   // the next step's rows
+        }
+        uint32_t h[2][4][4];   // layer-2 A fragments, one per k-chunk of 16 hidden units
+#pragma unroll
+        for (int c = 0; c < 4; c++)
+#pragma unroll
+            for (int half = 0; half < 2; half++) {
+                const int nt = 2 * c + half;
+                const uint2 b = s_w1[nt * 32 + lane];
+                const float2 off = s_c1[nt * 4 + t];
+#pragma unroll
+                for (int m = 0; m < 2; m++) {
+                    float d[4] = {0.f, 0.f, 0.f, 0.f};
+                    mma_16816_f16(d, x[m], b);
+                    h[m][c][2 * half] = act_pair(d[0], d[1], sc1, off);
+                    h[m][c][2 * half + 1] = act_pair(d[2], d[3], sc1, off);
+                }
+            }
+        float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+        for (int c3 = 0; c3 < 4; c3++) {
+            uint32_t y[2][4];
+#pragma unroll
+            for (int half = 0; half < 2; half++) {
+                const int nt = 2 * c3 + half;
+                float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const uint2 b = s_w2[(nt * 4 + c) * 32 + lane];
+#pragma unroll
+                    for (int m = 0; m < 2; m++) mma_16816_f16(d[m], h[m][c], b);
+                }
+                const float2 off = s_c2[nt * 4 + t];
+#pragma unroll
+                for (int m = 0; m < 2; m++) {
+                    y[m][2 * half] = act_pair(d[m][0], d[m][1], sc2, off);
+                    y[m][2 * half + 1] = act_pair(d[m][2], d[m][3], sc2, off);
+                }
+            }
+            const uint2 b = s_w3[c3 * 32 + lane];
+#pragma unroll
+            for (int m = 0; m < 2; m++) mma_16816_f16(o[m], y[m], b);
+        }
+        if (t == 0) {   // column 0 of the output product
+#pragma unroll
+            for (int m = 0; m < 2; m++) {
+                const int64_t r = step * 32 + 16 * m + g;
+                if (r < count) out[r] = b3 + __float2int_rn(o[m][0]);
+                if (r + 8 < count) out[r + 8] = b3 + __float2int_rn(o[m][2]);
+            }
         }
     }
 }
@@ -773,11 +941,18 @@ void merge_features(const LearnIn &X, cudaStream_t s) {
     HP_LAUNCH_CHECK();
 }
 
-void merge_scores(const uint8_t *feat, int64_t count, const hp_merge_model *dmodel, int32_t *out, cudaStream_t s) {
+void merge_scores(const uint8_t *feat, int64_t count, const hp_merge_model &model, int32_t *out, cudaStream_t s) {
     if (count <= 0) return;
+    if (mlp_exact(model) && (reinterpret_cast<uintptr_t>(feat) & 3) == 0) {
+        const int occ = prepare_kernel((const void *)k_merge_mlp_f16, MF16_WARPS * 32, 0);
+        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(cdiv(count, 32), MF16_WARPS), (int64_t)num_sms() * occ));
+        launch_k(k_merge_mlp_f16, grid, MF16_WARPS * 32, 0, s, feat, count, model, out);
+        HP_LAUNCH_CHECK();
+        return;
+    }
     const int64_t tiles = cdiv(count, 16);
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(tiles, MLP_WARPS), (int64_t)num_sms() * 8));
-    launch_k(k_merge_mlp, grid, MLP_WARPS * 32, 0, s, feat, count, dmodel, out);
+    launch_k(k_merge_mlp, grid, MLP_WARPS * 32, 0, s, feat, count, model, out);
     HP_LAUNCH_CHECK();
 }
 
@@ -794,7 +969,7 @@ void learned_candidates(LearnIn X, int32_t batch, cudaStream_t s) {
         const int64_t pairs = (int64_t)(X.v1 - X.v0) * X.K;
         launch_k(k_merge_feats_node, grid_for((int64_t)(X.v1 - X.v0) * 32, MF_T), MF_T, 0, s, X);
         HP_LAUNCH_CHECK();
-        merge_scores(X.feat, pairs, X.model, X.score, s);
+        merge_scores(X.feat, pairs, *X.model, X.score, s);
         launch_k(k_merge_select, grid_for(X.v1 - X.v0, 128), 128, 0, s, X);
         HP_LAUNCH_CHECK();
     }
