@@ -488,6 +488,21 @@ hp_status hp_connectivity(const int32_t *pins, const int32_t *offsets, int32_t n
         cudaStream_t s = static_cast<cudaStream_t>(stream);
         hp::noalloc_prepare();
         hp::Arena A(s);
+        if ((pins || num_hedges == 0) && hp::connectivity_scan_takes(num_parts)) {
+            // one pass over the pins; hyperedges whose destinations do not
+            // ascend need the incidence below to find duplicates
+            int64_t conn = 0, cut = 0;
+            uint32_t bad_part = 0;
+            const uint32_t err = hp::connectivity_scan(pins, offsets, num_hedges, num_nodes, weights, part, num_parts,
+                                                       &conn, &cut, &bad_part, A);
+            if (!(err & (1u << 31)) || (err & (hp::E_OFFSETS | hp::E_PIN | hp::E_DUP))) {
+                if (err & ~(1u << 31)) return hp::status_of(err & ~(1u << 31));
+                if (bad_part) return HP_ERR_INVALID_ARG;
+                if (conn_out) *conn_out = conn;
+                if (cutnet_out) *cutnet_out = cut;
+                return HP_OK;
+            }
+        }
         hp::Params P;
         P.omega = 1;
         P.delta = 0x7fffffff;

@@ -486,6 +486,12 @@ RefineOut refine_level(const Level &L, const int32_t *w, const Params &P, int32_
                        uint32_t *err_dev);
 void objective(const Level &L, const int32_t *w, const int32_t *rho, int32_t nparts, int64_t *conn_dev,
                int64_t *cutnet_dev, Arena &A);
+// Eq. 1 and Eq. 16 of a caller's arrays (hp_connectivity), up to
+// connectivity_scan_takes parts; see the definition
+uint32_t connectivity_scan(const int32_t *pins, const int32_t *offsets, int32_t e, int32_t n, const int32_t *weights,
+                           const int32_t *part, int32_t nparts, int64_t *conn, int64_t *cutnet, uint32_t *bad_part,
+                           Arena &A);
+bool connectivity_scan_takes(int32_t nparts);
 void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t nparts, int32_t omega, int32_t delta,
                 int64_t *out, Arena &A);
 
