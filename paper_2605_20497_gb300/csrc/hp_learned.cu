@@ -440,21 +440,24 @@ __global__ void __launch_bounds__(MF16_WARPS * 32, 2)
 #pragma unroll
         for (int c3 = 0; c3 < 4; c3++) {
             uint32_t y[2][4];
+            float d[2][2][4];   // four chains of four products side by side
+#pragma unroll
+            for (int q = 0; q < 16; q++) d[q >> 3][(q >> 2) & 1][q & 3] = 0.f;
+#pragma unroll
+            for (int c = 0; c < 4; c++)
+#pragma unroll
+                for (int half = 0; half < 2; half++) {
+                    const uint2 b = s_w2[((2 * c3 + half) * 4 + c) * 32 + lane];
+#pragma unroll
+                    for (int m = 0; m < 2; m++) mma_16816_f16(d[half][m], h[m][c], b);
+                }
 #pragma unroll
             for (int half = 0; half < 2; half++) {
-                const int nt = 2 * c3 + half;
-                float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-#pragma unroll
-                for (int c = 0; c < 4; c++) {
-                    const uint2 b = s_w2[(nt * 4 + c) * 32 + lane];
-#pragma unroll
-                    for (int m = 0; m < 2; m++) mma_16816_f16(d[m], h[m][c], b);
-                }
-                const float2 off = s_c2[nt * 4 + t];
+                const float2 off = s_c2[(2 * c3 + half) * 4 + t];
 #pragma unroll
                 for (int m = 0; m < 2; m++) {
-                    y[m][2 * half] = act_pair(d[m][0], d[m][1], sc2, off);
-                    y[m][2 * half + 1] = act_pair(d[m][2], d[m][3], sc2, off);
+                    y[m][2 * half] = act_pair(d[half][m][0], d[half][m][1], sc2, off);
+                    y[m][2 * half + 1] = act_pair(d[half][m][2], d[half][m][3], sc2, off);
                 }
             }
             const uint2 b = s_w3[c3 * 32 + lane];
@@ -522,7 +525,13 @@ __global__ void k_merge_select(LearnIn X) {
 constexpr int NPAR = HP_MERGE_NPARAM;
 constexpr int P_W1 = 0, P_B1 = 1024, P_W2 = 1088, P_B2 = 5184, P_W3 = 5248, P_B3 = 5312;
 static_assert(P_B3 + 1 == NPAR, "parameter layout");
-constexpr int GRAD_CTAS = 256;   // fixed: the reduction order does not depend on the GPU
+// fixed: the reduction order does not depend on the GPU.  One CTA an SM (its
+// registers allow no more), one wave: 256 CTAs took two waves of two tiles
+// each for 65,536 rows (33 us against 28.5), each with its own load of
+// the parameters and write of the partial sums.
+constexpr int GRAD_CTAS = 152;
+constexpr int GS_SEG = 8, GS_C = GRAD_CTAS / GS_SEG;   // k_merge_grad_sum: segments of GS_C CTAs
+static_assert(GS_SEG * GS_C == GRAD_CTAS, "equal segments");
 constexpr int GRAD_W = 8;        // warps per CTA, 16 rows each
 constexpr int GRAD_T = GRAD_W * 32;
 constexpr int GRAD_R = GRAD_W * 16;   // rows per tile
@@ -817,20 +826,35 @@ __global__ void __launch_bounds__(GRAD_T) k_merge_grad(const uint8_t *feat, cons
     }
 }
 
-// the CTAs' partial gradients summed in CTA order (deterministic)
-__global__ void k_merge_grad_sum(const float *partial, const double *loss_part, int64_t count, float *grad,
-                                 double *loss) {
+// The CTAs' partial gradients, summed in a fixed order: eight segments of 19
+// CTAs in CTA order, then the segments in order (deterministic).  A block takes
+// 32 parameters, a warp a segment; the block after the last sums the loss.
+// One thread a parameter left 21 CTAs in a chain of 256 loads: 22.5 us, 5.3 this way.
+__global__ void __launch_bounds__(GS_SEG * 32) k_merge_grad_sum(const float *partial, const double *loss_part,
+                                                                int64_t count, float *grad, double *loss) {
     HP_KERNEL_ENTER();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < NPAR) {
-        float a = 0.f;
-        for (int c = 0; c < GRAD_CTAS; c++) a += partial[(int64_t)c * NPAR + i];
-        grad[i] = a;
-    }
-    if (i == 0) {
+    __shared__ float s_sum[GS_SEG][32];
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+    if (blockIdx.x == gridDim.x - 1) {
+        if (seg) return;
         double t = 0.0;
-        for (int c = 0; c < GRAD_CTAS; c++) t += loss_part[c];
-        *loss = count > 0 ? t / (double)count : 0.0;
+        for (int c = lane; c < GRAD_CTAS; c += 32) t += loss_part[c];
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+        if (lane == 0) *loss = count > 0 ? t / (double)count : 0.0;
+        return;
+    }
+    const int i = blockIdx.x * 32 + lane;
+    float a = 0.f;
+    if (i < NPAR) {
+        const float *p = partial + (int64_t)seg * GS_C * NPAR + i;
+#pragma unroll
+        for (int c = 0; c < GS_C; c++) a += p[(int64_t)c * NPAR];
+    }
+    s_sum[seg][lane] = a;
+    __syncthreads();
+    if (seg == 0 && i < NPAR) {
+        for (int k = 1; k < GS_SEG; k++) a += s_sum[k][lane];
+        grad[i] = a;
     }
 }
 
@@ -852,15 +876,14 @@ __global__ void k_merge_adam(float *p, const float *g, float *m, float *v, float
 double merge_grad(const uint8_t *feat, const float *label, int64_t count, const float *params, float *grad,
                   Arena &A) {
     cudaStream_t s = A.stream();
-    float *partial = A.get<float>((int64_t)GRAD_CTAS * NPAR);
-    double *lp = A.get<double>(GRAD_CTAS + 1);
+    double *lp = A.get<double>(GRAD_CTAS + 1 + (GRAD_CTAS * NPAR + 1) / 2);   // the CTAs' losses, the loss, the partial sums
+    float *partial = reinterpret_cast<float *>(lp + GRAD_CTAS + 1);
     prepare_kernel((const void *)k_merge_grad, GRAD_T, sizeof(GradSmem));
     launch_k(k_merge_grad, GRAD_CTAS, GRAD_T, sizeof(GradSmem), s, feat, label, count, params, partial, lp);
     HP_LAUNCH_CHECK();
-    launch_k(k_merge_grad_sum, (NPAR + 255) / 256, 256, 0, s, partial, lp, count, grad, lp + GRAD_CTAS);
+    launch_k(k_merge_grad_sum, (NPAR + 31) / 32 + 1, GS_SEG * 32, 0, s, partial, lp, count, grad, lp + GRAD_CTAS);
     HP_LAUNCH_CHECK();
     const double loss = fetch<double>(lp + GRAD_CTAS, s);
-    A.release(partial);
     A.release(lp);
     return loss;
 }
