@@ -440,24 +440,21 @@ __global__ void __launch_bounds__(MF16_WARPS * 32, 2)
 #pragma unroll
         for (int c3 = 0; c3 < 4; c3++) {
             uint32_t y[2][4];
-            float d[2][2][4];   // four chains of four products side by side
-#pragma unroll
-            for (int q = 0; q < 16; q++) d[q >> 3][(q >> 2) & 1][q & 3] = 0.f;
-#pragma unroll
-            for (int c = 0; c < 4; c++)
-#pragma unroll
-                for (int half = 0; half < 2; half++) {
-                    const uint2 b = s_w2[((2 * c3 + half) * 4 + c) * 32 + lane];
-#pragma unroll
-                    for (int m = 0; m < 2; m++) mma_16816_f16(d[half][m], h[m][c], b);
-                }
 #pragma unroll
             for (int half = 0; half < 2; half++) {
-                const float2 off = s_c2[(2 * c3 + half) * 4 + t];
+                const int nt = 2 * c3 + half;
+                float d[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    const uint2 b = s_w2[(nt * 4 + c) * 32 + lane];
+#pragma unroll
+                    for (int m = 0; m < 2; m++) mma_16816_f16(d[m], h[m][c], b);
+                }
+                const float2 off = s_c2[nt * 4 + t];
 #pragma unroll
                 for (int m = 0; m < 2; m++) {
-                    y[m][2 * half] = act_pair(d[half][m][0], d[half][m][1], sc2, off);
-                    y[m][2 * half + 1] = act_pair(d[half][m][2], d[half][m][3], sc2, off);
+                    y[m][2 * half] = act_pair(d[m][0], d[m][1], sc2, off);
+                    y[m][2 * half + 1] = act_pair(d[m][2], d[m][3], sc2, off);
                 }
             }
             const uint2 b = s_w3[c3 * 32 + lane];
