@@ -37,6 +37,7 @@ static int grid_of(int64_t n, int block) {
 
 constexpr int PT = 256;          // proposal CTA size
 constexpr int DENSE_N = 16384;   // direct-indexed table up to this many nodes (12 B per node)
+constexpr int DENSE_NARROW_N = 26624;   // and up to this many with two-word counters (8 B per node)
 
 // ---------------------------------------------------------------- noise
 // SplitMix64 finaliser (Steele, Lea, Flood 2014) keyed by (seed, level,
@@ -494,35 +495,37 @@ __device__ __forceinline__ void warp_walk(const PropCtx &C, int32_t v, int32_t i
     }
 }
 
-// Shared-memory queue of the lists one CTA walks: blockDim.x entries.  n and
-// next are two words each, zero on entry and on exit of cta_walk.
-template <int BT> struct ListQueue {
-    unsigned long long q[BT];
-    int32_t beg[BT], end[BT], d0[BT];
-    uint32_t ic[BT];
+// Shared-memory queue of the lists one CTA walks: an entry per hyperedge of a
+// chunk.  n and next are two words each, zero on entry and on exit of cta_walk.
+template <int CHUNK> struct ListQueue {
+    static constexpr int CH = CHUNK;   // hyperedges read at a time, at most one a thread
+    unsigned long long q[CH];
+    int32_t beg[CH], end[CH], d0[CH];
+    uint32_t ic[CH];
     int32_t n[2], next[2];
 };
 
-// A CTA's walk over all of v's hyperedges in chunks of BT: small ones as
+// A CTA's walk over all of v's hyperedges in the queue's chunks: small ones as
 // above, larger ones queued and taken by the warps as they come free.  On
 // levels with destination-list groups the queue holds one entry per group of a
 // warp's hyperedges with equal lists, with the group's sum of q(e) and, when v
 // is one of those destinations, its size as the overlap; their source pins
 // are entered by the hyperedge's own lane.  The chunk after the current one
 // is loaded ahead.  Stops early (for every thread) once *stop is set.
-template <int BT, class Ins>
+template <class Queue, class Ins>
 __device__ void cta_walk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, int32_t nin_v, const int *stop,
-                         ListQueue<BT> &Q, const Ins &ins) {
+                         Queue &Q, const Ins &ins) {
     const unsigned FULL = 0xffffffffu;
     const int tid = threadIdx.x, lane = tid & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const int32_t slack = size_slack(C, v);
     const int32_t *canon = dst_groups_of(C);
     int par = 0;
-    Hedge nx = hedge_of(C, i0, tid, deg, nin_v);
-    for (int32_t base = 0; base < deg; base += BT, par ^= 1) {
+    constexpr int CH = Queue::CH;
+    Hedge nx = hedge_of(C, i0, tid < CH ? tid : deg, deg, nin_v);
+    for (int32_t base = 0; base < deg; base += CH, par ^= 1) {
         const Hedge x = nx;
-        if (base + BT < deg) nx = hedge_of(C, i0, base + BT + tid, deg, nin_v);
+        if (base + CH < deg) nx = hedge_of(C, i0, tid < CH ? base + CH + tid : deg, deg, nin_v);
         walk_small(C, v, slack, x, ins);
         const bool large = x.sz > SMALL_E;
         if (__any_sync(FULL, large)) {
@@ -742,9 +745,10 @@ template <bool WIDE, class Slot> struct HashTab {
 
 // ---------------------------------------------------------------- dense table
 // eta[m], inter[m] for every node of the level in shared memory (levels of at
-// most DENSE_N nodes, nodes with large neighbourhoods).
-template <int PIMAX, int BT, bool WIDE>
-__device__ void propose_dense_node(const PropCtx &C, int32_t v, const Tab &T, ListQueue<BT> &Q, Cand *s_top,
+// most DENSE_N nodes, nodes with large neighbourhoods; up to DENSE_NARROW_N
+// without the third word, for nodes that need none).
+template <int PIMAX, int BT, bool WIDE, class Queue>
+__device__ void propose_dense_node(const PropCtx &C, int32_t v, const Tab &T, Queue &Q, Cand *s_top,
                                    int32_t *s_tmp) {
     const int32_t i0 = C.ioff[v], deg = C.ioff[v + 1] - i0;
     const Fmt f = fmt_of(deg);
@@ -757,23 +761,25 @@ __device__ void propose_dense_node(const PropCtx &C, int32_t v, const Tab &T, Li
     const int32_t tot = block_sum_i32(cnt, s_tmp);
     if (threadIdx.x == 0) C.nbcnt[v] = tot;
 }
-template <int PIMAX, int BT>
+// (a chunk below BT leaves the queue's shared memory to the table)
+template <int PIMAX, int BT, int CH = BT>
 __global__ void __launch_bounds__(BT) k_propose_dense(PropCtx C, const int32_t *list, const int32_t *count_p) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) unsigned char smem[];
     uint32_t *w = reinterpret_cast<uint32_t *>(smem);
     const Tab T{nullptr, w, w + 2 * C.n, w + C.n};
-    __shared__ ListQueue<BT> Q;
+    __shared__ ListQueue<CH> Q;
     __shared__ Cand s_top[32 * EMIT_W + 1];
     __shared__ int32_t s_tmp[32];
     const int32_t count = *count_p;
     if ((int32_t)blockIdx.x >= count) return;
-    for (int32_t i = threadIdx.x; i < 3 * C.n; i += BT) w[i] = 0;
+    const bool both = C.n <= DENSE_N;
+    for (int32_t i = threadIdx.x; i < (both ? 3 : 2) * C.n; i += BT) w[i] = 0;
     if (threadIdx.x < 2) Q.n[threadIdx.x] = Q.next[threadIdx.x] = 0;
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
         const int32_t v = list[k];
-        if (C.ioff[v + 1] - C.ioff[v] <= C.deg_narrow) propose_dense_node<PIMAX, BT, false>(C, v, T, Q, s_top, s_tmp);
+        if (!both || C.ioff[v + 1] - C.ioff[v] <= C.deg_narrow) propose_dense_node<PIMAX, BT, false>(C, v, T, Q, s_top, s_tmp);
         else propose_dense_node<PIMAX, BT, true>(C, v, T, Q, s_top, s_tmp);
     }
 }
@@ -951,14 +957,16 @@ constexpr int32_t DENSE_ALL = 4096;
 struct TierRule {
     uint32_t warp_limit;
     int32_t dense_bound, deg_narrow;
+    int32_t large_bound;   // hashed nodes of a larger bound start in the largest shared-memory table
+    bool dense_wide;       // the dense tables hold the wide counters too
     long long warp_visits, hub_visits;
 };
 // First the bound on |N(v)| (its old value, the sum over I(v), the level's
 // other nodes) and the level's noise cap, from the sum of q.
 __global__ void k_tiers(int32_t *bound, const long long *nsum, LevelBox *box, int32_t e, int32_t permille,
                         const long long *vis, const int32_t *ioff, int32_t n, TierRule R,
-                        int32_t *lW, int32_t *lB, int32_t *lH, int32_t *lD, int32_t *lDH, int32_t *cnt, int32_t pi,
-                        int32_t *cand, uint64_t *cscore) {
+                        int32_t *lW, int32_t *lB, int32_t *lC, int32_t *lH, int32_t *lD, int32_t *lDH, int32_t *cnt,
+                        int32_t pi, int32_t *cand, uint64_t *cscore) {
     HP_KERNEL_ENTER();
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         box->cap = e > 0 ? (uint64_t)((box->qsum / (unsigned long long)e) * (unsigned long long)permille / 1000ull)
@@ -979,10 +987,11 @@ __global__ void k_tiers(int32_t *bound, const long long *nsum, LevelBox *box, in
         const int32_t deg = ioff[v + 1] - ioff[v];
         const bool wide = deg > R.deg_narrow, hub = vis[v] > R.hub_visits || deg > HUB_INCIDENCE || wide;
         if ((uint32_t)bv <= R.warp_limit && vis[v] <= R.warp_visits && !wide) lW[atomicAdd(&cnt[0], 1)] = (int32_t)v;
-        else if (bv > R.dense_bound) {
+        else if (bv > R.dense_bound && (R.dense_wide || !wide)) {
             if (hub) lDH[atomicAdd(&cnt[7], 1)] = (int32_t)v;
             else lD[atomicAdd(&cnt[6], 1)] = (int32_t)v;
-        } else if (hub) lH[atomicAdd(&cnt[5], 1)] = (int32_t)v;
+        } else if (bv > R.large_bound) lC[atomicAdd(&cnt[2], 1)] = (int32_t)v;
+        else if (hub) lH[atomicAdd(&cnt[5], 1)] = (int32_t)v;
         else lB[atomicAdd(&cnt[1], 1)] = (int32_t)v;
     }
 }
@@ -1032,13 +1041,24 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
     R.warp_visits = C.n <= DENSE_ALL ? WARP_VISITS_FEW : WARP_VISITS;
     R.hub_visits = HUB_VISITS;
     // dense tables only on small levels, for neighbourhoods too large for the first hashed table
-    R.dense_bound = 0x7fffffff;
-    if (C.n <= DENSE_N && dbg == 0) R.dense_bound = (int32_t)(capB / 2);
+    R.dense_bound = R.large_bound = 0x7fffffff;
+    R.dense_wide = C.n <= DENSE_N;
+    // Linear probing slows down steeply above half a table, so the first one
+    // is left at five eighths of its slots (at three quarters a level of
+    // 19,000 power-law nodes took 20.9 ms).  After level 0 the bound is the sum
+    // of two exact counts, so that a node whose bound is twice that limit
+    // would leave it anyway.
+    const uint32_t limB = dbg > 0 ? capB * 3 / 4 : capB * 5 / 8;
+    if (C.size_filter && dbg == 0) R.large_bound = (int32_t)(2 * limB);
+    // (a dense table is also scanned: above DENSE_N nodes it is for
+    // neighbourhoods of a fifth of the level)
+    if (C.n <= DENSE_NARROW_N && dbg == 0)
+        R.dense_bound = R.dense_wide ? (int32_t)(capB / 2) : std::max((int32_t)(capB / 2), C.n / 5);
     if (C.n <= DENSE_ALL && dbg == 0) {
         R.dense_bound = 0;
         R.hub_visits = HUB_VISITS_FEW;
     }
-    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.nsum, W.box, L.e, P.o.noise_permille, W.vis, L.ioff, C.n, R, W.lW, W.lB, W.lH, W.lD, W.lDH, W.cnt,
+    launch_k(k_tiers, grid_of(C.n, 256), 256, 0, s, L.nbnd, W.nsum, W.box, L.e, P.o.noise_permille, W.vis, L.ioff, C.n, R, W.lW, W.lB, W.lC, W.lH, W.lD, W.lDH, W.cnt,
              C.pi, C.cand, C.cscore);
     HP_LAUNCH_CHECK();
     // the tiers take disjoint node lists, so they run side by side: the warp
@@ -1062,32 +1082,37 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
     if (dense) {
         // hubs first; the other nodes by CTAs of 256 threads, of 1024 where
         // the tables leave room for few CTAs on an SM
-        size_t sm = (size_t)C.n * 12;
-        const int occ_h = prepare_kernel((const void *)k_propose_dense<PIMAX, 1024>, 1024, sm);
+        size_t sm = (size_t)C.n * (R.dense_wide ? 12 : 8);
         cudaStream_t sdh = hashed ? sd : s;   // (no hashed tiers: the main stream is free)
-        launch_k(k_propose_dense<PIMAX, 1024>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sdh, C, W.lDH,
-                 W.cnt + 7);
-        HP_LAUNCH_CHECK();
-        const int occ = prepare_kernel((const void *)k_propose_dense<PIMAX, PT>, PT, sm);
-        if (occ * PT >= occ_h * 1024)
-            launch_k(k_propose_dense<PIMAX, PT>, std::max(1, std::min<int>(C.n, sms * occ)), PT, sm, sd, C, W.lD, W.cnt + 6);
-        else
-            launch_k(k_propose_dense<PIMAX, 1024>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sd, C, W.lD,
-                     W.cnt + 6);
-        HP_LAUNCH_CHECK();
+        auto run = [&](auto kern, int bt, cudaStream_t x, const int32_t *list, const int32_t *count) {
+            const int occ = prepare_kernel((const void *)kern, bt, sm);
+            launch_k(kern, std::max(1, std::min<int>(C.n, sms * occ)), bt, sm, x, C, list, count);
+            HP_LAUNCH_CHECK();
+        };
+        if (!R.dense_wide) {
+            run(k_propose_dense<PIMAX, 1024, 512>, 1024, sdh, W.lDH, W.cnt + 7);
+            run(k_propose_dense<PIMAX, 1024, 512>, 1024, sd, W.lD, W.cnt + 6);
+        } else {
+            run(k_propose_dense<PIMAX, 1024>, 1024, sdh, W.lDH, W.cnt + 7);
+            if (prepare_kernel((const void *)k_propose_dense<PIMAX, PT>, PT, sm) * PT >=
+                prepare_kernel((const void *)k_propose_dense<PIMAX, 1024>, 1024, sm) * 1024)
+                run(k_propose_dense<PIMAX, PT>, PT, sd, W.lD, W.cnt + 6);
+            else
+                run(k_propose_dense<PIMAX, 1024>, 1024, sd, W.lD, W.cnt + 6);
+        }
         HPC(cudaEventRecord(W.ev[2], sd));
     }
     if (hashed) {
         size_t sm = hash_smem(capB, true);
         const int occ_h = prepare_kernel((const void *)k_propose_smem<PIMAX, 1024, true>, 1024, sm);
         launch_k(k_propose_smem<PIMAX, 1024, true>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sh, C, W.lH,
-                 W.cnt + 5, capB, capB * 3 / 4, W.lC, W.cnt + 2);
+                 W.cnt + 5, capB, limB, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
         HPC(cudaEventRecord(W.ev[3], sh));
         sm = hash_smem(capB, false);
         int occ = prepare_kernel((const void *)k_propose_smem<PIMAX, PB, false>, PB, sm);
         launch_k(k_propose_smem<PIMAX, PB, false>, std::max(1, std::min<int>(C.n, sms * occ)), PB, sm, s,
-            C, W.lB, W.cnt + 1, capB, capB * 3 / 4, W.lC, W.cnt + 2);
+            C, W.lB, W.cnt + 1, capB, limB, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
         HPC(cudaStreamWaitEvent(s, W.ev[3], 0));
         // nodes whose neighbourhood outgrew the first table (the bound can be far above the truth)

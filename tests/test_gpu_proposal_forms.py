@@ -50,7 +50,7 @@ def check_level(torch, g, level, omega=12, delta=10 ** 6, pi=4):
 
 
 # dense tables for every node up to 4,096 nodes, for large neighbourhoods up to 16,384
-@pytest.mark.parametrize("n", [1, 2, 33, 4096, 4097, 16384, 16385])
+@pytest.mark.parametrize("n", [1, 2, 33, 4096, 4097, 16384, 16385, 26624, 26625])
 @pytest.mark.parametrize("pi", [4, 16])
 def test_level_sizes(torch, n, pi):
     g = fixed_size(n, 2 * n + 1, min(n, 13), min(3, n - 1), n, None) if n > 1 else inputs.random_hypergraph(1, 3, 1)
@@ -92,3 +92,21 @@ def test_noise_caps(torch, permille):
         r = hp.partition(g, 16, 10 ** 6, seed=9, noise_permille=permille)
         o = oracle.partition(g, 16, 10 ** 6, seed=9, noise_permille=permille)
         assert r.status == o.status == hp.HP_OK and np.array_equal(r.part, o.part)
+
+
+# large neighbourhoods: dense tables up to 26,624 nodes, then the hashed tables' limits (2,560, 6,144 neighbours)
+@pytest.mark.parametrize("n", [16400, 26624, 26625, 40000])
+@pytest.mark.parametrize("pi", [4, 16])
+def test_large_neighbourhoods(torch, n, pi):
+    rng = np.random.default_rng(n)
+    rows = [rng.choice(n, size=k, replace=False) for k in [40] * 3000 + [700] * 30]
+    # nodes 0..5 in 64 to 280 hyperedges of 40 pins: 2,500 to 9,000 neighbours
+    for h, reps in enumerate((64, 66, 72, 158, 170, 280)):
+        for i in rng.choice(3000, size=reps, replace=False):
+            rows[i][h] = h
+    rows = [np.unique(r) for r in rows]
+    off = np.zeros(len(rows) + 1, np.int64)
+    off[1:] = np.cumsum([len(r) for r in rows])
+    g = inputs.Hypergraph(n, off.astype(np.int32), np.concatenate(rows).astype(np.int32), None, None)
+    check_level(torch, g, 0, pi=pi)
+    check_level(torch, g, 2, pi=pi)
