@@ -45,6 +45,7 @@ static double run_group(const hp_instance *inst, const std::vector<int32_t> &ids
     auto work = [&](int w) {
         cudaSetDevice(dev);
         t_plain_launches = true;
+        t_one_stream = true;
         for (;;) {
             const size_t k = next.fetch_add(1);
             if (k >= ids.size()) break;

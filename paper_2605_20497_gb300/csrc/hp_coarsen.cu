@@ -1065,19 +1065,22 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
     // tier, the dense tier and the hub tier each on a side stream, tier B on
     // the main one; tier C (overflows of B and the hubs) waits for the hubs,
     // and the global tier (whose error list reuses the warp list) for all
-    cudaStream_t sw = W.side[0], sd = W.side[1], sh = W.side[2];
+    const bool one = t_one_stream;
+    cudaStream_t sw = one ? s : W.side[0], sd = one ? s : W.side[1], sh = one ? s : W.side[2];
+    auto record = [&](int k, cudaStream_t x) { if (!one) HPC(cudaEventRecord(W.ev[k], x)); };
+    auto wait = [&](cudaStream_t x, int k) { if (!one) HPC(cudaStreamWaitEvent(x, W.ev[k], 0)); };
     const bool dense = R.dense_bound != 0x7fffffff, hashed = R.dense_bound != 0;
-    HPC(cudaEventRecord(W.ev[0], s));
-    HPC(cudaStreamWaitEvent(sw, W.ev[0], 0));
-    if (dense) HPC(cudaStreamWaitEvent(sd, W.ev[0], 0));
-    if (hashed) HPC(cudaStreamWaitEvent(sh, W.ev[0], 0));
+    record(0, s);
+    wait(sw, 0);
+    if (dense) wait(sd, 0);
+    if (hashed) wait(sh, 0);
     {
         size_t sm = (size_t)wcap * 12 * (WP_T / 32);
         int occ = prepare_kernel((const void *)k_propose_warp<PIMAX>, WP_T, sm);
         int grid = (int)std::min<int64_t>(cdiv(C.n, WP_T / 32), (int64_t)sms * occ);
         launch_k(k_propose_warp<PIMAX>, std::max(grid, 1), WP_T, sm, sw, C, W.lW, W.cnt + 0, wcap);
         HP_LAUNCH_CHECK();
-        HPC(cudaEventRecord(W.ev[1], sw));
+        record(1, sw);
     }
     if (dense) {
         // hubs first; the other nodes by CTAs of 256 threads, of 1024 where
@@ -1100,7 +1103,7 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
             else
                 run(k_propose_dense<PIMAX, 1024>, 1024, sd, W.lD, W.cnt + 6);
         }
-        HPC(cudaEventRecord(W.ev[2], sd));
+        record(2, sd);
     }
     if (hashed) {
         size_t sm = hash_smem(capB, true);
@@ -1108,13 +1111,13 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
         launch_k(k_propose_smem<PIMAX, 1024, true>, std::max(1, std::min<int>(C.n, sms * occ_h)), 1024, sm, sh, C, W.lH,
                  W.cnt + 5, capB, limB, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
-        HPC(cudaEventRecord(W.ev[3], sh));
+        record(3, sh);
         sm = hash_smem(capB, false);
         int occ = prepare_kernel((const void *)k_propose_smem<PIMAX, PB, false>, PB, sm);
         launch_k(k_propose_smem<PIMAX, PB, false>, std::max(1, std::min<int>(C.n, sms * occ)), PB, sm, s,
             C, W.lB, W.cnt + 1, capB, limB, W.lC, W.cnt + 2);
         HP_LAUNCH_CHECK();
-        HPC(cudaStreamWaitEvent(s, W.ev[3], 0));
+        wait(s, 3);
         // nodes whose neighbourhood outgrew the first table (the bound can be far above the truth)
         sm = hash_smem(capC, true);
         occ = prepare_kernel((const void *)k_propose_smem<PIMAX, 1024, true>, 1024, sm);
@@ -1122,8 +1125,8 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
             C, W.lC, W.cnt + 2, capC, capC * 3 / 4, W.lG, W.cnt + 3);
         HP_LAUNCH_CHECK();
     }
-    HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
-    if (dense) HPC(cudaStreamWaitEvent(s, W.ev[2], 0));
+    wait(s, 1);
+    if (dense) wait(s, 2);
     if (hashed) {
         launch_k(k_propose_global<PIMAX>, W.gnb, PT, 0, s, C, W.lG, W.cnt + 3, W.gcap, W.gkeys, W.geta, W.ginter, W.gslots,
                                                       W.lW, W.cnt + 4);
@@ -1527,8 +1530,10 @@ CoarsenWs *coarsen_workspace(int32_t n, int32_t e, const Params &P, Arena &A) {
 
 static CoarsenWs *coarsen_workspace_body(CoarsenWs *W, int32_t n, int32_t e, const Params &P, Arena &A) {
     cudaStream_t s = A.stream();
-    for (cudaStream_t &x : W->side) HPC(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
-    for (cudaEvent_t &x : W->ev) HPC(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    if (!t_one_stream) {
+        for (cudaStream_t &x : W->side) HPC(cudaStreamCreateWithFlags(&x, cudaStreamNonBlocking));
+        for (cudaEvent_t &x : W->ev) HPC(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    }
     const int32_t pi = P.o.pi, K = P.o.learned_k > 0 ? P.o.learned_k : pi;
     W->cn = n;
     W->ce = e;

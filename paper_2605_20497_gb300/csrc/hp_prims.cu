@@ -160,6 +160,7 @@ int prepare_kernel(const void *func, int block, size_t smem) {
 }
 
 thread_local bool t_plain_launches = false;
+thread_local bool t_one_stream = false;
 
 bool pdl_enabled() {
     static const bool on = [] {

@@ -2918,8 +2918,10 @@ LevelWs *refine_workspace(int32_t n, int64_t np, int32_t e, int32_t nparts, int3
 static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t e, int32_t nparts, int32_t max_e,
                                       const Params &P, Arena &A) {
     cudaStream_t s = A.stream();
-    for (cudaStream_t *x : {&W->side, &W->side2}) HPC(cudaStreamCreateWithFlags(x, cudaStreamNonBlocking));
-    for (cudaEvent_t &x : W->ev) HPC(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    if (!t_one_stream) {
+        for (cudaStream_t *x : {&W->side, &W->side2}) HPC(cudaStreamCreateWithFlags(x, cudaStreamNonBlocking));
+        for (cudaEvent_t &x : W->ev) HPC(cudaEventCreateWithFlags(&x, cudaEventDisableTiming));
+    }
     W->cn = n;
     W->cnp = np;
     W->ce = e;
@@ -3096,6 +3098,22 @@ static bool bits_pay(const Level &L, const LevelWs &W) {
     return W.cut_lam >= W.cuts * 4 * W.wq;
 }
 
+// Side streams of the gain kernels: fork_side lets one start after the work
+// queued on s, end_side marks the end of its work, join_side lets s wait for
+// that (all on s itself where the thread keeps to one stream).
+static cudaStream_t fork_side(const LevelWs &W, cudaStream_t s, cudaStream_t side) {
+    if (t_one_stream) return s;
+    HPC(cudaEventRecord(W.ev[0], s));
+    HPC(cudaStreamWaitEvent(side, W.ev[0], 0));
+    return side;
+}
+static void end_side(const LevelWs &W, cudaStream_t side, int k) {
+    if (!t_one_stream) HPC(cudaEventRecord(W.ev[k], side));
+}
+static void join_side(const LevelWs &W, cudaStream_t s, int k) {
+    if (!t_one_stream) HPC(cudaStreamWaitEvent(s, W.ev[k], 0));
+}
+
 // ---------------------------------------------------------------- gains by part
 // The list form for up to PB_PARTS parts and weight sums below 2^32: the
 // node's conn(v, p) in 32-bit counters indexed by part, so no table can
@@ -3217,43 +3235,41 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : NW * 32)
 // the three node classes side by side
 static void gains_parts(const GainArgs &G, const LevelWs &W, const int32_t *cnt, int32_t n, cudaStream_t s) {
     const size_t sm = 4 * (size_t)(cdiv(W.nparts, 32) * 32 + 32);
-    HPC(cudaEventRecord(W.ev[0], s));
-    for (int q = 0; q < 2; q++) HPC(cudaStreamWaitEvent(q ? W.side2 : W.side, W.ev[0], 0));
+    const cudaStream_t sh = fork_side(W, s, W.side), sm2 = fork_side(W, s, W.side2);
     const int occ_h = prepare_kernel((const void *)k_gains_parts<32>, 1024, sm);
-    launch_k(k_gains_parts<32>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 1024, sm, W.side, G, W.nparts, W.hubs,
+    launch_k(k_gains_parts<32>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 1024, sm, sh, G, W.nparts, W.hubs,
              cnt + C_HUB);
     HP_LAUNCH_CHECK();
-    HPC(cudaEventRecord(W.ev[1], W.side));
+    end_side(W, sh, 1);
     const int occ_m = prepare_kernel((const void *)k_gains_parts<8>, 256, sm);
-    launch_k(k_gains_parts<8>, std::max(1, std::min<int>(n, num_sms() * occ_m)), 256, sm, W.side2, G, W.nparts, W.cl,
+    launch_k(k_gains_parts<8>, std::max(1, std::min<int>(n, num_sms() * occ_m)), 256, sm, sm2, G, W.nparts, W.cl,
              cnt + C_CAND);
     HP_LAUNCH_CHECK();
-    HPC(cudaEventRecord(W.ev[2], W.side2));
+    end_side(W, sm2, 2);
     const int occ = prepare_kernel((const void *)k_gains_parts<1>, 256, 8 * sm);
     launch_k(k_gains_parts<1>, std::max(1, std::min<int>((int)cdiv(n, 8), num_sms() * occ)), 256, 8 * sm, s, G, W.nparts,
              W.cw, cnt + C_CW);
     HP_LAUNCH_CHECK();
-    HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
-    HPC(cudaStreamWaitEvent(s, W.ev[2], 0));
+    join_side(W, s, 1);
+    join_side(W, s, 2);
 }
 
 template <int WQ>
 static void gains_bits(const GainArgs &G, const LevelWs &W, const int32_t *cnt, int32_t n, cudaStream_t s) {
     // hub nodes on the side stream, beside the two lists of smaller ones
-    HPC(cudaEventRecord(W.ev[0], s));
-    HPC(cudaStreamWaitEvent(W.side, W.ev[0], 0));
+    const cudaStream_t sh = fork_side(W, s, W.side);
     const int occ_h = prepare_kernel((const void *)k_gains_bits<WQ, 16>, 512, 0);
-    launch_k(k_gains_bits<WQ, 16>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 512, 0, W.side, G, W.bits, W.nparts,
+    launch_k(k_gains_bits<WQ, 16>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 512, 0, sh, G, W.bits, W.nparts,
              W.hubs, cnt + C_HUB);
     HP_LAUNCH_CHECK();
-    HPC(cudaEventRecord(W.ev[1], W.side));
+    end_side(W, sh, 1);
     const int occ = prepare_kernel((const void *)k_gains_bits<WQ, 4>, 128, 0);
     const int grid = std::max(1, std::min<int>(n, num_sms() * occ));
     launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cw, cnt + C_CW);
     HP_LAUNCH_CHECK();
     launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cl, cnt + C_CAND);
     HP_LAUNCH_CHECK();
-    HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
+    join_side(W, s, 1);
 }
 
 // One repetition; returns the number of moves applied.
@@ -3346,13 +3362,12 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         {
             // hub nodes on the side stream, beside the warp and CTA tiers (disjoint
             // node lists; all append to the same move and overflow lists by atomics)
-            HPC(cudaEventRecord(W.ev[0], s));
-            HPC(cudaStreamWaitEvent(W.side, W.ev[0], 0));
+            const cudaStream_t sh = fork_side(W, s, W.side);
             const int occ_h = prepare_kernel((const void *)k_gains_smem<1024>, 1024, gsm);
-            launch_k(k_gains_smem<1024>, num_sms() * std::max(occ_h, 1), 1024, gsm, W.side, G, W.hubs, cnt + C_HUB, gcap_smem,
+            launch_k(k_gains_smem<1024>, num_sms() * std::max(occ_h, 1), 1024, gsm, sh, G, W.hubs, cnt + C_HUB, gcap_smem,
                      W.ovf, cnt + C_OVF);
             HP_LAUNCH_CHECK();
-            HPC(cudaEventRecord(W.ev[1], W.side));
+            end_side(W, sh, 1);
         }
         {
             const uint32_t wlimit = P.o.debug_table_cap > 0 ? std::min<uint32_t>(GW_SLOTS * 3 / 4, P.o.debug_table_cap / 2)
@@ -3367,7 +3382,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
             int grid = std::max(1, std::min<int>(n, num_sms() * occ));
             launch_k(k_gains_smem<GN_T>, grid, GN_T, gsm, s, G, W.cl, cnt + C_CAND, gcap_smem, W.ovf, cnt + C_OVF);
             HP_LAUNCH_CHECK();
-            HPC(cudaStreamWaitEvent(s, W.ev[1], 0));
+            join_side(W, s, 1);
             launch_k(k_gains_global, W.gnb, GN_T, 0, s, G, W.ovf, cnt + C_OVF, W.gcap, W.gk, W.gc, W.cl, cnt + C_BAD);
             HP_LAUNCH_CHECK();
         }
