@@ -219,7 +219,8 @@ static hp_status run(const int32_t *pins, const int32_t *offsets, int32_t e, int
             // the coarser level is no longer needed
             Level &c = lv[l + 1];
             for (int32_t *p : {c.off, c.pin, c.pedge, c.nsrc, c.size, c.ioff, c.inc, c.inode, c.nin, c.gamma, c.nbnd})
-                A.release(p);
+                A.release(p);   // (nothing for the arrays of a slab)
+            A.release(c.slab);
             c = Level();
         }
         PlainLaunchScope plain(g.n > PDL_MAX_N);

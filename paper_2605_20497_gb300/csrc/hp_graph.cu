@@ -286,6 +286,7 @@ __device__ __forceinline__ int32_t pin_keep(const int32_t *pin, const int32_t *p
 // Levels of up to CONTRACT_CLUSTER_NP pins run the steps in one launch on one
 // thread-block cluster; larger ones as a few grid-wide kernels.
 constexpr int64_t CONTRACT_CLUSTER_NP = int64_t(1) << 15;
+constexpr int64_t SLAB_NP = int64_t(1) << 22;   // at most 100 MB a level
 
 struct ContractArgs {
     Level L;                 // the fine level
@@ -487,24 +488,51 @@ bool contract_level(const Level &L, const int32_t *mate, LevelBox *box, LevelBox
     X.L = L;
     X.mate = mate;
     X.box = box;
-    X.isrep = A.get<int32_t>(n);
-    X.cid = A.get<int32_t>(n);
-    X.kflag = A.get<int64_t>(np);
-    X.kscan = A.get<int64_t>(np + 1);
-    X.rep_of = A.get<int32_t>(n);
-    X.ccnt = A.get<int32_t>(n);
-    // the coarse level at the fine level's sizes (nodes and pins only shrink)
+    // The coarse level at the fine level's sizes (nodes and pins only shrink).
+    // The scratch is one block, and so is a coarse level of up to SLAB_NP pins:
+    // a chain of small levels otherwise spends 34 allocator calls on each, which
+    // the workers of a batch contend for.  Larger levels are separate
+    // blocks, some of which are given back before the refinement.
     Level K;
-    K.size = A.get<int32_t>(n);
-    K.nbnd = A.get<int32_t>(n);
-    K.off = A.get<int32_t>(e + 1);
-    K.nsrc = A.get<int32_t>(e);
-    K.pin = A.get<int32_t>(np);
-    K.pedge = A.get<int32_t>(np);
-    K.ioff = A.get<int32_t>(n + 1);
-    K.nin = A.get<int32_t>(n);
-    K.inc = A.get<int32_t>(np);
-    K.inode = A.get<int32_t>(np);
+    void *scratch = nullptr;
+    const bool slab = np <= SLAB_NP;
+    for (int pass = 0; pass < 2; pass++) {
+        Carve S, T;
+        if (pass == 1) S.at = static_cast<unsigned char *>(scratch);
+        X.isrep = S.take<int32_t>(n);
+        X.cid = S.take<int32_t>(n);
+        X.kflag = S.take<int64_t>(np);
+        X.kscan = S.take<int64_t>(np + 1);
+        X.rep_of = S.take<int32_t>(n);
+        X.ccnt = S.take<int32_t>(n);
+        if (pass == 0) scratch = A.raw(S.size);
+        if (!slab) continue;
+        if (pass == 1) T.at = static_cast<unsigned char *>(K.slab);
+        (void)T.take<unsigned char>(1);   // no array starts the block: releasing an array releases nothing
+        K.size = T.take<int32_t>(n);
+        K.nbnd = T.take<int32_t>(n);
+        K.off = T.take<int32_t>(e + 1);
+        K.nsrc = T.take<int32_t>(e);
+        K.pin = T.take<int32_t>(np);
+        K.pedge = T.take<int32_t>(np);
+        K.ioff = T.take<int32_t>(n + 1);
+        K.nin = T.take<int32_t>(n);
+        K.inc = T.take<int32_t>(np);
+        K.inode = T.take<int32_t>(np);
+        if (pass == 0) K.slab = A.raw(T.size);
+    }
+    if (!slab) {
+        K.size = A.get<int32_t>(n);
+        K.nbnd = A.get<int32_t>(n);
+        K.off = A.get<int32_t>(e + 1);
+        K.nsrc = A.get<int32_t>(e);
+        K.pin = A.get<int32_t>(np);
+        K.pedge = A.get<int32_t>(np);
+        K.ioff = A.get<int32_t>(n + 1);
+        K.nin = A.get<int32_t>(n);
+        K.inc = A.get<int32_t>(np);
+        K.inode = A.get<int32_t>(np);
+    }
     X.C = K;
     X.gamma = A.get<int32_t>(n);
     if (np <= CONTRACT_CLUSTER_NP && np > 0 && n > 0) {
@@ -525,12 +553,12 @@ bool contract_level(const Level &L, const int32_t *mate, LevelBox *box, LevelBox
         HP_LAUNCH_CHECK();
     }
     fetch_bytes(hb, box, sizeof(LevelBox), s);
-    for (void *p : {(void *)X.isrep, (void *)X.cid, (void *)X.kflag, (void *)X.kscan, (void *)X.rep_of, (void *)X.ccnt})
-        A.release(p);
+    A.release(scratch);
     if (hb->pairs + hb->iso == 0) {
         for (void *p : {(void *)K.size, (void *)K.nbnd, (void *)K.off, (void *)K.nsrc, (void *)K.pin, (void *)K.pedge,
                         (void *)K.ioff, (void *)K.nin, (void *)K.inc, (void *)K.inode, (void *)X.gamma})
-            A.release(p);
+            A.release(p);   // (nothing for the arrays of a slab)
+        A.release(K.slab);
         return false;
     }
     const_cast<Level &>(L).gamma = X.gamma;

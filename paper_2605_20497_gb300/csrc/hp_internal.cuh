@@ -377,6 +377,19 @@ struct Level {
     int32_t *nin = nullptr;    // [n] |in(v)|
     int32_t *gamma = nullptr;  // [n] node -> node of the next level
     int32_t *nbnd = nullptr;   // [n] upper bound on |N(v)| (neighbour table sizing)
+    void *slab = nullptr;      // the one block all of these lie in, on small levels
+};
+
+// Consecutive arrays in one block, each aligned to 256 bytes: sizes are added
+// up by a first pass over `take` with no block, addresses given by a second.
+struct Carve {
+    unsigned char *at = nullptr;
+    size_t size = 0;
+    template <class T> T *take(size_t n) {
+        const size_t b = (n * sizeof(T) + 255) & ~size_t(255), o = size;
+        size += b;
+        return at ? reinterpret_cast<T *>(at + o) : nullptr;
+    }
 };
 
 struct Params {
