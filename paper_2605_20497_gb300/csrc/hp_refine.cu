@@ -913,12 +913,13 @@ __global__ void __launch_bounds__(PB_T) k_part_bits(const int32_t *off, Plist PL
     }
 }
 
-// One node per CTA of NW warps, the warps taking its cut hyperedges in chunks
-// of 32.  The counters are 32 bits wide: the host takes this path only when
+// One node per CTA of NW warps (from list and then list2, which may be none),
+// the warps taking its cut hyperedges in chunks of 32.  The counters are 32 bits wide: the host takes this path only when
 // the sum of all weights is below 2^32.
 template <int WQ, int NW>
 __global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 *bits, int32_t nparts,
-                                                        const int32_t *list, const int32_t *count_p) {
+                                                        const int32_t *list, const int32_t *count_p,
+                                                        const int32_t *list2, const int32_t *count2_p) {
     HP_KERNEL_ENTER();
     __shared__ uint32_t s_conn[WQ * 128];
     __shared__ long long s_rg[NW];
@@ -926,11 +927,11 @@ __global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const uint32_t my = 1u << lane;
-    const int32_t count = *count_p;
+    const int32_t n1 = *count_p, count = n1 + (list2 ? *count2_p : 0);
     for (int i = threadIdx.x; i < WQ * 128; i += NW * 32) s_conn[i] = 0;
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
-        const int32_t v = list[k], s = G.rho[v];
+        const int32_t v = k < n1 ? list[k] : list2[k - n1], s = G.rho[v];
         const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
         uint32_t acc[WQ * 4];
 #pragma unroll
@@ -3258,16 +3259,18 @@ template <int WQ>
 static void gains_bits(const GainArgs &G, const LevelWs &W, const int32_t *cnt, int32_t n, cudaStream_t s) {
     // hub nodes on the side stream, beside the two lists of smaller ones
     const cudaStream_t sh = fork_side(W, s, W.side);
-    const int occ_h = prepare_kernel((const void *)k_gains_bits<WQ, 16>, 512, 0);
-    launch_k(k_gains_bits<WQ, 16>, std::max(1, std::min<int>(n, num_sms() * occ_h)), 512, 0, sh, G, W.bits, W.nparts,
-             W.hubs, cnt + C_HUB);
+    // (16 warps a hub while the registers let two CTAs of them on an SM: wider
+    // rows hold 74 a thread, and one such CTA an SM took 130.7 instead of 126.4
+    // ms on the 16,384-node random net)
+    constexpr int HW = WQ <= 2 ? 16 : 8;
+    const int occ_h = prepare_kernel((const void *)k_gains_bits<WQ, HW>, HW * 32, 0);
+    launch_k(k_gains_bits<WQ, HW>, std::max(1, std::min<int>(n, num_sms() * occ_h)), HW * 32, 0, sh, G, W.bits, W.nparts,
+             W.hubs, cnt + C_HUB, nullptr, nullptr);
     HP_LAUNCH_CHECK();
     end_side(W, sh, 1);
     const int occ = prepare_kernel((const void *)k_gains_bits<WQ, 4>, 128, 0);
     const int grid = std::max(1, std::min<int>(n, num_sms() * occ));
-    launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cw, cnt + C_CW);
-    HP_LAUNCH_CHECK();
-    launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cl, cnt + C_CAND);
+    launch_k(k_gains_bits<WQ, 4>, grid, 128, 0, s, G, W.bits, W.nparts, W.cl, cnt + C_CAND, W.cw, cnt + C_CW);
     HP_LAUNCH_CHECK();
     join_side(W, s, 1);
 }
@@ -3572,7 +3575,8 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
             launch_k(k_inseq_small, std::max(grid, 1), IS_T, sm, s, Z, W.touched, cnt + C_TOUCH, emax, cnt + C_MOVES, lo);
             HP_LAUNCH_CHECK();
         };
-        if (W.small_max > MID_SPLIT) {
+        // (two launches on larger levels: the smaller buffers let more warps in)
+        if (W.small_max > MID_SPLIT && !(small_level && nparts <= PB_PARTS)) {
             inseq_mid(0, MID_SPLIT);
             inseq_mid(MID_SPLIT, W.small_max);
         } else {
