@@ -112,6 +112,7 @@ static hp_status run(const int32_t *pins, const int32_t *offsets, int32_t e, int
     P.omega = omega;
     P.delta = delta;
     P.seed = seed;
+    P.unit_sizes = true;
     if (opt) P.o = *opt;
     else hp_default_options(&P.o);
     if (n < 0 || e < 0 || omega < 1 || delta < 0 || !offsets || (n > 0 && !part_out) || !options_ok(P.o) ||

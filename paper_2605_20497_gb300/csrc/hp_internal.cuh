@@ -398,6 +398,7 @@ struct Params {
     hp_options o;
     int64_t wsum = 0;   // sum of hyperedge weights (bounds any gain)
     int32_t wmax = 65536;   // no weight is above
+    bool unit_sizes = false;   // level 0 has unit sizes: a node of level l has at most 2^l
 };
 
 // graph construction (hp_graph.cu)
