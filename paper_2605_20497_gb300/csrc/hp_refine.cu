@@ -166,11 +166,31 @@ __host__ __device__ inline size_t plist_parts_smem(int32_t nparts) {
     const size_t words = (size_t)(nparts + 31) / 32;
     return 4 * ((PP_T / 32) * (words * 32 + 32) + words * 32);
 }
+// The applied moves of the repetition before: node v moved when its sequence
+// position lies below *applied, from the part of its move.
+struct Applied {
+    const int32_t *mvpos, *seqmove, *src, *applied;
+    __device__ __forceinline__ int32_t old_part(int32_t v, int32_t now, int32_t len) const {
+        const int32_t k = mvpos[v];
+        return k >= 0 && k < len ? src[seqmove[k]] : now;
+    }
+};
+// UPDATE: the list holds the hyperedges that may have a pin among the applied
+// moves (*count_p of them); the ones that do take their old contributions to
+// D(p) and saving(v) back, read off their old pins list, before they are
+// rebuilt.
+template <bool UPDATE>
 __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const int32_t *pin, const int32_t *nsrc,
                                                       const int32_t *w, const int32_t *rho, const int32_t *list,
-                                                      int32_t count, int32_t nparts, Plist PL, int32_t *D,
-                                                      long long *saving) {
+                                                      int32_t count, const int32_t *count_p, Applied M, int32_t nparts,
+                                                      Plist PL, int32_t *D, long long *saving) {
     HP_KERNEL_ENTER();
+    int32_t len = 0;
+    if (UPDATE) {
+        count = *count_p;
+        len = *M.applied;
+        if ((int64_t)blockIdx.x * (PP_T / 32) >= count) return;
+    }
     extern __shared__ __align__(16) uint32_t smw[];
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nwb = PP_T / 32;
@@ -195,6 +215,32 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
 #pragma unroll
             for (int k = 0; k < R; k++) pp[k] = vv[k] >= 0 ? rho[vv[k]] : 0;
         };
+        if (UPDATE) {
+            bool moved = false;
+            for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
+                load(j0);
+#pragma unroll
+                for (int k = 0; k < R; k++) moved |= vv[k] >= 0 && M.old_part(vv[k], pp[k], len) != pp[k];
+            }
+            if (!__any_sync(FULL, moved)) continue;
+            const int32_t lam = PL.lam[e];
+            for (int32_t x2 = lane; x2 < lam; x2 += 32) {
+                const int32_t p = PL.p[a + x2], ci = PL.cin[a + x2];
+                cnt[p] = (uint32_t)PL.cnt[a + x2];
+                if (ci > 0) atomicAdd(&s_d[p], 0xffffffffu);
+            }
+            __syncwarp();
+            for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
+                if (b - a > 32 * R) load(j0);
+#pragma unroll
+                for (int k = 0; k < R; k++)
+                    if (vv[k] >= 0 && cnt[M.old_part(vv[k], pp[k], len)] == 1u)
+                        atomicAdd((unsigned long long *)&saving[vv[k]], 0ull - we);
+            }
+            __syncwarp();
+            for (int32_t x2 = lane; x2 < lam; x2 += 32) cnt[PL.p[a + x2]] = 0;
+            __syncwarp();
+        }
         for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
             load(j0);
 #pragma unroll
@@ -1200,6 +1246,127 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
     }
 }
 
+// After a repetition that applied few moves, the next one updates the
+// partition-dependent state where they changed it instead of rebuilding it:
+// |p| and the single-pin hyperedges' share of D(p) per move, and the pins
+// list, D(p) and saving(v) of the hyperedges with a moved pin.  All are sums
+// of integers, so the result is the rebuilt one.  406 rebuilds on the 1M
+// Gaussian net (88 moves applied in each on average) took 63 and 36 ms in the
+// pins-list kernels; 69 rebuilds and 337 updates take 4 + 10 and 6 + 3 ms, and
+// 16 to list the hyperedges: 719 -> 651 ms a call.
+__global__ void k_move_nodes(Applied M, const int32_t *node, const int32_t *dst, const int32_t *size,
+                             const int32_t *singin, long long *psize, int32_t *D0, int32_t *upd) {
+    HP_KERNEL_ENTER();
+    const int32_t len = *M.applied;
+    if (blockIdx.x == 0 && threadIdx.x < 2) upd[threadIdx.x] = 0;
+    GRID_STRIDE(k, (int64_t)len) {
+        const int32_t i = M.seqmove[k], v = node[i], ps = M.src[i], pd = dst[i];
+        const unsigned long long sz = (unsigned long long)size[v];
+        atomicAdd((unsigned long long *)&psize[ps], 0ull - sz);
+        atomicAdd((unsigned long long *)&psize[pd], sz);
+        if (singin[v]) {
+            atomicAdd(&D0[ps], -singin[v]);
+            atomicAdd(&D0[pd], singin[v]);
+        }
+    }
+}
+// the hyperedges of the moved nodes (a warp per node), each once: `mark` holds
+// the number of the last update that listed a hyperedge
+__global__ void k_moved_edges(Applied M, const int32_t *node, const int32_t *off, const int32_t *ioff, const int32_t *inc,
+                              int32_t epoch, int32_t *mark, int32_t *tiny, int32_t *mid, int32_t *upd) {
+    HP_KERNEL_ENTER();
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const uint32_t lt = (1u << lane) - 1u;
+    const int32_t len = *M.applied;
+    for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < len;
+         k += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int32_t v = node[M.seqmove[k]], i1 = ioff[v + 1];
+        for (int32_t t0 = ioff[v]; t0 < i1; t0 += 32) {
+            int cls = -1;
+            int32_t e = 0;
+            if (t0 + lane < i1) {
+                e = inc[t0 + lane];
+                const int32_t sz = off[e + 1] - off[e];
+                if (sz >= 2 && atomicExch(&mark[e], epoch) != epoch) cls = sz <= TINY_E ? 0 : 1;
+            }
+#pragma unroll
+            for (int c = 0; c < 2; c++) {
+                const unsigned m = __ballot_sync(FULL, cls == c);
+                if (!m) continue;
+                int32_t at = 0;
+                if (lane == 0) at = atomicAdd(&upd[c], __popc(m));
+                at = __shfl_sync(FULL, at, 0);
+                if (cls == c) (c ? mid : tiny)[at + __popc(m & lt)] = e;
+            }
+        }
+    }
+}
+// hyperedges of 2..TINY_E pins from the list, one thread each
+__global__ void k_plist_tiny_update(const int32_t *off, const int32_t *pin, const int32_t *nsrc, const int32_t *w,
+                                    const int32_t *rho, const int32_t *list, const int32_t *count_p, Applied M, Plist PL,
+                                    int32_t *D, long long *saving) {
+    HP_KERNEL_ENTER();
+    const int32_t count = *count_p, len = *M.applied;
+    GRID_STRIDE(x, (int64_t)count) {
+        const int32_t e = list[x], a = off[e], sz = off[e + 1] - a;
+        int32_t vv[TINY_E], np[TINY_E], op[TINY_E];
+        bool moved = false;
+#pragma unroll
+        for (int j = 0; j < TINY_E; j++) {
+            vv[j] = np[j] = op[j] = -1;
+            if (j < sz) {
+                vv[j] = pin[a + j];
+                np[j] = rho[vv[j]];
+                op[j] = M.old_part(vv[j], np[j], len);
+                moved |= op[j] != np[j];
+            }
+        }
+        if (!moved) continue;
+        const int32_t dst0 = nsrc[e];
+        const long long we = w[e];
+        int32_t lam = 0;
+#pragma unroll
+        for (int j = 0; j < TINY_E; j++) {
+            if (j >= sz) break;
+            int32_t co = 0, cn = 0, ci = 0, rank = 0;   // pins of j's old and new part; inbound ones; smaller new parts
+            bool nfirst = true, odst = j >= dst0, ndst = j >= dst0;   // first pin of its new part; first destination of its parts
+#pragma unroll
+            for (int k = 0; k < TINY_E; k++) {
+                if (k >= sz) break;
+                co += op[k] == op[j];
+                if (np[k] == np[j]) {
+                    cn++;
+                    ci += k >= dst0;
+                    if (k < j) nfirst = false;
+                    if (k < j && k >= dst0) ndst = false;
+                }
+                if (op[k] == op[j] && k < j && k >= dst0) odst = false;
+                if (np[k] < np[j]) {
+                    bool first = true;
+#pragma unroll
+                    for (int q = 0; q < TINY_E; q++)
+                        if (q < k && np[q] == np[k]) first = false;
+                    rank += first;
+                }
+            }
+            const long long ds = (cn == 1 ? we : 0) - (co == 1 ? we : 0);
+            if (ds) atomicAdd((unsigned long long *)&saving[vv[j]], (unsigned long long)ds);
+            if (odst != ndst || op[j] != np[j]) {
+                if (odst) atomicAdd(&D[op[j]], -1);
+                if (ndst) atomicAdd(&D[np[j]], 1);
+            }
+            if (nfirst) {
+                PL.p[a + rank] = np[j];
+                PL.cnt[a + rank] = cn;
+                PL.cin[a + rank] = ci;
+                lam++;
+            }
+        }
+        PL.lam[e] = lam;
+    }
+}
+
 // counters of one repetition (device)
 enum { C_CAND, C_MOVES, C_OVF, C_BAD, C_NH, C_BAD0, C_APPLIED, C_NV, C_HUB, C_CW, C_TOUCH, C_PAD,
        C_ACC,          // three 64-bit byte counters (even index: 8-byte aligned), see k_cut_bits
@@ -1212,6 +1379,7 @@ constexpr int SMALLM = 6144, SEQ_T = 1024;
 // refinement levels of at most this many nodes run their repetitions on the
 // cluster kernels with one read-back each (every move count fits them)
 constexpr int32_t SMALL_LEVEL = 32768;
+constexpr int64_t UPDATE_NP = int64_t(1) << 19;   // pins of a level from which on few moves update its state
 
 #define STRIDE(i, n, t0, nt) for (int64_t i = (t0); i < (int64_t)(n); i += (nt))
 #define G_T0 (blockIdx.x * (int64_t)blockDim.x + threadIdx.x)
@@ -1233,8 +1401,9 @@ struct RepArrays {
 __device__ __forceinline__ int64_t rep_zero_span(const RepArrays &R) {
     return max(max((int64_t)R.n, (int64_t)R.nparts + 1), max((int64_t)C_N, (int64_t)R.rounds + 1));
 }
-// keep: the partition is the one of the previous repetition (it applied
-// nothing), so D(p), |p| and saving(v) are still valid
+// keep 1: the partition is the one of the previous repetition (it applied
+// nothing), so D(p), |p|, saving(v) and the cut lists are still valid; keep 2:
+// the first three have been updated
 __global__ void k_rep_zero(RepArrays R, int keep) {
     HP_KERNEL_ENTER();
     GRID_STRIDE(i, rep_zero_span(R)) {
@@ -1244,10 +1413,8 @@ __global__ void k_rep_zero(RepArrays R, int keep) {
         }
         if (i <= R.nparts) R.pc[i] = 0;
         if (i < R.n) {
-            if (!keep) {
-                R.saving[i] = 0;
-                R.cutn[i] = 0;
-            }
+            if (!keep) R.saving[i] = 0;
+            if (keep != 1) R.cutn[i] = 0;
             R.pred[i] = -1;
             R.succ[i] = -1;
             R.chain[i] = -1;
@@ -2860,7 +3027,9 @@ struct LevelWs {
     bool bits_valid = false;
     uint4 *bits = nullptr;   // [ce][wq] parts of every cut hyperedge (k_part_bits), or none
     int wq = 0;
-    int32_t *touched;                        // hyperedges of mid with a moved pin
+    int32_t *touched, *ttouched;             // hyperedges of mid (of tiny) with a moved pin
+    int32_t *emark, *upd;                    // [ce] last update that listed a hyperedge; its two counts
+    int32_t epoch = 0;
     Moves M, S;
     uint64_t *keys;
     uint32_t *idx;
@@ -2963,6 +3132,10 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->tiny = A.get<int32_t>(e);
     W->mid = A.get<int32_t>(e);
     W->touched = A.get<int32_t>(e);
+    W->ttouched = A.get<int32_t>(e);
+    W->emark = A.get<int32_t>(std::max(e, 1));
+    W->upd = A.get<int32_t>(2);
+    HPC(cudaMemsetAsync(W->emark, 0, sizeof(int32_t) * std::max(e, 1), s));
     for (Moves *m : {&W->M, &W->S}) {
         m->node = A.get<int32_t>(n);
         m->src = A.get<int32_t>(n);
@@ -3037,7 +3210,7 @@ void refine_workspace_free(LevelWs *W, Arena &A) {
     for (void *p : std::initializer_list<void *>{
              W->big, W->wns, W->singin, W->PL.p, W->PL.cnt, W->PL.cin, W->PL.lam, W->R.cnt, W->R.linked,
              W->R.D0, W->R.psize, W->R.saving, W->R.pc, W->R.pred, W->R.succ, W->R.chain, W->R.mvpos, W->R.cgain,
-             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->M.node, W->M.src, W->M.dst, W->M.gain,
+             W->R.gseq, W->R.acc0, W->R.dDs, W->R.dDd, W->R.viol, W->cl, W->hubs, W->cw, W->cutbits, W->cut, W->R.cutn, W->tiny, W->mid, W->touched, W->ttouched, W->emark, W->upd, W->M.node, W->M.src, W->M.dst, W->M.gain,
              W->S.node, W->S.src, W->S.dst, W->S.gain, W->keys, W->idx, W->msz, W->mni, W->first, W->choice, W->accnode, W->pen,
              W->minpen, W->acc1, W->acc2, W->pos, W->clen, W->lens, W->starts, W->cstart, W->seqmove, W->heads, W->hkeys,
              W->vkey, W->vidx, W->vsz, W->vdd, W->gsz, W->gdd, W->esz, W->edd, W->vhead, W->bgain, W->lvl, W->pmark, W->pnew, W->ovf, W->gk, W->gc, W->ptab, W->ibuf, W->bits})
@@ -3279,18 +3452,42 @@ static void gains_bits(const GainArgs &G, const LevelWs &W, const int32_t *cnt, 
 // reuse: rho is unchanged since the previous repetition of this level (which
 // applied nothing), so its pins lists, D(p), |p|, saving(v) and cut lists,
 // all functions of rho, are reused instead of rebuilt
+// update: the previous repetition of this level applied that many moves, and
+// the first four of these are updated for them instead of rebuilt
 static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_t *rho, int second_half, LevelWs &W,
-                       Arena &A, uint32_t *err_dev, const RepDebug *dbg, bool reuse = false) {
+                       Arena &A, uint32_t *err_dev, const RepDebug *dbg, bool reuse = false, int32_t update = 0) {
     cudaStream_t s = A.stream();
     const int32_t n = L.n, nparts = W.nparts;
     RepArrays &R = W.R;
     int32_t *cnt = R.cnt;
     const int64_t zspan = std::max<int64_t>(std::max<int64_t>(n, (int64_t)nparts + 1),
                                             std::max<int64_t>((int64_t)C_N, (int64_t)P.o.chain_rounds + 1));
-    launch_k(k_rep_zero, grid_of(zspan, 256), 256, 0, s, R, reuse ? 1 : 0);
+    const Applied moved{R.mvpos, W.seqmove, W.S.src, cnt + C_APPLIED};
+    if (update > 0) {
+        // the previous repetition applied `update` moves
+        launch_k(k_move_nodes, grid_of(update, 256), 256, 0, s, moved, W.S.node, W.S.dst, L.size, W.singin, R.psize, R.D0,
+                 W.upd);
+        HP_LAUNCH_CHECK();
+        launch_k(k_moved_edges, grid_of((int64_t)update * 32, 256), 256, 0, s, moved, W.S.node, L.off, L.ioff, L.inc,
+                 ++W.epoch, W.emark, W.ttouched, W.touched, W.upd);
+        HP_LAUNCH_CHECK();
+        if (W.n_mid > 0) {
+            const size_t sm = plist_parts_smem(nparts);
+            const int occ = prepare_kernel((const void *)k_plist_parts<true>, PP_T, sm);
+            const int grid = (int)std::min<int64_t>(cdiv(W.n_mid, PP_T / 32), (int64_t)num_sms() * occ);
+            launch_k(k_plist_parts<true>, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.touched, 0, W.upd + 1, moved,
+                     nparts, W.PL, R.D0, R.saving);
+            HP_LAUNCH_CHECK();
+        }
+        if (W.n_tiny > 0) {
+            launch_k(k_plist_tiny_update, std::min(grid_of(W.n_tiny, 128), 8 * num_sms()), 128, 0, s, L.off, L.pin, L.nsrc,
+                     w, rho, W.ttouched, W.upd, moved, W.PL, R.D0, R.saving);
+            HP_LAUNCH_CHECK();
+        }
+    }
+    launch_k(k_rep_zero, grid_of(zspan, 256), 256, 0, s, R, reuse ? 1 : update ? 2 : 0);
     HP_LAUNCH_CHECK();
-    if (!reuse) {
-        W.bits_valid = false;
+    if (!reuse && update == 0) {
         // (a few CTAs an SM: each ends with a pass over the parts; the step call takes any sizes)
         launch_k(k_rep_nodes, std::min(grid_of(n, 256), 4 * num_sms()), 256, 0, s, rho, L.size, W.singin, n, dbg ? RN_PARTS + 1 : nparts,
                  R.psize, R.D0);
@@ -3298,10 +3495,10 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         // pins(p,e), pins_in(p,e), D(p), saving(v)
         if (W.n_mid > 0 && nparts <= PB_PARTS) {
             const size_t sm = plist_parts_smem(nparts);
-            const int occ = prepare_kernel((const void *)k_plist_parts, PP_T, sm);
+            const int occ = prepare_kernel((const void *)k_plist_parts<false>, PP_T, sm);
             const int grid = (int)std::min<int64_t>(cdiv(W.n_mid, PP_T / 32), (int64_t)num_sms() * occ);
-            launch_k(k_plist_parts, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.mid, W.n_mid, nparts, W.PL, R.D0,
-                     R.saving);
+            launch_k(k_plist_parts<false>, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.mid, W.n_mid, nullptr, moved,
+                     nparts, W.PL, R.D0, R.saving);
             HP_LAUNCH_CHECK();
         } else if (W.n_mid > 0) {
             // hyperedges of up to MID_SPLIT pins in small tables (many warps
@@ -3332,6 +3529,9 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
                      W.PL, R.D0, R.saving);
             HP_LAUNCH_CHECK();
         }
+    }
+    if (!reuse) {
+        W.bits_valid = false;
         // moves in isolation (Eq. 13)
         if (L.np > 0) {
             launch_k(k_cut_bits, grid_of(L.e, 256), 256, 0, s, L.off, W.PL.lam, L.e, W.cutbits,
@@ -3682,8 +3882,14 @@ RefineOut refine_level(const Level &L, const int32_t *w, const Params &P, int32_
     const int64_t bytes0 = W->alg_bytes;
     const int32_t half = P.o.theta / 2;
     bool same_rho = false;   // the previous repetition applied nothing
+    int32_t applied = 0;     // moves the previous one applied
     for (int32_t rep = 0; rep < P.o.theta; rep++) {
-        const int32_t k = rep_run(L, w, P, rho, rep >= half, *W, A, err_dev, nullptr, same_rho);
+        // an update touches the moved nodes' hyperedges only; on small levels a
+        // rebuild is as short as the update's four launches
+        const int32_t update = L.np >= UPDATE_NP && W->n_big == 0 && W->nparts <= PB_PARTS && 8 * (int64_t)applied <= L.n
+                                   ? applied : 0;
+        const int32_t k = rep_run(L, w, P, rho, rep >= half, *W, A, err_dev, nullptr, same_rho, update);
+        applied = k;
         same_rho = k == 0;
         out.reps++;
         out.moves += k;

@@ -100,3 +100,33 @@ def test_renumbered_parts(torch, max_levels, omega):
     for k, v in o.stats.items():
         assert r.stats[k] == v, k
     assert [t["moves"] for t in r.trace] == [t["moves"] for t in o.trace]
+
+
+# several repetitions a level that apply moves: the state updated for them (levels of 2^19 pins or more, so
+# here down to the level that falls below that) equals the rebuilt one
+@pytest.mark.parametrize("weights,kind", [(False, 0), (True, 1)])
+def test_updated_repetitions(torch, weights, kind):
+    n, e, max_size = 20000, 26000, 60
+    rng = np.random.default_rng(5)
+    # hyperedges around a ring: moves between neighbouring parts, a few at a time
+    rows, src = [], []
+    for i in range(e):
+        k = int(rng.integers(1, max_size + 1)) if i % 3 else int(rng.integers(1, 9))
+        r = np.unique((rng.integers(0, n) + np.round(rng.normal(0, 90, size=k)).astype(np.int64)) % n)
+        rng.shuffle(r)
+        s = int(rng.integers(0, len(r) + 1)) if weights else 1
+        rows.append(np.concatenate([np.sort(r[:s]), np.sort(r[s:])]))
+        src.append(s)
+    off = np.zeros(len(rows) + 1, np.int64)
+    off[1:] = np.cumsum([len(r) for r in rows])
+    assert off[-1] >= 1 << 19
+    g = inputs.Hypergraph(n, off.astype(np.int32), np.concatenate(rows).astype(np.int32),
+                          np.asarray(src, np.int32), rng.integers(1, 30, size=len(rows)).astype(np.int32) if weights else None)
+    r = hp.partition(g, 300, 6000, seed=3, trace=True, count_kind=kind)
+    o = oracle.partition(g, 300, 6000, seed=3, trace=True, count_kind=kind)
+    assert r.status == o.status == hp.HP_OK, hp.hp_last_error()
+    assert np.array_equal(r.part, o.part)
+    for k, v in o.stats.items():
+        assert r.stats[k] == v, k
+    assert [(t["moves"], t["reps"], t["conn"]) for t in r.trace] == [(t["moves"], t["reps"], t["conn"]) for t in o.trace]
+    assert any(t["reps"] > 3 and t["pins"] >= 1 << 19 for t in o.trace)
