@@ -1253,7 +1253,7 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
 // of integers, so the result is the rebuilt one.  406 rebuilds on the 1M
 // Gaussian net (88 moves applied in each on average) took 63 and 36 ms in the
 // pins-list kernels; 69 rebuilds and 337 updates take 4 + 10 and 6 + 3 ms, and
-// 16 to list the hyperedges: 719 -> 651 ms a call.
+// 6 to list the hyperedges: 719 -> 640 ms a call.
 __global__ void k_move_nodes(Applied M, const int32_t *node, const int32_t *dst, const int32_t *size,
                              const int32_t *singin, long long *psize, int32_t *D0, int32_t *upd) {
     HP_KERNEL_ENTER();
@@ -1270,19 +1270,18 @@ __global__ void k_move_nodes(Applied M, const int32_t *node, const int32_t *dst,
         }
     }
 }
-// the hyperedges of the moved nodes (a warp per node), each once: `mark` holds
-// the number of the last update that listed a hyperedge
-__global__ void k_moved_edges(Applied M, const int32_t *node, const int32_t *off, const int32_t *ioff, const int32_t *inc,
+// the hyperedges of the moved nodes (a CTA per node: hubs have ten thousand),
+// each once: `mark` holds the number of the last update that listed a hyperedge
+__global__ void __launch_bounds__(256) k_moved_edges(Applied M, const int32_t *node, const int32_t *off, const int32_t *ioff, const int32_t *inc,
                               int32_t epoch, int32_t *mark, int32_t *tiny, int32_t *mid, int32_t *upd) {
     HP_KERNEL_ENTER();
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const uint32_t lt = (1u << lane) - 1u;
     const int32_t len = *M.applied;
-    for (int64_t k = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; k < len;
-         k += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    for (int32_t k = blockIdx.x; k < len; k += gridDim.x) {
         const int32_t v = node[M.seqmove[k]], i1 = ioff[v + 1];
-        for (int32_t t0 = ioff[v]; t0 < i1; t0 += 32) {
+        for (int32_t t0 = ioff[v] + (int32_t)(threadIdx.x & ~31u); t0 < i1; t0 += 256) {
             int cls = -1;
             int32_t e = 0;
             if (t0 + lane < i1) {
@@ -3468,7 +3467,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         launch_k(k_move_nodes, grid_of(update, 256), 256, 0, s, moved, W.S.node, W.S.dst, L.size, W.singin, R.psize, R.D0,
                  W.upd);
         HP_LAUNCH_CHECK();
-        launch_k(k_moved_edges, grid_of((int64_t)update * 32, 256), 256, 0, s, moved, W.S.node, L.off, L.ioff, L.inc,
+        launch_k(k_moved_edges, std::min(update, 16 * num_sms()), 256, 0, s, moved, W.S.node, L.off, L.ioff, L.inc,
                  ++W.epoch, W.emark, W.ttouched, W.touched, W.upd);
         HP_LAUNCH_CHECK();
         if (W.n_mid > 0) {
