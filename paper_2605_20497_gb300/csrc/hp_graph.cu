@@ -491,8 +491,7 @@ bool contract_level(const Level &L, const int32_t *mate, LevelBox *box, LevelBox
     // The coarse level at the fine level's sizes (nodes and pins only shrink).
     // The scratch is one block, and so is a coarse level of up to SLAB_NP pins:
     // a chain of small levels otherwise spends 34 allocator calls on each, which
-    // the workers of a batch contend for.  Larger levels are separate
-    // blocks, some of which are given back before the refinement.
+    // the workers of a batch contend for.
     Level K;
     void *scratch = nullptr;
     const bool slab = np <= SLAB_NP;
@@ -510,18 +509,22 @@ bool contract_level(const Level &L, const int32_t *mate, LevelBox *box, LevelBox
         if (pass == 1) T.at = static_cast<unsigned char *>(K.slab);
         (void)T.take<unsigned char>(1);   // no array starts the block: releasing an array releases nothing
         K.size = T.take<int32_t>(n);
-        K.nbnd = T.take<int32_t>(n);
         K.off = T.take<int32_t>(e + 1);
         K.nsrc = T.take<int32_t>(e);
         K.pin = T.take<int32_t>(np);
-        K.pedge = T.take<int32_t>(np);
         K.ioff = T.take<int32_t>(n + 1);
         K.nin = T.take<int32_t>(n);
         K.inc = T.take<int32_t>(np);
         K.inode = T.take<int32_t>(np);
         if (pass == 0) K.slab = A.raw(T.size);
     }
-    if (!slab) {
+    if (slab) {
+        // given back together before the refinement: one block that pedge starts
+        const size_t at = (sizeof(int32_t) * np + 255) & ~size_t(255);
+        unsigned char *u = static_cast<unsigned char *>(A.raw(at + sizeof(int32_t) * n));
+        K.pedge = reinterpret_cast<int32_t *>(u);
+        K.nbnd = reinterpret_cast<int32_t *>(u + at);
+    } else {
         K.size = A.get<int32_t>(n);
         K.nbnd = A.get<int32_t>(n);
         K.off = A.get<int32_t>(e + 1);

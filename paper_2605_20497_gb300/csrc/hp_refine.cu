@@ -3057,11 +3057,12 @@ struct LevelWs {
 
 // rows of part bits (16 * wq bytes per hyperedge) for the current number of
 // parts, where every sum of weights fits their 32-bit counters and they take
-// at most PB_BYTES
+// at most PB_BYTES, and no more than 8 bytes a pin (beyond a megabyte): rows
+// longer than their hyperedges' lists do not pay
 static void part_bits_rows(LevelWs &W, const Params &P, Arena &A) {
     if (W.nparts > PB_PARTS || P.wsum >= (1ll << 32) || P.o.debug_table_cap != 0) return;
     W.wq = (int)pow2_at_least(std::max<int64_t>(cdiv(W.nparts, 128), 1));
-    if (!W.bits && (int64_t)W.ce * W.wq * 16 <= PB_BYTES) W.bits = A.get<uint4>((int64_t)W.ce * W.wq);
+    if (!W.bits && (int64_t)W.ce * W.wq * 16 <= std::min(PB_BYTES, 8 * W.cnp + (int64_t(1) << 20))) W.bits = A.get<uint4>((int64_t)W.ce * W.wq);
 }
 
 static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t e, int32_t nparts, int32_t max_e,
