@@ -510,8 +510,9 @@ def main():
             "peak_source": f"{peak_kind} hbm_gbs",
             "basis": ("hp_stats.alg_bytes: per coarsening level the proposal traversal (as in 'roofline'), 48 B "
                       "per node per matching round and 12 B per pin + 8 B per coarse pin + 16 B per node of "
-                      "contraction; per refinement repetition 12 B per pin + 12 B per pins-list entry when the "
-                      "lists are rebuilt, 4 B per cut incidence entry + 12 B per list entry behind it, 48 B per "
+                      "contraction; per refinement repetition 8 B per pin + 12 B per pins-list entry when the "
+                      "lists are rebuilt (of the hyperedges with a moved pin only when they are updated), 4 B per "
+                      "incidence entry scanned after either, 4 B per cut incidence entry + 12 B per list entry behind it, 48 B per "
                       "proposed move; divided by ms_per_step")},
         "gpu_launches": launches,
         "clocks": clocks,

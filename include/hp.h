@@ -185,9 +185,10 @@ typedef struct {
                                   neighbour, 12 B per incidence entry, 12*pi+4 B per node), the
                                   matching (48 B per node per round) and the contraction (12 B per
                                   pin, 8 B per coarse pin, 16 B per node); per refinement
-                                  repetition the pins lists when rebuilt (12 B per pin + 12 B per
-                                  list entry), the cut entries and their list entries (4 B + 12 B),
-                                  and 48 B per proposed move */
+                                  repetition the pins lists when rebuilt (8 B per pin + 12 B per
+                                  list entry; of the hyperedges with a moved pin only when updated),
+                                  the incidence scanned after either (4 B per pin), the cut entries
+                                  and their list entries (4 B + 12 B), and 48 B per proposed move */
 } hp_stats;
 
 /* Per-level trace record (optional output of hp_partition_ex). */

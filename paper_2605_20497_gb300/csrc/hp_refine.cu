@@ -178,14 +178,16 @@ struct Applied {
 // UPDATE: the list holds the hyperedges that may have a pin among the applied
 // moves (*count_p of them); the ones that do take their old contributions to
 // D(p) and saving(v) back, read off their old pins list, before they are
-// rebuilt.
+// rebuilt; their pins and new list entries are counted into acc[0] and acc[1].
 template <bool UPDATE>
 __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const int32_t *pin, const int32_t *nsrc,
                                                       const int32_t *w, const int32_t *rho, const int32_t *list,
                                                       int32_t count, const int32_t *count_p, Applied M, int32_t nparts,
-                                                      Plist PL, int32_t *D, long long *saving) {
+                                                      Plist PL, int32_t *D, long long *saving,
+                                                      unsigned long long *acc) {
     HP_KERNEL_ENTER();
     int32_t len = 0;
+    unsigned long long n_pins = 0, n_ent = 0;
     if (UPDATE) {
         count = *count_p;
         len = *M.applied;
@@ -276,12 +278,26 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
             if (c >> 16) atomicAdd(&s_d[p], 1u);
         }
         used[lane] = 0;
-        if (lane == 31) PL.lam[e] = inc;
+        if (lane == 31) {
+            PL.lam[e] = inc;
+            n_pins += (unsigned long long)(b - a);
+            n_ent += (unsigned long long)inc;
+        }
         __syncwarp();
     }
+    __shared__ unsigned long long s_acc[2];
+    if (UPDATE && threadIdx.x < 2) s_acc[threadIdx.x] = 0;
     __syncthreads();
     for (int32_t p = threadIdx.x; p < nparts; p += PP_T)
         if (s_d[p]) atomicAdd(&D[p], (int32_t)s_d[p]);
+    if (UPDATE) {
+        if (lane == 31 && n_pins) {
+            atomicAdd(&s_acc[0], n_pins);
+            atomicAdd(&s_acc[1], n_ent);
+        }
+        __syncthreads();
+        if (threadIdx.x < 2 && s_acc[threadIdx.x]) atomicAdd(&acc[threadIdx.x], s_acc[threadIdx.x]);
+    }
 }
 
 // edges with |e| > small_max, one CTA each, tables in global memory
@@ -1246,6 +1262,9 @@ __global__ void k_plist_tiny(const int32_t *off, const int32_t *pin, const int32
     }
 }
 
+// words of `upd`: hyperedges of 2..TINY_E pins and larger ones among the moved
+// nodes', and two 64-bit sums over them, pins and new list entries
+enum { U_TINY, U_MID, U_ACC, U_N = U_ACC + 4 };
 // After a repetition that applied few moves, the next one updates the
 // partition-dependent state where they changed it instead of rebuilding it:
 // |p| and the single-pin hyperedges' share of D(p) per move, and the pins
@@ -1258,7 +1277,7 @@ __global__ void k_move_nodes(Applied M, const int32_t *node, const int32_t *dst,
                              const int32_t *singin, long long *psize, int32_t *D0, int32_t *upd) {
     HP_KERNEL_ENTER();
     const int32_t len = *M.applied;
-    if (blockIdx.x == 0 && threadIdx.x < 2) upd[threadIdx.x] = 0;
+    if (blockIdx.x == 0 && threadIdx.x < U_N) upd[threadIdx.x] = 0;
     GRID_STRIDE(k, (int64_t)len) {
         const int32_t i = M.seqmove[k], v = node[i], ps = M.src[i], pd = dst[i];
         const unsigned long long sz = (unsigned long long)size[v];
@@ -1304,9 +1323,14 @@ __global__ void __launch_bounds__(256) k_moved_edges(Applied M, const int32_t *n
 // hyperedges of 2..TINY_E pins from the list, one thread each
 __global__ void k_plist_tiny_update(const int32_t *off, const int32_t *pin, const int32_t *nsrc, const int32_t *w,
                                     const int32_t *rho, const int32_t *list, const int32_t *count_p, Applied M, Plist PL,
-                                    int32_t *D, long long *saving) {
+                                    int32_t *D, long long *saving, unsigned long long *acc) {
     HP_KERNEL_ENTER();
     const int32_t count = *count_p, len = *M.applied;
+    if ((int64_t)blockIdx.x * blockDim.x >= count) return;
+    __shared__ unsigned long long s_acc[2];
+    if (threadIdx.x < 2) s_acc[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned long long n_pins = 0, n_ent = 0;
     GRID_STRIDE(x, (int64_t)count) {
         const int32_t e = list[x], a = off[e], sz = off[e + 1] - a;
         int32_t vv[TINY_E], np[TINY_E], op[TINY_E];
@@ -1363,13 +1387,26 @@ __global__ void k_plist_tiny_update(const int32_t *off, const int32_t *pin, cons
             }
         }
         PL.lam[e] = lam;
+        n_pins += (unsigned long long)sz;
+        n_ent += (unsigned long long)lam;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        n_pins += __shfl_down_sync(0xffffffffu, n_pins, o);
+        n_ent += __shfl_down_sync(0xffffffffu, n_ent, o);
+    }
+    if ((threadIdx.x & 31) == 0 && n_pins) {
+        atomicAdd(&s_acc[0], n_pins);
+        atomicAdd(&s_acc[1], n_ent);
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 && s_acc[threadIdx.x]) atomicAdd(&acc[threadIdx.x], s_acc[threadIdx.x]);
 }
 
 // counters of one repetition (device)
 enum { C_CAND, C_MOVES, C_OVF, C_BAD, C_NH, C_BAD0, C_APPLIED, C_NV, C_HUB, C_CW, C_TOUCH, C_PAD,
        C_ACC,          // three 64-bit byte counters (even index: 8-byte aligned), see k_cut_bits
-       C_N = C_ACC + 6 };
+       C_UPD = C_ACC + 6,   // the two 64-bit sums of an update (upd[U_ACC])
+       C_N = C_UPD + 4 };
 
 // moves of at most SMALLM are validated by one CTA (k_val_small) with the
 // sorts in shared memory; moves of at most sq_max<uint64_t>() are sequenced by one
@@ -1402,8 +1439,8 @@ __device__ __forceinline__ int64_t rep_zero_span(const RepArrays &R) {
 }
 // keep 1: the partition is the one of the previous repetition (it applied
 // nothing), so D(p), |p|, saving(v) and the cut lists are still valid; keep 2:
-// the first three have been updated
-__global__ void k_rep_zero(RepArrays R, int keep) {
+// the first three have been updated, and `upd` says what that took
+__global__ void k_rep_zero(RepArrays R, int keep, const int32_t *upd) {
     HP_KERNEL_ENTER();
     GRID_STRIDE(i, rep_zero_span(R)) {
         if (i < R.nparts && !keep) {
@@ -1425,7 +1462,7 @@ __global__ void k_rep_zero(RepArrays R, int keep) {
             R.dDd[i] = 0;
             R.viol[i] = 0;
         }
-        if (i < C_N) R.cnt[i] = 0;
+        if (i < C_N) R.cnt[i] = keep == 2 && i >= C_UPD ? upd[U_ACC + i - C_UPD] : 0;
         if (i <= R.rounds) R.linked[i] = 0;
     }
 }
@@ -3027,7 +3064,7 @@ struct LevelWs {
     uint4 *bits = nullptr;   // [ce][wq] parts of every cut hyperedge (k_part_bits), or none
     int wq = 0;
     int32_t *touched, *ttouched;             // hyperedges of mid (of tiny) with a moved pin
-    int32_t *emark, *upd;                    // [ce] last update that listed a hyperedge; its two counts
+    int32_t *emark, *upd;                    // [ce] last update that listed a hyperedge; its counts (U_N words)
     int32_t epoch = 0;
     Moves M, S;
     uint64_t *keys;
@@ -3134,7 +3171,7 @@ static LevelWs *refine_workspace_body(LevelWs *W, int32_t n, int64_t np, int32_t
     W->touched = A.get<int32_t>(e);
     W->ttouched = A.get<int32_t>(e);
     W->emark = A.get<int32_t>(std::max(e, 1));
-    W->upd = A.get<int32_t>(2);
+    W->upd = A.get<int32_t>(U_N);
     HPC(cudaMemsetAsync(W->emark, 0, sizeof(int32_t) * std::max(e, 1), s));
     for (Moves *m : {&W->M, &W->S}) {
         m->node = A.get<int32_t>(n);
@@ -3463,6 +3500,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
     const int64_t zspan = std::max<int64_t>(std::max<int64_t>(n, (int64_t)nparts + 1),
                                             std::max<int64_t>((int64_t)C_N, (int64_t)P.o.chain_rounds + 1));
     const Applied moved{R.mvpos, W.seqmove, W.S.src, cnt + C_APPLIED};
+    unsigned long long *uacc = reinterpret_cast<unsigned long long *>(W.upd + U_ACC);
     if (update > 0) {
         // the previous repetition applied `update` moves
         launch_k(k_move_nodes, grid_of(update, 256), 256, 0, s, moved, W.S.node, W.S.dst, L.size, W.singin, R.psize, R.D0,
@@ -3475,17 +3513,17 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
             const size_t sm = plist_parts_smem(nparts);
             const int occ = prepare_kernel((const void *)k_plist_parts<true>, PP_T, sm);
             const int grid = (int)std::min<int64_t>(cdiv(W.n_mid, PP_T / 32), (int64_t)num_sms() * occ);
-            launch_k(k_plist_parts<true>, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.touched, 0, W.upd + 1, moved,
-                     nparts, W.PL, R.D0, R.saving);
+            launch_k(k_plist_parts<true>, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.touched, 0, W.upd + U_MID, moved,
+                     nparts, W.PL, R.D0, R.saving, uacc);
             HP_LAUNCH_CHECK();
         }
         if (W.n_tiny > 0) {
             launch_k(k_plist_tiny_update, std::min(grid_of(W.n_tiny, 128), 8 * num_sms()), 128, 0, s, L.off, L.pin, L.nsrc,
-                     w, rho, W.ttouched, W.upd, moved, W.PL, R.D0, R.saving);
+                     w, rho, W.ttouched, W.upd + U_TINY, moved, W.PL, R.D0, R.saving, uacc);
             HP_LAUNCH_CHECK();
         }
     }
-    launch_k(k_rep_zero, grid_of(zspan, 256), 256, 0, s, R, reuse ? 1 : update ? 2 : 0);
+    launch_k(k_rep_zero, grid_of(zspan, 256), 256, 0, s, R, reuse ? 1 : update ? 2 : 0, W.upd);
     HP_LAUNCH_CHECK();
     if (!reuse && update == 0) {
         // (a few CTAs an SM: each ends with a pass over the parts; the step call takes any sizes)
@@ -3498,7 +3536,7 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
             const int occ = prepare_kernel((const void *)k_plist_parts<false>, PP_T, sm);
             const int grid = (int)std::min<int64_t>(cdiv(W.n_mid, PP_T / 32), (int64_t)num_sms() * occ);
             launch_k(k_plist_parts<false>, grid, PP_T, sm, s, L.off, L.pin, L.nsrc, w, rho, W.mid, W.n_mid, nullptr, moved,
-                     nparts, W.PL, R.D0, R.saving);
+                     nparts, W.PL, R.D0, R.saving, nullptr);
             HP_LAUNCH_CHECK();
         } else if (W.n_mid > 0) {
             // hyperedges of up to MID_SPLIT pins in small tables (many warps
@@ -3598,14 +3636,16 @@ static int32_t rep_run(const Level &L, const int32_t *w, const Params &P, int32_
         if (hc[C_BAD]) throw Error(HP_ERR_INTERNAL, "gain table overflow");
         // algorithmic bytes (scope of Sec. VI-B..VI-D): a rebuilt repetition
         // reads each pin and its part (8 B) and writes the pins-list entries
-        // (12 B each) and scans the incidence for cut hyperedges (4 B per
-        // entry); every repetition reads the cut entries (4 B) and the list
-        // entries behind them (12 B), and moves 48 B per proposed move (sort
-        // read and write, sequence, in-sequence gain, two capacity events, apply)
-        unsigned long long acc[3];
+        // (12 B each), an updated one those of the hyperedges with a moved pin;
+        // both scan the incidence for cut hyperedges (4 B per entry); every
+        // repetition reads the cut entries (4 B) and the list entries behind
+        // them (12 B), and moves 48 B per proposed move (sort read and write,
+        // sequence, in-sequence gain, two capacity events, apply)
+        unsigned long long acc[5];   // C_ACC, C_UPD
         std::memcpy(acc, hc + C_ACC, sizeof acc);
         if (!reuse) {
-            W.alg_bytes += 12 * L.np + 12 * (int64_t)acc[0];
+            W.alg_bytes += 4 * L.np + (update > 0 ? 8 * (int64_t)acc[3] + 12 * (int64_t)acc[4]
+                                                  : 8 * L.np + 12 * (int64_t)acc[0]);
             W.cuts = (int64_t)acc[1];
             W.cut_lam = (int64_t)acc[2];
         }
