@@ -424,15 +424,15 @@ struct Hedge {
     unsigned long long q;
     bool vin;
 };
-__device__ __forceinline__ Hedge hedge_of(const PropCtx &C, int32_t i0, int32_t t, int32_t deg, int32_t nin_v) {
+__device__ __forceinline__ Hedge hedge_of(const PropCtx &C, int32_t i0, uint32_t t, int32_t deg, int32_t nin_v) {
     Hedge x{-1, 0, 0, 0, 0ull, false};
-    if (t < deg) {
-        x.e = C.inc[i0 + t];
+    if (t < (uint32_t)deg) {
+        x.e = C.inc[i0 + (int32_t)t];
         x.a = C.off[x.e];
         x.sz = C.off[x.e + 1] - x.a;
         x.d0 = x.a + C.nsrc[x.e];
         x.q = C.q[x.e];
-        x.vin = t < nin_v;
+        x.vin = t < (uint32_t)nin_v;
         if (x.sz < 2) x.sz = 0;
     }
     return x;
@@ -457,7 +457,7 @@ __device__ __forceinline__ void walk_small(const PropCtx &C, int32_t v, int32_t 
         if (m == v) m = -1;
         const unsigned g = __match_any_sync(FULL, m);
         const bool on = m >= 0;
-        uint32_t y[3] = {(uint32_t)(x.q & 0x1FFFFFull), (uint32_t)(x.q >> 21), x.vin && x.a + j >= x.d0 ? 1u : 0u};
+        uint32_t y[3] = {(uint32_t)(x.q & 0x1FFFFFull), (uint32_t)(x.q >> 21), x.vin && j >= x.d0 - x.a ? 1u : 0u};
         group_sum(g, on, y);
         const bool lead = on && (g & lt) == 0u && size_ok(C, slack, m);
         ins(lead, m, (unsigned long long)y[0] + ((unsigned long long)y[1] << 21), y[2]);
@@ -467,12 +467,14 @@ __device__ __forceinline__ void walk_small(const PropCtx &C, int32_t v, int32_t 
 template <class Ins>
 __device__ __forceinline__ void walk_list(const PropCtx &C, int32_t v, int32_t slack, int32_t beg, int32_t end,
                                           int32_t d0, unsigned long long q, uint32_t ic, const Ins &ins) {
-    int32_t j = beg + (int32_t)(threadIdx.x & 31);
-    int32_t mn = j < end ? __ldg(&C.pin[j]) : -1;
-    for (int32_t j0 = beg; j0 < end; j0 += 32, j += 32) {
+    // (unsigned positions: they may pass 2^31 behind the level's last pin)
+    const uint32_t e1 = (uint32_t)end, s1 = (uint32_t)d0;
+    uint32_t j = (uint32_t)beg + (threadIdx.x & 31);
+    int32_t mn = j < e1 ? __ldg(&C.pin[j]) : -1;
+    for (uint32_t j0 = (uint32_t)beg; j0 < e1; j0 += 32, j += 32) {
         const int32_t m = mn;
-        mn = j + 32 < end ? __ldg(&C.pin[j + 32]) : -1;   // the next pin is loaded before this one is entered
-        ins(m >= 0 && m != v && size_ok(C, slack, m), m, q, j >= d0 ? ic : 0u);
+        mn = j + 32 < e1 ? __ldg(&C.pin[j + 32]) : -1;   // the next pin is loaded before this one is entered
+        ins(m >= 0 && m != v && size_ok(C, slack, m), m, q, j >= s1 ? ic : 0u);
     }
 }
 
@@ -482,8 +484,8 @@ __device__ __forceinline__ void warp_walk(const PropCtx &C, int32_t v, int32_t i
                                           const Ins &ins) {
     const unsigned FULL = 0xffffffffu;
     const int32_t slack = size_slack(C, v);
-    for (int32_t base = 0; base < deg; base += 32) {
-        const Hedge x = hedge_of(C, i0, base + (int32_t)(threadIdx.x & 31), deg, nin_v);
+    for (uint32_t base = 0; base < (uint32_t)deg; base += 32) {
+        const Hedge x = hedge_of(C, i0, base + (threadIdx.x & 31), deg, nin_v);
         walk_small(C, v, slack, x, ins);
         unsigned lm = __ballot_sync(FULL, x.sz > SMALL_E);
         while (lm) {
@@ -524,9 +526,9 @@ __device__ void cta_walk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, i
     int par = 0;
     constexpr int CH = Queue::CH;
     Hedge nx = hedge_of(C, i0, tid < CH ? tid : deg, deg, nin_v);
-    for (int32_t base = 0; base < deg; base += CH, par ^= 1) {
+    for (uint32_t base = 0; base < (uint32_t)deg; base += CH, par ^= 1) {
         const Hedge x = nx;
-        if (base + CH < deg) nx = hedge_of(C, i0, tid < CH ? base + CH + tid : deg, deg, nin_v);
+        if (base + CH < (uint32_t)deg) nx = hedge_of(C, i0, tid < CH ? base + CH + tid : deg, deg, nin_v);
         walk_small(C, v, slack, x, ins);
         const bool large = x.sz > SMALL_E;
         if (__any_sync(FULL, large)) {
@@ -540,7 +542,7 @@ __device__ void cta_walk(const PropCtx &C, int32_t v, int32_t i0, int32_t deg, i
                 group_sum(grp, large, y);
                 const int smax = (int)__reduce_max_sync(FULL, large ? (unsigned)(x.d0 - x.a) : 0u);
                 for (int j = 0; j < smax; j++) {
-                    const int32_t m = large && x.a + j < x.d0 ? C.pin[x.a + j] : -1;
+                    const int32_t m = large && j < x.d0 - x.a ? C.pin[x.a + j] : -1;
                     ins(m >= 0 && m != v && size_ok(C, slack, m), m, x.q, 0u);
                 }
                 q = (unsigned long long)y[0] + ((unsigned long long)y[1] << 21);
@@ -597,7 +599,7 @@ __global__ void k_dst_hash(const int32_t *off, const int32_t *pin, const int32_t
     for (int64_t i = w0; i < e; i += nw) {
         const int32_t d0 = off[i] + nsrc[i], b = off[i + 1];
         uint32_t h = 0;
-        for (int32_t j = d0 + lane; j < b; j += 32) h += fmix32((uint32_t)pin[j] ^ ((uint32_t)(j - d0) * 0x9E3779B9u));
+        for (int64_t j = (int64_t)d0 + lane; j < b; j += 32) h += fmix32((uint32_t)pin[j] ^ ((uint32_t)(j - d0) * 0x9E3779B9u));
         for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
         if (lane == 0) {
             key[i] = fmix32(h ^ (uint32_t)(b - d0));

@@ -55,7 +55,7 @@ __global__ void k_pin_edges(const int32_t *off, int32_t e, int32_t *pedge) {
     int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = warp; i < e; i += nw)
-        for (int32_t j = off[i] + lane; j < off[i + 1]; j += 32) pedge[j] = (int32_t)i;
+        for (int64_t j = (int64_t)off[i] + lane; j < off[i + 1]; j += 32) pedge[j] = (int32_t)i;
 }
 
 __global__ void k_check_pins(const int32_t *pin, int64_t np, int32_t n, uint32_t *err) {

@@ -96,7 +96,7 @@ __device__ void na_distinct(int32_t a, int32_t b, int gt, int group, const int32
                             int32_t num_nodes, int32_t num_parts, uint32_t *tab, uint32_t cap, uint32_t *head,
                             int32_t *count, Sync sync) {
     const uint32_t mask = cap - 1;
-    for (int32_t j = a + gt; j < b; j += group) {
+    for (int64_t j = (int64_t)a + gt; j < b; j += group) {
         const int32_t v = pins[j];
         if (v < 0 || v >= num_nodes) {
             na_flag(head, NE_CSR);

@@ -60,7 +60,7 @@ __device__ void plist_edge(int32_t e, int gt, const int32_t *off, const int32_t 
     const int32_t a = off[e], b = off[e + 1], dst0 = a + nsrc[e];
     if (gt == 0) *g_cnt = 0;
     gsync<G>();
-    for (int32_t j = a + gt; j < b; j += G) {
+    for (int64_t j = (int64_t)a + gt; j < b; j += G) {
         int32_t p = rho[pin[j]];
         uint32_t h = hslot(p, mask);
         for (uint32_t probe = 0; probe < cap; probe++) {
@@ -86,7 +86,7 @@ __device__ void plist_edge(int32_t e, int gt, const int32_t *off, const int32_t 
     const int32_t lam = *(volatile int32_t *)g_cnt;
     if (saving && b - a >= 2) {
         const long long we = w[e];
-        for (int32_t j = a + gt; j < b; j += G) {
+        for (int64_t j = (int64_t)a + gt; j < b; j += G) {
             int32_t v = pin[j], p = rho[v];
             uint32_t h = hslot(p, mask);
             for (uint32_t probe = 0; probe < cap && keys[h] != p; probe++) h = (h + 1) & mask;
@@ -205,21 +205,22 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
     constexpr int R = 4;   // pins a lane holds at a time
     for (int64_t x = w0; x < count; x += nw) {
         const int32_t e = list[x];
-        const int32_t a = off[e], b = off[e + 1], dst0 = a + nsrc[e];
+        // (positions within the hyperedge: the level's last pin may be number 2^31 - 2)
+        const int32_t a = off[e], sz = off[e + 1] - a, dst0 = nsrc[e];
         const unsigned long long we = (unsigned long long)w[e];
         int32_t vv[R], pp[R];
         auto load = [&](int32_t j0) {
 #pragma unroll
             for (int k = 0; k < R; k++) {
                 const int32_t j = j0 + 32 * k + lane;
-                vv[k] = j < b ? pin[j] : -1;
+                vv[k] = j < sz ? pin[a + j] : -1;
             }
 #pragma unroll
             for (int k = 0; k < R; k++) pp[k] = vv[k] >= 0 ? rho[vv[k]] : 0;
         };
         if (UPDATE) {
             bool moved = false;
-            for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
+            for (int32_t j0 = 0; j0 < sz; j0 += 32 * R) {
                 load(j0);
 #pragma unroll
                 for (int k = 0; k < R; k++) moved |= vv[k] >= 0 && M.old_part(vv[k], pp[k], len) != pp[k];
@@ -232,8 +233,8 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
                 if (ci > 0) atomicAdd(&s_d[p], 0xffffffffu);
             }
             __syncwarp();
-            for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
-                if (b - a > 32 * R) load(j0);
+            for (int32_t j0 = 0; j0 < sz; j0 += 32 * R) {
+                if (sz > 32 * R) load(j0);
 #pragma unroll
                 for (int k = 0; k < R; k++)
                     if (vv[k] >= 0 && cnt[M.old_part(vv[k], pp[k], len)] == 1u)
@@ -243,7 +244,7 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
             for (int32_t x2 = lane; x2 < lam; x2 += 32) cnt[PL.p[a + x2]] = 0;
             __syncwarp();
         }
-        for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
+        for (int32_t j0 = 0; j0 < sz; j0 += 32 * R) {
             load(j0);
 #pragma unroll
             for (int k = 0; k < R; k++)
@@ -261,8 +262,8 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
         }
         at = a + inc - at;
         // a pin alone in its part can be spared a cut
-        for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
-            if (b - a > 32 * R) load(j0);
+        for (int32_t j0 = 0; j0 < sz; j0 += 32 * R) {
+            if (sz > 32 * R) load(j0);
 #pragma unroll
             for (int k = 0; k < R; k++)
                 if (vv[k] >= 0 && (cnt[pp[k]] & 0xffffu) == 1u) atomicAdd((unsigned long long *)&saving[vv[k]], we);
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(PP_T) k_plist_parts(const int32_t *off, const 
         used[lane] = 0;
         if (lane == 31) {
             PL.lam[e] = inc;
-            n_pins += (unsigned long long)(b - a);
+            n_pins += (unsigned long long)sz;
             n_ent += (unsigned long long)inc;
         }
         __syncwarp();
@@ -444,9 +445,10 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     constexpr int R = 4;   // pins a lane holds at a time
     int32_t na = 0, nb = 0, nv[R];
+    // (lengths are compared, not positions, which may pass 2^31 behind the last pin)
     auto pins_of = [&](int32_t j0, int32_t b, int32_t (&v)[R]) {
 #pragma unroll
-        for (int k = 0; k < R; k++) v[k] = j0 + 32 * k + lane < b ? pin[j0 + 32 * k + lane] : -1;
+        for (int k = 0; k < R; k++) v[k] = 32 * k + lane < b - j0 ? pin[j0 + (32 * k + lane)] : -1;
     };
     if (w0 < e) {
         na = off[w0];
@@ -472,8 +474,8 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
             if (j0 != a) pins_of(j0, b, vv);
 #pragma unroll
             for (int k = 0; k < R; k++) {
-                const int32_t j = j0 + 32 * k + lane;
-                const bool in = j < b;
+                const bool in = 32 * k + lane < b - j0;
+                const int32_t j = in ? j0 + (32 * k + lane) : a;
                 bool ok = in;
                 if (CHECK) {
                     int32_t pv = __shfl_up_sync(FULL, vv[k], 1);
@@ -495,6 +497,7 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
                     }
                 }
             }
+            if (b - j0 <= 32 * R) break;
         }
         __syncwarp();
         uint32_t lam = 0;
@@ -674,10 +677,12 @@ __device__ void gains_node(int32_t v, const int32_t *off, const int32_t *ioff, c
     // before one table update per distinct part, so that the few parts a
     // node touches are not hammered by every lane.
     {
-        const int32_t c0 = ioff[v], c1 = c0 + cutn[v];
-        for (int32_t base = c0; base < c1; base += blockDim.x) {
+        // (unsigned positions, here and in the other gain kernels: they may pass 2^31
+        // behind the last incidence entry)
+        const uint32_t c0 = ioff[v], c1 = c0 + cutn[v];
+        for (uint32_t base = c0; base < c1; base += blockDim.x) {
             if (__any_sync(0xffffffffu, *(volatile int *)s_flag)) break;
-            const int32_t t = base + (int32_t)threadIdx.x;
+            const uint32_t t = base + threadIdx.x;
             int32_t a = 0, lam = 0;
             uint32_t we = 0;
             if (t < c1) {
@@ -853,10 +858,10 @@ __global__ void __launch_bounds__(GW_T) k_gains_warp(GainArgs G, const int32_t *
     for (int64_t k = gw; k < count; k += nw) {
         const int32_t v = list[k];
         const int32_t s = G.rho[v];
-        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
-        for (int32_t base = c0; base < c1; base += 32) {
+        const uint32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
+        for (uint32_t base = c0; base < c1; base += 32) {
             if (*(volatile int32_t *)&s_used[wid] > (int32_t)limit) break;   // same value for the whole warp
-            const int32_t t = base + lane;
+            const uint32_t t = base + lane;
             int32_t a = 0, lam = 0;
             uint32_t we = 0;
             if (t < c1) {
@@ -994,19 +999,19 @@ __global__ void __launch_bounds__(NW * 32) k_gains_bits(GainArgs G, const uint4 
     __syncthreads();
     for (int32_t k = blockIdx.x; k < count; k += gridDim.x) {
         const int32_t v = k < n1 ? list[k] : list2[k - n1], s = G.rho[v];
-        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
+        const uint32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
         uint32_t acc[WQ * 4];
 #pragma unroll
         for (int q = 0; q < WQ * 4; q++) acc[q] = 0;
-        for (int32_t base = c0 + wid * 32; base < c1; base += NW * 32) {
-            const int32_t t = base + lane;
+        for (uint32_t base = c0 + wid * 32; base < c1; base += NW * 32) {
+            const uint32_t t = base + lane;
             int32_t e = 0;
             uint32_t we = 0;
             if (t < c1) {
                 e = G.inc[t];
                 we = (uint32_t)G.w[e];
             }
-            const int cnt = min(32, c1 - base);
+            const int cnt = (int)min(32u, c1 - base);
 #pragma unroll 4
             for (int u = 0; u < cnt; u++) {
                 const uint4 *r = bits + (int64_t)__shfl_sync(FULL, e, u) * WQ;
@@ -1299,8 +1304,9 @@ __global__ void __launch_bounds__(256) k_moved_edges(Applied M, const int32_t *n
     const uint32_t lt = (1u << lane) - 1u;
     const int32_t len = *M.applied;
     for (int32_t k = blockIdx.x; k < len; k += gridDim.x) {
-        const int32_t v = node[M.seqmove[k]], i1 = ioff[v + 1];
-        for (int32_t t0 = ioff[v] + (int32_t)(threadIdx.x & ~31u); t0 < i1; t0 += 256) {
+        const int32_t v = node[M.seqmove[k]];
+        const uint32_t i1 = ioff[v + 1];
+        for (uint32_t t0 = ioff[v] + (threadIdx.x & ~31u); t0 < i1; t0 += 256) {
             int cls = -1;
             int32_t e = 0;
             if (t0 + lane < i1) {
@@ -2707,7 +2713,7 @@ __device__ void inseq_edge(const SeqSim &Q, int32_t e, int gt, int32_t *bk, int3
     const int32_t a = Q.off[e], b = Q.off[e + 1], dst0 = a + Q.nsrc[e];
     if (gt == 0) *g_cnt = 0;
     gsync<G>();
-    for (int32_t j = a + gt; j < b; j += G) {
+    for (int64_t j = (int64_t)a + gt; j < b; j += G) {
         int32_t k = Q.mvpos[Q.pin[j]];
         if (k >= 0) {
             int32_t s = atomicAdd(g_cnt, 1);
@@ -2792,7 +2798,7 @@ __global__ void k_touched(const int32_t *off, const int32_t *pin, const int32_t 
             big &= big - 1;
             const int32_t ea = __shfl_sync(FULL, a, l), eb = __shfl_sync(FULL, b, l);
             bool found = false;
-            for (int32_t j0 = ea; j0 < eb; j0 += 32) {
+            for (int64_t j0 = ea; j0 < eb; j0 += 32) {
                 const bool h = j0 + lane < eb && mvpos[pin[j0 + lane]] >= 0;
                 if (__any_sync(FULL, h)) {
                     found = true;
@@ -2851,14 +2857,14 @@ __global__ void __launch_bounds__(IS_T) k_inseq_parts(SeqSim Q, const int32_t *l
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t x = w0; x < count; x += nw) {
         const int32_t e = list[x];
-        const int32_t a = Q.off[e], b = Q.off[e + 1], sz = b - a;
+        const int32_t a = Q.off[e], sz = Q.off[e + 1] - a;
         if (sz <= lo || sz > emax) continue;
-        const int32_t dst0 = a + Q.nsrc[e], lam = Q.PL.lam[e];
+        const int32_t dst0 = Q.nsrc[e], lam = Q.PL.lam[e];
         const long long we = Q.w[e];
         int32_t c = 0;
-        for (int32_t j0 = a; j0 < b; j0 += 32) {
+        for (int32_t j0 = 0; j0 < sz; j0 += 32) {
             const int32_t j = j0 + lane;
-            const int32_t k = j < b ? Q.mvpos[Q.pin[j]] : -1;
+            const int32_t k = j < sz ? Q.mvpos[Q.pin[a + j]] : -1;
             const unsigned m = __ballot_sync(FULL, k >= 0);
             if (k >= 0) mv[c + __popc(m & lt)] = ((uint32_t)k << 1) | (j >= dst0 ? 1u : 0u);
             c += __popc(m);
@@ -3354,8 +3360,8 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : NW * 32)
     gsync<NW * 32>();
     for (int64_t x = (int64_t)blockIdx.x * GROUPS + grp; x < count; x += (int64_t)gridDim.x * GROUPS) {
         const int32_t v = list[x], s = G.rho[v];
-        const int32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
-        auto hedge = [&](int32_t t, int32_t &a, int32_t &lam, uint32_t &we) {
+        const uint32_t c0 = G.ioff[v], c1 = c0 + G.cutn[v];
+        auto hedge = [&](uint32_t t, int32_t &a, int32_t &lam, uint32_t &we) {
             a = lam = 0;
             we = 0;
             if (t < c1) {
@@ -3369,7 +3375,7 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : NW * 32)
         uint32_t nwe;
         hedge(c0 + gt, na, nlam, nwe);
         const int w32 = NW == 1 ? 0 : wid * 32;
-        for (int32_t base = c0 + w32; base < c1; base += NW * 32) {
+        for (uint32_t base = c0 + w32; base < c1; base += NW * 32) {
             const int32_t a = na, lam = nlam;
             const uint32_t we = nwe;
             if (base + NW * 32 < c1) hedge(base + NW * 32 + lane, na, nlam, nwe);
