@@ -231,7 +231,7 @@ static hp_status run(const int32_t *pins, const int32_t *offsets, int32_t e, int
         tr[l].reps = ro.reps;
         tr[l].moves = ro.moves;
         if (trace_cap > 0 && l < trace_cap) {
-            objective(g, w, rho, nparts, obj, obj + 1, A);
+            objective(g, w, rho, nparts, max_e0, obj, obj + 1, A);
             tr[l].conn = fetch<int64_t>(obj, s);
         }
     }
@@ -253,7 +253,7 @@ static hp_status run(const int32_t *pins, const int32_t *offsets, int32_t e, int
     launch_k(k_check_parts, grid_of(n, 256), 256, 0, s, part, n, k, err_dev);
     HP_LAUNCH_CHECK();
     int64_t *ps = A.get<int64_t>(5);
-    part_stats(lv[0], w, part, k, omega, delta, ps, A);
+    part_stats(lv[0], w, part, k, max_e0, omega, delta, ps, A);
     int64_t hs[5];
     fetch_bytes(hs, ps, sizeof hs, s);
     uint32_t derr = fetch<uint32_t>(err_dev, s);
@@ -522,7 +522,7 @@ hp_status hp_connectivity(const int32_t *pins, const int32_t *offsets, int32_t n
         }
         if (hp::fetch<uint32_t>(e2, s)) return HP_ERR_INVALID_ARG;
         int64_t *obj = A.get<int64_t>(2);
-        hp::objective(L, w, part, num_parts, obj, obj + 1, A);
+        hp::objective(L, w, part, num_parts, hp::max_edge_size(L, A), obj, obj + 1, A);
         int64_t h[2];
         hp::fetch_bytes(h, obj, sizeof h, s);
         if (conn_out) *conn_out = h[0];

@@ -504,7 +504,8 @@ void refine_workspace_free(LevelWs *W, Arena &A);
 int32_t max_edge_size(const Level &L, Arena &A);
 RefineOut refine_level(const Level &L, const int32_t *w, const Params &P, int32_t *rho, LevelWs *W, Arena &A,
                        uint32_t *err_dev);
-void objective(const Level &L, const int32_t *w, const int32_t *rho, int32_t nparts, int64_t *conn_dev,
+// max_e: no hyperedge is larger
+void objective(const Level &L, const int32_t *w, const int32_t *rho, int32_t nparts, int32_t max_e, int64_t *conn_dev,
                int64_t *cutnet_dev, Arena &A);
 // Eq. 1 and Eq. 16 of a caller's arrays (hp_connectivity), up to
 // connectivity_scan_takes parts; see the definition
@@ -512,8 +513,8 @@ uint32_t connectivity_scan(const int32_t *pins, const int32_t *offsets, int32_t 
                            const int32_t *part, int32_t nparts, int64_t *conn, int64_t *cutnet, uint32_t *bad_part,
                            Arena &A);
 bool connectivity_scan_takes(int32_t nparts);
-void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t nparts, int32_t omega, int32_t delta,
-                int64_t *out, Arena &A);
+void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t nparts, int32_t max_e, int32_t omega,
+                int32_t delta, int64_t *out, Arena &A);
 
 // allocator hook (hp_prims.cu)
 void set_allocator(void *(*a)(size_t, void *), void (*f)(void *, void *), void *ctx);

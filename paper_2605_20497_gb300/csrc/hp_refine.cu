@@ -414,22 +414,28 @@ __global__ void k_objective(const int32_t *lam, const int32_t *w, int32_t e, uns
 // equal to its hyperedge's source raises E_DUP / E_PIN, destinations that do
 // not ascend raise PS_UNSORTED (duplicates among them are then to be looked
 // for elsewhere), parts outside [0, nparts) are skipped (the caller's check
-// reports them), and nothing is read when *pre, left by an earlier kernel, is
-// set.  Bound by the chain pin -> part -> shared memory of each hyperedge.
+// reports them), and nothing is read when *pre, left by an earlier kernel, has
+// a bit of `stop`.  Bound by the chain pin -> part -> shared memory of each hyperedge.
 // Sorting the incidence to find duplicates and building pins lists to count
 // their entries took 6.5 ms on the 80 M pins of the 1M Gaussian net; this 0.43.
+// BIG: hyperedges of more than PS_BIG pins are left to k_part_scan_big below (a
+// warp takes 2.4 us for 128 pins).  A form of its own, which the host takes where
+// there are such hyperedges: the test alone made 0.44 ms of the calls above 0.47.
 constexpr int PS_T = 256;
 constexpr int32_t PS_PARTS = 32768;   // bit rows of up to 4 KB a warp
-constexpr uint32_t PS_UNSORTED = 1u << 31;
+constexpr uint32_t PS_UNSORTED = 1u << 31, PS_HAS_BIG = 1u << 30;
+constexpr int PSB_T = 1024;
+constexpr int32_t PS_BIG = 8192;
 inline size_t part_scan_smem(int32_t nparts, bool d) {
     const size_t words = (size_t)cdiv(std::max(nparts, 1), 1024) * 32;
     return 4 * ((PS_T / 32) * words * (d ? 2 : 1) + (d ? words * 32 : 0));
 }
-template <bool CHECK>
+template <bool CHECK, bool BIG>
 __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const int32_t *pin, const int32_t *nsrc,
                                                     const int32_t *w, int32_t e, const int32_t *part, int32_t n,
                                                     int32_t nparts, int32_t *D, unsigned long long *conn,
-                                                    unsigned long long *cutnet, const uint32_t *pre, uint32_t *err) {
+                                                    unsigned long long *cutnet, const uint32_t *pre, uint32_t stop,
+                                                    uint32_t *err) {
     HP_KERNEL_ENTER();
     extern __shared__ __align__(16) uint32_t smw[];
     __shared__ unsigned long long s_sum[2];
@@ -438,17 +444,18 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
     const int words = (nparts + 1023) / 1024 * 32;   // a multiple of 32
     const int rows = (PS_T / 32) * words * (D ? 2 : 1);
     uint32_t *bm = smw + (size_t)wid * words * (D ? 2 : 1), *bd = bm + words, *s_d = smw + rows;
-    if (CHECK && *pre) return;
+    if (CHECK && (*pre & stop)) return;
     for (int i = threadIdx.x; i < rows + (D ? words * 32 : 0); i += PS_T) smw[i] = 0;
     if (threadIdx.x < 2) s_sum[threadIdx.x] = 0;
     __syncthreads();
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
     constexpr int R = 4;   // pins a lane holds at a time
-    int32_t na = 0, nb = 0, nv[R];
-    // (lengths are compared, not positions, which may pass 2^31 behind the last pin)
-    auto pins_of = [&](int32_t j0, int32_t b, int32_t (&v)[R]) {
+    uint32_t na = 0, nb = 0;
+    int32_t nv[R];
+    // (unsigned positions: they may pass 2^31 behind the last pin)
+    auto pins_of = [&](uint32_t j0, uint32_t b, int32_t (&v)[R]) {
 #pragma unroll
-        for (int k = 0; k < R; k++) v[k] = 32 * k + lane < b - j0 ? pin[j0 + (32 * k + lane)] : -1;
+        for (int k = 0; k < R; k++) v[k] = j0 + 32 * k + lane < b ? pin[j0 + 32 * k + lane] : -1;
     };
     if (w0 < e) {
         na = off[w0];
@@ -458,7 +465,7 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
     unsigned long long c = 0, cn = 0;
     uint32_t bad = 0;
     for (int64_t i = w0; i < e; i += nw) {
-        const int32_t a = na, b = nb;
+        const uint32_t a = na, b = nb;
         int32_t vv[R];
 #pragma unroll
         for (int k = 0; k < R; k++) vv[k] = nv[k];
@@ -467,15 +474,16 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
             nb = off[i + nw + 1];
             pins_of(na, nb, nv);
         }
-        const int32_t dst0 = D ? a + nsrc[i] : a + 1;
+        if (BIG && b - a > PS_BIG) continue;
+        const uint32_t dst0 = D ? a + nsrc[i] : a + 1;
         int32_t src = 0, last = INT32_MIN;   // CHECK: the source; the last pin of the chunk before
         if (CHECK) src = __shfl_sync(FULL, vv[0], 0);
-        for (int32_t j0 = a; j0 < b; j0 += 32 * R) {
+        for (uint32_t j0 = a; j0 < b; j0 += 32 * R) {
             if (j0 != a) pins_of(j0, b, vv);
 #pragma unroll
             for (int k = 0; k < R; k++) {
-                const bool in = 32 * k + lane < b - j0;
-                const int32_t j = in ? j0 + (32 * k + lane) : a;
+                const uint32_t j = j0 + 32 * k + lane;
+                const bool in = j < b;
                 bool ok = in;
                 if (CHECK) {
                     int32_t pv = __shfl_up_sync(FULL, vv[k], 1);
@@ -497,7 +505,6 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
                     }
                 }
             }
-            if (b - j0 <= 32 * R) break;
         }
         __syncwarp();
         uint32_t lam = 0;
@@ -530,16 +537,111 @@ __global__ void __launch_bounds__(PS_T) k_part_scan(const int32_t *off, const in
         for (int32_t p = threadIdx.x; p < nparts; p += PS_T)
             if (s_d[p]) atomicAdd(&D[p], (int32_t)s_d[p]);
 }
+// The same for the listed hyperedges of more than PS_BIG pins, a CTA each
+// (the row of bits, its checks and its counts are k_part_scan's).  One
+// hyperedge of 30 M pins: 575 ms by a warp, 180 by the pins lists before.
+template <bool CHECK>
+__global__ void __launch_bounds__(PSB_T) k_part_scan_big(const int32_t *off, const int32_t *pin, const int32_t *nsrc,
+                                                         const int32_t *w, const int32_t *list,
+                                                         const int32_t *count_p, const int32_t *part, int32_t n, int32_t nparts, int32_t *D, unsigned long long *conn,
+                                                         unsigned long long *cutnet, uint32_t *err) {
+    HP_KERNEL_ENTER();
+    extern __shared__ __align__(16) uint32_t smw[];
+    __shared__ int32_t s_lam;
+    const int words = (nparts + 1023) / 1024 * 32;
+    uint32_t *bm = smw, *bd = smw + words, *s_d = bd + words;
+    const int32_t count = *count_p;
+    if ((int32_t)blockIdx.x >= count) return;
+    for (int i = threadIdx.x; i < words * (D ? 34 : 1); i += PSB_T) smw[i] = 0;
+    if (threadIdx.x == 0) s_lam = 0;
+    __syncthreads();
+    uint32_t bad = 0;
+    for (int32_t x = blockIdx.x; x < count; x += gridDim.x) {
+        const int32_t i = list[x], a = off[i], len = off[i + 1] - a;
+        const int32_t *pe = pin + a;
+        const int32_t dst0 = D ? nsrc[i] : 1, src = CHECK ? pe[0] : 0;
+        constexpr int R = 4;
+        for (int64_t j0 = threadIdx.x; j0 < len; j0 += R * PSB_T) {
+            int32_t v[R], pv[R];
+#pragma unroll
+            for (int k = 0; k < R; k++) {
+                const int64_t j = j0 + k * PSB_T;
+                v[k] = j < len ? pe[j] : -1;
+                pv[k] = CHECK && j > 1 && j < len ? pe[j - 1] : INT32_MIN;
+            }
+#pragma unroll
+            for (int k = 0; k < R; k++) {
+                const int64_t j = j0 + k * PSB_T;
+                if (j >= len) break;
+                if (CHECK) {
+                    if (j > 0 && v[k] == src) bad |= E_DUP;
+                    if (v[k] <= pv[k] && j > 1) bad |= PS_UNSORTED;
+                    if (v[k] < 0 || v[k] >= n) {
+                        bad |= E_PIN;
+                        continue;
+                    }
+                }
+                const uint32_t p = (uint32_t)part[v[k]];
+                if (CHECK && p >= (uint32_t)nparts) continue;
+                const uint32_t bit = 1u << (p & 31);
+                if (!(*(volatile uint32_t *)&bm[p >> 5] & bit)) atomicOr(&bm[p >> 5], bit);
+                if (D && j >= dst0 && !(*(volatile uint32_t *)&bd[p >> 5] & bit)) atomicOr(&bd[p >> 5], bit);
+            }
+        }
+        __syncthreads();
+        int32_t lam = 0;
+        for (int y = threadIdx.x; y < words; y += PSB_T) {
+            lam += __popc(bm[y]);
+            bm[y] = 0;
+            if (D) {
+                for (uint32_t z = bd[y]; z; z &= z - 1) atomicAdd(&s_d[32 * y + __ffs(z) - 1], 1u);
+                bd[y] = 0;
+            }
+        }
+        if (lam) atomicAdd(&s_lam, lam);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            const unsigned long long we = w ? (unsigned long long)w[i] : 1ull;
+            if (s_lam > 1) {
+                atomicAdd(conn, we * (unsigned long long)(s_lam - 1));
+                atomicAdd(cutnet, we);
+            }
+            s_lam = 0;
+        }
+        __syncthreads();
+    }
+    if (CHECK && bad) atomicOr(err, bad);
+    if (D)
+        for (int32_t p = threadIdx.x; p < nparts; p += PSB_T)
+            if (s_d[p]) atomicAdd(&D[p], (int32_t)s_d[p]);
+}
+// part_scan: k_part_scan alone; with `big`, without the hyperedges of more than
+// PS_BIG pins, and k_part_scan_big for these
 template <bool CHECK>
 static void part_scan(const int32_t *off, const int32_t *pin, const int32_t *nsrc, const int32_t *w, int32_t e,
                       const int32_t *part, int32_t n, int32_t nparts, int32_t *D, int64_t *conn, int64_t *cutnet,
-                      const uint32_t *pre, uint32_t *err, cudaStream_t s) {
-    const size_t sm = part_scan_smem(nparts, D != nullptr);
-    const int occ = prepare_kernel((const void *)k_part_scan<CHECK>, PS_T, sm);
-    launch_k(k_part_scan<CHECK>, (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(e, PS_T / 32), (int64_t)num_sms() * occ)),
-             PS_T, sm, s, off, pin, nsrc, w, e, part, n, nparts, D, (unsigned long long *)conn,
-             (unsigned long long *)cutnet, pre, err);
+                      const uint32_t *pre, uint32_t stop, uint32_t *err, bool big, Arena &A) {
+    cudaStream_t s = A.stream();
+    unsigned long long *c = (unsigned long long *)conn, *cn = (unsigned long long *)cutnet;
+    size_t sm = part_scan_smem(nparts, D != nullptr);
+    auto scan = [&](auto kern) {
+        const int occ = prepare_kernel((const void *)kern, PS_T, sm);
+        launch_k(kern, (int)std::max<int64_t>(1, std::min<int64_t>(cdiv(e, PS_T / 32), (int64_t)num_sms() * occ)), PS_T,
+                 sm, s, off, pin, nsrc, w, e, part, n, nparts, D, c, cn, pre, stop, err);
+        HP_LAUNCH_CHECK();
+    };
+    if (!big) return scan(k_part_scan<CHECK, false>);
+    scan(k_part_scan<CHECK, true>);
+    int32_t *list = A.get<int32_t>(2 + (size_t)std::min<int64_t>(e, (int64_t(1) << 31) / PS_BIG)), *cnt = list, *maxe = list + 1;
+    HPC(cudaMemsetAsync(cnt, 0, 2 * sizeof(int32_t), s));
+    launch_k(k_big_edges, grid_of(e, 256), 256, 0, s, off, e, PS_BIG, list + 2, cnt, maxe);
     HP_LAUNCH_CHECK();
+    sm = 4 * (size_t)cdiv(std::max(nparts, 1), 1024) * 32 * (D ? 34 : 1);
+    const int occ = prepare_kernel((const void *)k_part_scan_big<CHECK>, PSB_T, sm);
+    launch_k(k_part_scan_big<CHECK>, num_sms() * occ, PSB_T, sm, s, off, pin, nsrc, w, list + 2, cnt, part, n, nparts,
+             D, c, cn, err);
+    HP_LAUNCH_CHECK();
+    A.release(list);
 }
 
 // A caller's offsets, weights and parts, before any pin is read.
@@ -550,6 +652,7 @@ __global__ void k_conn_check(const int32_t *off, int32_t e, const int32_t *weigh
     unsigned long long ws = 0;
     GRID_STRIDE(i, (int64_t)e) {
         if (off[i + 1] <= off[i]) bad |= E_OFFSETS;
+        else if ((int64_t)off[i + 1] - off[i] > PS_BIG) bad |= PS_HAS_BIG;
         if (weights) {
             const int32_t x = weights[i];
             if (x < 1 || x > 65536) bad |= E_WEIGHT;
@@ -562,7 +665,7 @@ __global__ void k_conn_check(const int32_t *off, int32_t e, const int32_t *weigh
     for (int o = 16; o > 0; o >>= 1) ws += __shfl_down_sync(0xffffffffu, ws, o);
     bad = __reduce_or_sync(0xffffffffu, bad);
     if ((threadIdx.x & 31) == 0) {
-        if (bad & E_OFFSETS) atomicOr(err, E_OFFSETS);
+        if (bad & (E_OFFSETS | PS_HAS_BIG)) atomicOr(err, bad & (E_OFFSETS | PS_HAS_BIG));
         if (bad & E_WEIGHT) atomicOr(err + 1, E_WEIGHT);   // (the pins are still to be checked)
         if (ws) atomicAdd(wsum, ws);
     }
@@ -586,10 +689,17 @@ uint32_t connectivity_scan(const int32_t *pins, const int32_t *offsets, int32_t 
     launch_k(k_conn_check, grid_of(std::max(e, n), 256), 256, 0, s, offsets, e, weights, part, n, nparts, &box->err,
              &box->wsum, &box->bad_part);
     HP_LAUNCH_CHECK();
-    if (e > 0)
+    auto scan = [&](uint32_t stop, bool big) {
         part_scan<true>(offsets, pins, nullptr, weights, e, part, n, nparts, nullptr, &box->conn, &box->cutnet, &box->err,
-                        &box->scan_err, s);
+                        stop, &box->scan_err, big, A);
+    };
+    if (e > 0) scan(E_OFFSETS | PS_HAS_BIG, false);
     fetch_bytes(&hb, box, sizeof hb, s);
+    if (hb.err == PS_HAS_BIG) {   // nothing scanned yet
+        scan(E_OFFSETS, true);
+        fetch_bytes(&hb, box, sizeof hb, s);
+    }
+    hb.err &= ~PS_HAS_BIG;
     A.release(box);
     *conn = hb.conn;
     *cutnet = hb.cutnet;
@@ -598,14 +708,15 @@ uint32_t connectivity_scan(const int32_t *pins, const int32_t *offsets, int32_t 
 }
 bool connectivity_scan_takes(int32_t nparts) { return nparts <= PS_PARTS; }
 
-void objective(const Level &L, const int32_t *w, const int32_t *rho, int32_t nparts, int64_t *conn_dev,
+void objective(const Level &L, const int32_t *w, const int32_t *rho, int32_t nparts, int32_t max_e, int64_t *conn_dev,
                int64_t *cutnet_dev, Arena &A) {
     cudaStream_t s = A.stream();
     HPC(cudaMemsetAsync(conn_dev, 0, sizeof(int64_t), s));
     HPC(cudaMemsetAsync(cutnet_dev, 0, sizeof(int64_t), s));
     if (L.e == 0) return;
     if (nparts <= PS_PARTS) {
-        part_scan<false>(L.off, L.pin, L.nsrc, w, L.e, rho, L.n, nparts, nullptr, conn_dev, cutnet_dev, nullptr, nullptr, s);
+        part_scan<false>(L.off, L.pin, L.nsrc, w, L.e, rho, L.n, nparts, nullptr, conn_dev, cutnet_dev, nullptr, 0,
+                         nullptr, max_e > PS_BIG, A);
         return;
     }
     int32_t *maxe = A.get<int32_t>(1);
@@ -3975,9 +4086,9 @@ __global__ void k_part_max(const long long *psize, const int32_t *D, int32_t npa
 }
 
 // out (device int64[5]): connectivity, cut-net, max part size, max distinct
-// inbound hyperedges of a part, parts violating Omega or Delta
-void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t nparts, int32_t omega, int32_t delta,
-                int64_t *out, Arena &A) {
+// inbound hyperedges of a part, parts violating Omega or Delta; max_e: the largest hyperedge
+void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t nparts, int32_t max_e, int32_t omega,
+                int32_t delta, int64_t *out, Arena &A) {
     cudaStream_t s = A.stream();
     HPC(cudaMemsetAsync(out, 0, 5 * sizeof(int64_t), s));
     if (nparts <= 0) return;
@@ -3986,7 +4097,8 @@ void part_stats(const Level &L, const int32_t *w, const int32_t *part, int32_t n
     HPC(cudaMemsetAsync(D, 0, sizeof(int32_t) * nparts, s));
     HPC(cudaMemsetAsync(psize, 0, sizeof(long long) * nparts, s));
     if (L.e > 0 && nparts <= PB_PARTS) {
-        part_scan<false>(L.off, L.pin, L.nsrc, w, L.e, part, L.n, nparts, D, out, out + 1, nullptr, nullptr, s);
+        part_scan<false>(L.off, L.pin, L.nsrc, w, L.e, part, L.n, nparts, D, out, out + 1, nullptr, 0, nullptr,
+                         max_e > PS_BIG, A);
     } else if (L.e > 0) {
         int32_t *maxe = A.get<int32_t>(1);
         HPC(cudaMemsetAsync(maxe, 0, sizeof(int32_t), s));
