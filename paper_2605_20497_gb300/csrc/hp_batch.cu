@@ -18,6 +18,7 @@
 #include <thread>
 #include <vector>
 
+#include "hp_host.h"
 #include "hp_internal.cuh"
 
 namespace hp {
@@ -41,22 +42,23 @@ static double run_group(const hp_instance *inst, const std::vector<int32_t> &ids
         HPC(cudaEventCreateWithFlags(&done[w], cudaEventDisableTiming));
         HPC(cudaStreamWaitEvent(ss[w], start, 0));
     }
-    std::atomic<size_t> next{0};
+    std::atomic<size_t> next{0}, finished{0};
     auto work = [&](int w) {
         cudaSetDevice(dev);
         t_plain_launches = true;
-        t_one_stream = true;
         for (;;) {
             const size_t k = next.fetch_add(1);
             if (k >= ids.size()) break;
             const int32_t i = ids[k];
             const hp_instance &x = inst[i];
+            t_one_stream = batch_one_stream(batch_in_flight(W, (int64_t)(ids.size() - finished.load())));
             hp_stats sx{};
             const hp_status r = hp_partition(x.pins, x.offsets, x.num_hedges, x.num_nodes, x.src_counts, x.weights,
                                              x.omega, x.delta, x.seed, opt, x.part_out, &sx, ss[w]);
             st[i] = r;
             if (r != HP_OK) msg[i] = hp_last_error();
             if (stats_out) stats_out[i] = sx;
+            finished.fetch_add(1);
         }
         cudaEventRecord(done[w], ss[w]);
     };

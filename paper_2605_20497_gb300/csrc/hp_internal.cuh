@@ -51,9 +51,10 @@ extern thread_local int64_t t_launches;
 extern thread_local bool t_plain_launches;
 // The kernels that run side by side on side streams for one instance go to
 // its one stream instead where the calling thread set t_one_stream: the batch
-// workers do, whose streams already fill the GPU (24 power-law nets, 16 in
-// flight: 251 -> 209 ms; the events and waits of five streams an instance only
-// add to the calls the workers contend for).
+// workers do while enough of them run that their streams already fill the GPU
+// (batch_one_stream; 24 power-law nets, 16 in flight: 251 -> 209 ms; the events
+// and waits of five streams an instance only add to the calls the workers
+// contend for).  Not to be changed during a call.
 extern thread_local bool t_one_stream;
 bool pdl_enabled();
 
