@@ -9,6 +9,7 @@
 #include <mutex>
 
 #include "hp_cluster.cuh"
+#include "hp_host.h"
 #include "hp_internal.cuh"
 
 namespace hp {
@@ -123,39 +124,45 @@ template double fetch<double>(const double *, cudaStream_t);
 
 int prepare_kernel(const void *func, int block, size_t smem) {
     // per (kernel, device): the dynamic shared memory limit is set on first
-    // use and only ever grows, so a size admitted once stays admitted;
-    // occupancy cached per size
-    struct Entry {
-        const void *f;
-        int dev, block;
-        size_t smem;
-        int occ;
-    };
+    // use and only ever grows, so a size admitted once stays admitted.  A thread
+    // looks its kernels up in a table of its own and takes the lock, which the
+    // workers of a batch would contend for, once per kernel and size step.
     static std::mutex mu;
-    static std::vector<Entry> occ_cache;
+    static OccTable shared;
     static std::vector<std::pair<std::pair<const void *, int>, size_t>> limit;
+    static thread_local OccTable mine;
     int dev = 0;
     HPC(cudaGetDevice(&dev));
+    const OccTable::Key key{func, dev, block, smem_steps(smem)};
+    if (const int occ = mine.find(key)) return occ;
     std::lock_guard<std::mutex> lk(mu);
-    size_t *lim = nullptr;
-    for (auto &l : limit)
-        if (l.first.first == func && l.first.second == dev) lim = &l.second;
-    if (!lim) {
-        // nothing assumed: without the attribute a kernel gets 48 KB minus
-        // its static shared memory, so the first request always sets it
-        limit.push_back({{func, dev}, (size_t)0});
-        lim = &limit.back().second;
+    int occ = shared.find(key);
+    if (!occ) {
+        // the whole step, as far as the kernel's static shared memory leaves room
+        cudaFuncAttributes at;
+        int most = 0;
+        HPC(cudaFuncGetAttributes(&at, func));
+        HPC(cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+        const size_t room = (size_t)most - std::min((size_t)most, at.sharedSizeBytes);
+        const size_t size = std::max(smem, std::min(key.steps * SMEM_STEP, room));
+        size_t *lim = nullptr;
+        for (auto &l : limit)
+            if (l.first.first == func && l.first.second == dev) lim = &l.second;
+        if (!lim) {
+            // nothing assumed: without the attribute a kernel gets 48 KB minus
+            // its static shared memory, so the first request always sets it
+            limit.push_back({{func, dev}, (size_t)0});
+            lim = &limit.back().second;
+        }
+        if (size > *lim) {
+            HPC(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)size));
+            *lim = size;
+        }
+        HPC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, func, block, size));
+        occ = std::max(occ, 1);
+        shared.put(key, occ);
     }
-    if (smem > *lim) {
-        HPC(cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        *lim = smem;
-    }
-    for (auto &c : occ_cache)
-        if (c.f == func && c.dev == dev && c.block == block && c.smem == smem) return c.occ;
-    int occ = 0;
-    HPC(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, func, block, smem));
-    occ = std::max(occ, 1);
-    occ_cache.push_back({func, dev, block, smem, occ});
+    mine.put(key, occ);
     return occ;
 }
 

@@ -19,3 +19,23 @@ def test_batch_streams(tmp_path):
               'for (auto &x : c) std::printf("%d ", (int)hp::batch_one_stream(hp::batch_in_flight(x[0], x[1]))); }\n')
     assert out == [str(int(min(c) >= 6)) for c in cases]
     assert out == ["0"] * 5 + ["1"] * 4
+
+
+# the table of occupancies stays small however many sizes a process asks for
+def test_occupancy_table_is_bounded(tmp_path):
+    out = run(tmp_path, """
+int main() {
+    hp::OccTable t;
+    const char k[3] = {};
+    for (size_t bytes = 0; bytes <= 227 * 1024; bytes++)
+        for (int x = 0; x < 3; x++) {
+            const hp::OccTable::Key key{&k[x], 0, 256, hp::smem_steps(bytes)};
+            if (!t.find(key)) t.put(key, 1 + (int)(key.steps % 31) + x);
+            if (t.find(key) != 1 + (int)(key.steps % 31) + x) return 1;
+        }
+    std::printf("%zu ", t.size());
+    for (size_t b : {0, 1, 1023, 1024, 1025, 227 * 1024}) std::printf("%zu ", hp::smem_steps(b));
+    std::printf("%d %d", t.find({&k[0], 1, 256, 5}), t.find({&k[0], 0, 512, 5}));
+}
+""")
+    assert out == ["684", "0", "1", "1", "1", "2", "227", "0", "0"]
