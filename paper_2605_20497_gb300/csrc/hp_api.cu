@@ -551,6 +551,7 @@ hp_status hp_debug_coarsen_level(int32_t num_nodes, int32_t num_hedges, const in
         hp::make_level(num_nodes, num_hedges, offsets, pins, src_counts, size, L, A);
         uint32_t *err = A.get<uint32_t>(1);
         HPC(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));
+        hp::weight_bounds(weights, num_hedges, P, A);
         hp::CoarsenWs *CW = hp::coarsen_workspace(num_nodes, num_hedges, P, A);
         hp::coarsen_level(L, level, weights, P, mate_out, *CW, A, err, cand_out, score_out);
         hp::LevelBox hb;
@@ -584,7 +585,7 @@ hp_status hp_debug_refine_rep(int32_t num_nodes, int32_t num_hedges, const int32
         hp::Arena A(s);
         hp::Level L;
         hp::make_level(num_nodes, num_hedges, offsets, pins, src_counts, size, L, A);
-        P.wsum = (int64_t)num_hedges * 65536;
+        hp::weight_bounds(weights, num_hedges, P, A);
         uint32_t *err = A.get<uint32_t>(1);
         long long *bg = A.get<long long>(1);
         HPC(cudaMemsetAsync(err, 0, sizeof(uint32_t), s));

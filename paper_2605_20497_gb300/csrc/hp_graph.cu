@@ -48,6 +48,25 @@ __global__ void k_edges_level0(const int32_t *off, int32_t e, const int32_t *src
     if ((threadIdx.x & 31) == 0 && mx > 0) atomicMax(wmax, mx);
 }
 
+// sum and largest of a step call's weights
+__global__ void k_weight_bounds(const int32_t *w, int32_t e, unsigned long long *sum, int32_t *mx) {
+    HP_KERNEL_ENTER();
+    unsigned long long s = 0;
+    int32_t m = 0;
+    GRID_STRIDE(i, (int64_t)e) {
+        s += (unsigned long long)max(w[i], 0);
+        m = max(m, w[i]);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_down_sync(0xffffffffu, s, o);
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    }
+    if ((threadIdx.x & 31) == 0 && m > 0) {
+        atomicAdd(sum, s);
+        atomicMax(mx, m);
+    }
+}
+
 // pedge[j] = hyperedge of pin position j (one warp per hyperedge)
 __global__ void k_pin_edges(const int32_t *off, int32_t e, int32_t *pedge) {
     HP_KERNEL_ENTER();
@@ -147,6 +166,25 @@ void build_incidence(Level &L, Arena &A) {
     }
     A.release(keys);
     A.release(cnt);
+}
+
+// The step calls do not limit the weights, while the kernels' counters are as
+// wide as P says: bounds of at least what hp_partition admits, and of the weights given.
+void weight_bounds(const int32_t *w, int32_t e, Params &P, Arena &A) {
+    P.wsum = (int64_t)e * 65536;
+    if (e == 0) return;
+    cudaStream_t s = A.stream();
+    struct Box {
+        unsigned long long sum;
+        int32_t mx, pad;
+    } hb, *box = A.get<Box>(1);
+    HPC(cudaMemsetAsync(box, 0, sizeof(Box), s));
+    launch_k(k_weight_bounds, grid_of(e, 256), 256, 0, s, w, e, &box->sum, &box->mx);
+    HP_LAUNCH_CHECK();
+    fetch_bytes(&hb, box, sizeof(Box), s);
+    A.release(box);
+    P.wsum = std::max(P.wsum, (int64_t)hb.sum);
+    P.wmax = std::max(P.wmax, hb.mx);
 }
 
 uint32_t validate_and_build_level0(const int32_t *pins, const int32_t *offsets, int32_t e, int32_t n,

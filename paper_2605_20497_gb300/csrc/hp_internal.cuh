@@ -403,6 +403,7 @@ struct Params {
 };
 
 // graph construction (hp_graph.cu)
+void weight_bounds(const int32_t *w, int32_t e, Params &P, Arena &A);
 uint32_t validate_and_build_level0(const int32_t *pins, const int32_t *offsets, int32_t e, int32_t n,
                                    const int32_t *src_counts, const int32_t *weights, Params &P, Level &L,
                                    int32_t *w_out, Arena &A);
