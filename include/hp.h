@@ -419,7 +419,7 @@ HP_API hp_status hp_merge_quantize(const float *params, const uint8_t *calib, in
 /*
  * Step-level entry points (test hooks) on one level graph given in device
  * memory: num_nodes, num_hedges, offsets, pins, src_counts (required, one
- * count per hyperedge), weights (required) and node sizes.  They run one step
+ * count per hyperedge), weights (required, positive, below 2^26) and node sizes.  They run one step
  * of the method exactly as hp_partition runs it inside its level loop.
  *
  * hp_debug_coarsen_level -- one coarsening level (Sec. V-C, V-D): the top-pi

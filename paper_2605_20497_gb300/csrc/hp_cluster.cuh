@@ -93,7 +93,7 @@ __device__ __forceinline__ int dev_bits(unsigned long long x) { return x ? 64 - 
 // ---------------------------------------------------------------- cluster-wide
 // A cluster of SQ_CS CTAs of SQ_T threads; each CTA holds up to sq_chunk<K>()
 // sort items in shared memory, so one cluster sorts up to sq_max<K>() items
-// (45,056 with 64-bit keys, 65,536 with 32-bit keys).
+// (46,592 with 64-bit keys, 65,536 with 32-bit keys).
 constexpr int SQ_CS = 8;                        // CTAs per cluster (portable size)
 constexpr int SQ_T = 1024;                      // threads per CTA
 // dynamic shared memory of a cluster-sort CTA: two key and two value buffers

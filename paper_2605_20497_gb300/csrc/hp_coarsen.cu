@@ -6,7 +6,7 @@
 // The proposal fuses neighbour deduplication with the eta/inter histogram:
 // one CTA per node walks I(n) and the pins of every incident hyperedge and
 // accumulates into a shared-memory table (direct-indexed on levels of at most
-// 4,096 nodes, and for large neighbourhoods up to 16,384; open-addressing
+// 4,096 nodes, and for large neighbourhoods up to 26,624; open-addressing
 // otherwise; nodes whose neighbourhood outgrows the table are redone with a
 // larger table and finally with a table in global memory).  Sums and counts
 // are integers, so the result does not depend on the order of the atomic
@@ -954,6 +954,13 @@ __global__ void __launch_bounds__(PT) k_propose_global(PropCtx C, const int32_t 
 // levels of at most DENSE_ALL nodes there are too few nodes to fill the GPU a
 // warp each: only walks of up to WARP_VISITS_FEW pins stay with a warp, and
 // every other node takes a dense table, which costs it no probes.
+// Where the lines lie (whole calls): DENSE_ALL at 1,024 nodes the 16,384-node
+// random net takes 117.7 ms instead of 113.6, at 16,384 nodes a 16,384-node
+// Gaussian net 42.2 instead of 41.8; WARP_VISITS_FEW at 2,048 the 1,021-node
+// irregular net 4.46 instead of 4.30 and the 4,096-node random net 11.4 instead
+// of 11.1, at 128 the first 4.20 and the second 11.2; HUB_VISITS_FEW at 4,096
+// the 20k irregular net 62.8 instead of 60.8, at 65,536 the 4,096-node random
+// net 11.7 instead of 11.1 (but the 16,384-node one 107.1 instead of 113.6).
 constexpr long long WARP_VISITS = 4096, WARP_VISITS_FEW = 512, HUB_VISITS = 262144, HUB_VISITS_FEW = 16384;
 constexpr int32_t HUB_INCIDENCE = 4096;   // incidence entries: chunks of a walk
 constexpr int32_t DENSE_ALL = 4096;
@@ -1054,7 +1061,9 @@ static void run_proposal(const PropCtx &C, Level &L, const Params &P, CoarsenWs 
     const uint32_t limB = dbg > 0 ? capB * 3 / 4 : capB * 5 / 8;
     if (C.exact_bound && dbg == 0) R.large_bound = (int32_t)(2 * limB);
     // (a dense table is also scanned: above DENSE_N nodes it is for
-    // neighbourhoods of a fifth of the level)
+    // neighbourhoods of a fifth of the level.  From a tenth on: 20k irregular
+    // net 61.9 ms instead of 60.8; from a third on: 60k power-law net 112.2
+    // instead of 98.9)
     if (C.n <= DENSE_NARROW_N && dbg == 0)
         R.dense_bound = R.dense_wide ? (int32_t)(capB / 2) : std::max((int32_t)(capB / 2), C.n / 5);
     if (C.n <= DENSE_ALL && dbg == 0) {
@@ -1710,7 +1719,9 @@ static void propose_lists(Level &L, int32_t level, const int32_t *w, const Param
         // contraction) are walked once per warp group.  After a level whose
         // lists were nearly all distinct the grouping is not tried again
         // before a quarter of its pins has gone: it costs a hash, a sort and
-        // a comparison of every list (0.2 ms on the 16,384-node random net).
+        // a comparison of every list (tried on every level: 16,384-node random net
+        // 116.7 -> 119.5 ms, 4,096-node one 11.1 -> 11.7; waiting for half of the
+        // pins to go is no faster than for a quarter).
         dst_groups(L, W.canon, W.canon + std::max(W.ce, 1), box, A);
         C.canon = W.canon;
     }

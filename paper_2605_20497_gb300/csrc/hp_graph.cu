@@ -324,7 +324,9 @@ __device__ __forceinline__ int32_t pin_keep(const int32_t *pin, const int32_t *p
 // Levels of up to CONTRACT_CLUSTER_NP pins run the steps in one launch on one
 // thread-block cluster; larger ones as a few grid-wide kernels.
 constexpr int64_t CONTRACT_CLUSTER_NP = int64_t(1) << 15;
-constexpr int64_t SLAB_NP = int64_t(1) << 22;   // at most 100 MB a level
+// pins of a fine level up to which the coarse one lies in one block (12 B a pin
+// and a node and 8 B a hyperedge of the fine level)
+constexpr int64_t SLAB_NP = int64_t(1) << 22;
 
 struct ContractArgs {
     Level L;                 // the fine level

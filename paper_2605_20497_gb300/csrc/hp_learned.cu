@@ -319,9 +319,9 @@ __global__ void __launch_bounds__(MLP_WARPS * 32) k_merge_mlp(const uint8_t *fea
 // layer is a third matrix product with one column.  A warp takes 32 rows a
 // step, so that a weight fragment serves two products, and a lane reads its
 // four features of a row as one word (the k order of both operands is
-// permuted alike).  Bound by the mma.sync rate: 8,388,608 rows in 310 us,
-// 540 us in the general form above, which spent 67 % of its time on integer
-// instructions.
+// permuted alike).  Bound by the mma.sync rate and latency: 8,388,608 rows in
+// 272 us, 476 us in the general form above (both under ncu), which spent 67 % of
+// its time on integer instructions.
 __device__ __forceinline__ void mma_16816_f16(float (&d)[4], const uint32_t (&a)[4], uint2 b) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "

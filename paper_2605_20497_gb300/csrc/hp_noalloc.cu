@@ -2,10 +2,10 @@
 // cut-net count for a given part vector, computed without allocating any
 // device memory.
 //
-// Why it exists: hp_connectivity builds the full level-0 incidence and the
-// sorted pins(p, e) lists of the refinement, which takes workspace from the
-// library's memory pool (or from the allocator installed by
-// hp_set_allocator).  Some callers cannot allow that at the moment they need
+// Why it exists: hp_connectivity takes workspace from the library's memory pool
+// (or from the allocator installed by hp_set_allocator): a few words for its one
+// pass over the pins, and the full level-0 incidence where destinations do not
+// ascend or there are more than 32,768 parts.  Some callers cannot allow that at the moment they need
 // the number: a caller whose allocator hook refuses requests while its own
 // step is in flight, a process that has handed all free device memory to
 // another pool, or a monitoring thread that must not take an allocator lock
