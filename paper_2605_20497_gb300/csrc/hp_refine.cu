@@ -425,6 +425,8 @@ constexpr int PS_T = 256;
 constexpr int32_t PS_PARTS = 32768;   // bit rows of up to 4 KB a warp
 constexpr uint32_t PS_UNSORTED = 1u << 31, PS_HAS_BIG = 1u << 30;
 constexpr int PSB_T = 1024;
+// (from 2,048 pins on, 20,000 hyperedges of 3,000 pins take 0.28 ms instead of
+// 0.18; from 32,768 on, one of 20,000 takes 0.24 instead of 0.07)
 constexpr int32_t PS_BIG = 8192;
 inline size_t part_scan_smem(int32_t nparts, bool d) {
     const size_t words = (size_t)cdiv(std::max(nparts, 1), 1024) * 32;
